@@ -269,14 +269,16 @@ int lbm_time_kernels(lbm_handle h, int64_t n, double *ms);
 
 /* Planes per CTA along the march axis (z; the 2D y axis for D2Q9) of the
  * fused FP32 step, >= 1 (default 16 for D3Q27, 64 for D2Q9). A tuning knob:
- * results do not depend on it. */
+ * results do not depend on it; D2Q9 steps, which march along nothing, take
+ * it and run the same. */
 int lbm_set_chunk(lbm_handle h, int chunk);
 
 /* Pick the chunk of the fused FP32 step by timing candidates (4 to 128
  * planes and, on a longer march axis, 10/16 to 16/16 of it) on the
  * handle's own state (saved to a temporary device buffer and restored
  * afterwards, so the state is unchanged). Sets and returns it in
- * *chunk_out (0 for FP64 storage, which has no tile parameter). With
+ * *chunk_out (0 for FP64 storage, which has no tile parameter; D2Q9, whose
+ * step has one form, returns the chunk it has and times nothing). With
  * LBM_F32 storage it also picks the form of the step
  * (lbm_set_fused_variant), and for D3Q27 the tile height, 8 or 7
  * rows of 32 nodes (7 rows fill every SM with two CTAs in one wave where 8
@@ -288,7 +290,8 @@ int lbm_set_chunk(lbm_handle h, int chunk);
 int lbm_autotune(lbm_handle h, int *chunk_out);
 
 /* The tile of the fused step in use, in nodes: *tile_x = 32, *tile_y = 8 or
- * 7 (D3Q27; 7 only after lbm_autotune chose it), or 128 x 1 for D2Q9 rows;
+ * 7 (D3Q27; 7 only after lbm_autotune chose it); for D2Q9 nominally 128 x 1
+ * (a row of the march axis's frame; its blocks take 32 x 8 nodes);
  * 0 x 0 for LBM_F64 storage, which runs one thread per node. Either pointer
  * may be NULL. */
 int lbm_get_tile(lbm_handle h, int *tile_x, int *tile_y);
@@ -315,8 +318,11 @@ int lbm_set_tile(lbm_handle h, int tile_y);
  *     call return LBM_ETIMEOUT.
  *   LBM_FUSED_TMEM: the plain form, with each node's populations kept in the
  *     SM's Tensor Memory from the plane's entry to its collision instead of
- *     being read twice; each block holds 256 columns (D3Q27; 64 for D2Q9) of
- *     Tensor Memory while it runs. */
+ *     being read twice; each block holds 256 columns of Tensor Memory while
+ *     it runs.
+ * D2Q9 takes LBM_FUSED_PLAIN, LBM_FUSED_WARP_SPECIALISED (FP32) and
+ * LBM_FUSED_TMEM and runs its one kernel for each: a node's populations stay
+ * in registers there. */
 enum {
     LBM_FUSED_PLAIN = 0,
     LBM_FUSED_WARP_SPECIALISED = 1,
@@ -363,8 +369,8 @@ int lbm_get_fused_variant(lbm_handle h, int *variant);
  * storage (LBM_F32, LBM_F16S or LBM_BF16S, not LBM_F64) and the same lattice
  * type, of any sizes and parameters; otherwise LBM_EINVAL. Each
  * lbm_batch_step launch gives every member one time step (the fused step of
- * that storage over all members' tiles, spread over a persistent grid of two
- * CTAs per SM); steps after the first replay a CUDA graph of two launches. Each
+ * that storage over all members' tiles: D3Q27 spread over a persistent grid
+ * of two CTAs per SM, D2Q9 one CTA per tile); steps after the first replay a CUDA graph of two launches. Each
  * member's result is bitwise the same as stepping it alone. While the batch
  * exists the members' work is ordered on the batch's stream (members must
  * not be stepped, initialised or written individually); lbm_batch_destroy

@@ -17,6 +17,7 @@
 #include "lbm_fused_f32.cuh"
 #include "lbm_fused_f32_r7.cuh"
 #include "lbm_kernels.cuh"
+#include "lbm_step2d.cuh"
 #include "lbm_step_tma.h"
 
 using lbmk::Geo;
@@ -421,6 +422,30 @@ void launch_fused_e64(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
+// The D2Q9 step of a reduced storage from population buffer k: one kernel,
+// whatever form, chunk or tile the handle names (lbm_step2d.cuh).
+template <typename ST, bool MASK, bool E64>
+void launch_2d_m(lbm_ctx *h, cudaStream_t s, int k)
+{
+    const GeoF &g = h->geof;
+    const dim3 grid((g.nx + lbmf2::TX - 1) / lbmf2::TX, (g.nz + lbmf2::TY - 1) / lbmf2::TY);
+    lbmf2::k_step2d<MASK, ST, E64><<<grid, lbmf2::NT, 0, s>>>(
+        g, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]), h->rs[k],
+        h->rs[k ^ 1], h->status);
+}
+
+template <typename ST>
+void launch_2d(lbm_ctx *h, cudaStream_t s, int k)
+{
+    if (has_solid(h)) {
+        if (h->e64) launch_2d_m<ST, true, true>(h, s, k);
+        else        launch_2d_m<ST, true, false>(h, s, k);
+    } else {
+        if (h->e64) launch_2d_m<ST, false, true>(h, s, k);
+        else        launch_2d_m<ST, false, false>(h, s, k);
+    }
+}
+
 template <int LAT>
 void launch_fused(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
@@ -467,6 +492,13 @@ void launch_fused(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
         lbmf::k_step_f32<LAT, false><<<gr, L::TX * L::TY, bytes, s>>>(h->geof, h->physf, h->mask, src,
                                                                      dst, h->status);
     }
+}
+
+// One step of FP32 storage from population buffer k.
+void launch_f32(lbm_ctx *h, cudaStream_t s, int k)
+{
+    if (h->lattice == LBM_D2Q9) launch_2d<float>(h, s, k);
+    else                        launch_fused<1>(h, s, f32(h, k), f32(h, k ^ 1));
 }
 
 template <int LAT, typename ST, bool E64, bool MASK>
@@ -532,11 +564,17 @@ void launch_shifted_t(lbm_ctx *h, cudaStream_t s, int k)
     else              launch_shifted_m<LAT, ST, false>(h, s, k);
 }
 
-template <int LAT>
+// One step of shifted storage from population buffer k.
 void launch_shifted(lbm_ctx *h, cudaStream_t s, int k)
 {
-    if (h->storage == LBM_F16S) launch_shifted_t<LAT, __half>(h, s, k);
-    else                        launch_shifted_t<LAT, __nv_bfloat16>(h, s, k);
+    const bool half = h->storage == LBM_F16S;
+    if (h->lattice == LBM_D2Q9) {
+        if (half) launch_2d<__half>(h, s, k);
+        else      launch_2d<__nv_bfloat16>(h, s, k);
+    } else {
+        if (half) launch_shifted_t<1, __half>(h, s, k);
+        else      launch_shifted_t<1, __nv_bfloat16>(h, s, k);
+    }
 }
 
 // One time step; returns the number of kernels launched (0 on error).
@@ -544,10 +582,10 @@ template <int LAT>
 int launch_step(lbm_ctx *h, cudaStream_t s, int *nk)
 {
     if (shifted(h->storage)) {
-        launch_shifted<LAT>(h, s, h->cur);
+        launch_shifted(h, s, h->cur);
         *nk = 1;
     } else if (h->storage == LBM_F32) {
-        launch_fused<LAT>(h, s, f32(h, h->cur), f32(h, h->cur ^ 1));
+        launch_f32(h, s, h->cur);
         *nk = 1;
     } else {
         const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
@@ -1389,35 +1427,41 @@ struct lbm_batch_ctx {
 
 namespace {
 
-template <int LAT, typename ST>
+template <typename ST>
 void launch_batch_shifted(lbm_batch_ctx *b, int parity, cudaStream_t s)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    const int bytes = (int)sizeof(lbmf::SharedS<LAT>);
-    smem_opt_in(lbmf::k_step_shifted_batch<LAT, ST>, bytes, done);
-    lbmf::k_step_shifted_batch<LAT, ST>
-        <<<b->grid, lbmf::LatF<LAT>::TX * lbmf::LatF<LAT>::TY, bytes, s>>>(
-            b->d_members[parity], b->d_items, b->n_items);
+    const int bytes = (int)sizeof(lbmf::SharedS<1>);
+    smem_opt_in(lbmf::k_step_shifted_batch<1, ST>, bytes, done);
+    lbmf::k_step_shifted_batch<1, ST><<<b->grid, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(
+        b->d_members[parity], b->d_items, b->n_items);
 }
 
-template <int LAT>
 void launch_batch(lbm_batch_ctx *b, int parity, cudaStream_t s)
 {
-    if (b->storage == LBM_F16S) launch_batch_shifted<LAT, __half>(b, parity, s);
-    else if (b->storage == LBM_BF16S) launch_batch_shifted<LAT, __nv_bfloat16>(b, parity, s);
+    if (b->storage == LBM_F16S) launch_batch_shifted<__half>(b, parity, s);
+    else if (b->storage == LBM_BF16S) launch_batch_shifted<__nv_bfloat16>(b, parity, s);
     else {
         static std::atomic<unsigned long long> done{0};   // devices already opted in
-        const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
-        smem_opt_in(lbmf::k_step_f32_batch<LAT>, bytes, done);
-        lbmf::k_step_f32_batch<LAT><<<b->grid, lbmf::LatF<LAT>::TX * lbmf::LatF<LAT>::TY, bytes, s>>>(
+        const int bytes = (int)sizeof(lbmf::SharedF<1>);
+        smem_opt_in(lbmf::k_step_f32_batch<1>, bytes, done);
+        lbmf::k_step_f32_batch<1><<<b->grid, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(
             b->d_members[parity], b->d_items, b->n_items);
     }
 }
 
+template <typename ST>
+void launch_batch_2d(lbm_batch_ctx *b, int parity, cudaStream_t s)
+{
+    lbmf2::k_step2d_batch<ST><<<b->n_items, lbmf2::NT, 0, s>>>(b->d_members[parity], b->d_items);
+}
+
 void batch_launch(lbm_batch_ctx *b, int parity, cudaStream_t s)
 {
-    if (b->lattice == LBM_D2Q9) launch_batch<0>(b, parity, s);
-    else launch_batch<1>(b, parity, s);
+    if (b->lattice != LBM_D2Q9) launch_batch(b, parity, s);
+    else if (b->storage == LBM_F32) launch_batch_2d<float>(b, parity, s);
+    else if (b->storage == LBM_F16S) launch_batch_2d<__half>(b, parity, s);
+    else launch_batch_2d<__nv_bfloat16>(b, parity, s);
 }
 
 void batch_free(lbm_batch_ctx *b)
@@ -1470,10 +1514,10 @@ int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
     std::vector<lbmf::WorkItem> items;
     for (int k = 0; k < count; ++k) {
         lbm_ctx *h = b->members[k];
-        const int TX = lattice == LBM_D2Q9 ? lbmf::LatF<0>::TX : lbmf::LatF<1>::TX;
-        const int TY = lattice == LBM_D2Q9 ? lbmf::LatF<0>::TY : lbmf::LatF<1>::TY;
-        const int tx = (h->geof.nx + TX - 1) / TX, ty = (h->geof.ny + TY - 1) / TY;
-        const int tz = (h->geof.nz + h->geof.chunk - 1) / h->geof.chunk;
+        // D3Q27: 32 x 8 columns by z-chunks; D2Q9: 32 x 8 tiles of the (x, 2D y) plane
+        const int tx = (h->geof.nx + 31) / 32;
+        const int ty = ((lattice == LBM_D2Q9 ? h->geof.nz : h->geof.ny) + 7) / 8;
+        const int tz = lattice == LBM_D2Q9 ? 1 : (h->geof.nz + h->geof.chunk - 1) / h->geof.chunk;
         for (int par = 0; par < 2; ++par) {
             lbmf::MemberF m;
             m.g = h->geof;
@@ -1599,14 +1643,8 @@ int lbm_time_kernels(lbm_handle h, int64_t n, double *ms)
         CU(h, cudaEventRecord(ev[3 * k], h->stream));
         if (fused) {
             CU(h, cudaEventRecord(ev[3 * k + 1], h->stream));
-            if (shifted(h->storage)) {
-                if (h->lattice == LBM_D2Q9) launch_shifted<0>(h, h->stream, h->cur);
-                else launch_shifted<1>(h, h->stream, h->cur);
-            } else if (h->lattice == LBM_D2Q9) {
-                launch_fused<0>(h, h->stream, f32(h, h->cur), f32(h, h->cur ^ 1));
-            } else {
-                launch_fused<1>(h, h->stream, f32(h, h->cur), f32(h, h->cur ^ 1));
-            }
+            if (shifted(h->storage)) launch_shifted(h, h->stream, h->cur);
+            else                     launch_f32(h, h->stream, h->cur);
             h->launches += 1;
         } else {
             const double *src = f64(h, h->cur);
@@ -1652,6 +1690,10 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
     if (h->storage == LBM_F64) {
         if (chunk_out) *chunk_out = 0;
         return LBM_OK;   // the FP64 step has no tile parameters
+    }
+    if (h->lattice == LBM_D2Q9) {   // nor has the D2Q9 step: its chunk changes nothing
+        if (chunk_out) *chunk_out = h->geof.chunk;
+        return LBM_OK;
     }
     if (h->bad) return fail(h, LBM_ESTATE, "state holds a non-finite density; re-initialise");
     const size_t bytes = pop_bytes(h->storage) * (size_t)h->Q * h->geo.N;
