@@ -38,6 +38,8 @@ struct lbm_ctx {
     double t_over_tc, tau;
     std::vector<uint8_t> mask_host, zsolid_host;
     bool any_solid = false;
+    int sms = 148;         // SMs of the device
+    int sweep_chunk = 16;  // planes per block of the D3Q27 force sweep (FP64 kernels)
     int device;
     cudaStream_t own_stream = nullptr, stream = nullptr, cap_stream = nullptr;
     // device memory
@@ -327,6 +329,43 @@ void make_tensor_maps(lbm_ctx *h)
     h->tmap_ready = true;
 }
 
+// The force sweep over the lattice (lbm_kernels.cuh) with the given body.
+template <int LAT, typename Body>
+void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
+{
+    const Geo &g = h->geo;
+    const int tx = (g.nx + lbmk::SWX - 1) / lbmk::SWX;
+    if constexpr (LAT == 1) {
+        const int chunk = h->sweep_chunk;
+        const dim3 grid(tx, (g.ny + lbmk::SWY - 1) / lbmk::SWY, (g.nz + chunk - 1) / chunk);
+        lbmk::k_force_sweep3<<<grid, lbmk::SWX * lbmk::SWY, 0, s>>>(g, h->phys, h->rp, chunk, body);
+    } else if (tx * ((g.ny + 7) / 8) < h->sms) {
+        lbmk::k_force_sweep2<2, 4><<<dim3(tx, (g.ny + 1) / 2), 128, 0, s>>>(g, h->phys, h->rp, body);
+    } else {
+        lbmk::k_force_sweep2<8, 8><<<dim3(tx, (g.ny + 7) / 8), 256, 0, s>>>(g, h->phys, h->rp, body);
+    }
+}
+
+// Planes per block of the D3Q27 force sweep: its blocks share each SM's FP64
+// pipe, so the SM with the most blocks sets the time; a block of c planes
+// also sums 4 more (64 of about 200 operations per node).
+int sweep_chunk(const Geo &g, int sms)
+{
+    const long long tiles = (long long)((g.nx + lbmk::SWX - 1) / lbmk::SWX) *
+                            ((g.ny + lbmk::SWY - 1) / lbmk::SWY);
+    int best = 1;
+    double cost = 1e300;
+    for (int c = 1; c <= g.nz; ++c) {
+        const long long blocks = tiles * ((g.nz + c - 1) / c);
+        const double t = (double)((blocks + sms - 1) / sms) * (c * 200.0 + 4 * 64.0);
+        if (t < cost) {
+            cost = t;
+            best = c;
+        }
+    }
+    return best;
+}
+
 double *f64(lbm_ctx *h, int k) { return static_cast<double *>(h->fv[k]); }
 float *f32(lbm_ctx *h, int k) { return static_cast<float *>(h->fv[k]); }
 
@@ -577,6 +616,17 @@ void launch_shifted(lbm_ctx *h, cudaStream_t s, int k)
     }
 }
 
+// The collision of the FP64 step: the force sweep with its body, without the
+// terms in 1 - omega where the relaxation time is 1 everywhere.
+template <int LAT>
+void launch_collide64(lbm_ctx *h, cudaStream_t s, const double *src, double *dst)
+{
+    if (h->phys.omega == 1.0 && !h->phys.var_visc)
+        launch_sweep<LAT>(h, s, lbmk::CollideBody<LAT, true>{h->mask, src, dst, h->rp, h->u, h->gflux});
+    else
+        launch_sweep<LAT>(h, s, lbmk::CollideBody<LAT, false>{h->mask, src, dst, h->rp, h->u, h->gflux});
+}
+
 // One time step; returns the number of kernels launched (0 on error).
 template <int LAT>
 int launch_step(lbm_ctx *h, cudaStream_t s, int *nk)
@@ -593,8 +643,7 @@ int launch_step(lbm_ctx *h, cudaStream_t s, int *nk)
         double *dst = f64(h, h->cur ^ 1);
         lbmk::k_macro<LAT><<<gr, bl, 0, s>>>(h->geo, h->phys, h->mask, src, h->rp, h->u,
                                              h->gflux, h->status);
-        lbmk::k_collide<LAT><<<gr, bl, 0, s>>>(h->geo, h->phys, h->mask, src, dst, h->rp, h->u,
-                                               h->gflux);
+        launch_collide64<LAT>(h, s, src, dst);
         *nk = 2;
     }
     if (h->nb > 0) {   // interpolated bounce-back on the new state
@@ -744,8 +793,10 @@ int launch_macro_and_out(lbm_ctx *h, double *rho, double *u, double *U)
     else
         lbmk::k_macro<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, f64(h, h->cur),
                                                      h->rp, h->u, h->gflux, h->status);
-    lbmk::k_moments_out<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, h->u,
-                                                       rho, u, U);
+    if (U)
+        launch_sweep<LAT>(h, h->stream, lbmk::MomentsBody<LAT>{h->mask, h->rp, h->u, rho, u, U});
+    else
+        lbmk::k_moments_out<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, h->u, rho, u);
     CU(h, cudaGetLastError());
     h->launches += 2;
     return LBM_OK;
@@ -794,7 +845,7 @@ int launch_init(lbm_ctx *h, const double *rho0, const double *u0)
         TempF64 t;
         int rc = temp_alloc(h, t);
         if (rc) return rc;
-        lbmk::k_init<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0, t.p);
+        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT>{h->mask, h->rp, u0, t.p});
         rc = encode_from<LAT>(h, t.p);
         if (rc) return rc;
         CU(h, cudaGetLastError());
@@ -802,11 +853,9 @@ int launch_init(lbm_ctx *h, const double *rho0, const double *u0)
         return LBM_OK;
     }
     if (h->storage == LBM_F32)
-        lbmk::k_init<LAT, float><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0,
-                                                           f32(h, h->cur));
+        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT, float>{h->mask, h->rp, u0, f32(h, h->cur)});
     else
-        lbmk::k_init<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0,
-                                                    f64(h, h->cur));
+        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT>{h->mask, h->rp, u0, f64(h, h->cur)});
     CU(h, cudaGetLastError());
     return LBM_OK;
 }
@@ -952,11 +1001,14 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
     ph.b = prm.b;
     ph.RT = eos_temperature(eos, prm.a, prm.b, t_over_tc);
     ph.alpha = eos_alpha(eos, prm.acentric, t_over_tc);
+    ph.aalpha = ph.a * ph.alpha;
     ph.kappa = kappa;
+    ph.kr = kappa * (lattice == LBM_D2Q9 ? -1.0 / 6.0 : -1.0 / 36.0);
     ph.omega = 1.0 / tau;
     ph.phi_pref = (prm.flags & LBM_FLAG_PHI_OFF) ? 0.0 : -(1.0 - 0.5 * ph.omega);
     ph.rho_w = prm.rho_w;
     for (int a = 0; a < 3; ++a) ph.g[a] = (a < (lattice == LBM_D2Q9 ? 2 : 3)) ? prm.g[a] : 0.0;
+    ph.body = ph.g[0] != 0.0 || ph.g[1] != 0.0 || ph.g[2] != 0.0;
     ph.var_visc = prm.tau_v > 0.0 ? 1 : 0;
     ph.nu_l = (tau - 0.5) / 3.0;
     ph.nu_v = ph.var_visc ? (prm.tau_v - 0.5) / 3.0 : ph.nu_l;
@@ -1036,6 +1088,9 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
         return LBM_ECUDA;
     }
     h->stream = h->own_stream;
+    if (cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+        cudaGetLastError();   // the default stands
+    h->sweep_chunk = sweep_chunk(h->geo, h->sms);
     *out = h;
     return LBM_OK;
 }
@@ -1656,12 +1711,8 @@ int lbm_time_kernels(lbm_handle h, int64_t n, double *ms)
                 lbmk::k_macro<1><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, h->rp,
                                                            h->u, h->gflux, h->status);
             CU(h, cudaEventRecord(ev[3 * k + 1], h->stream));
-            if (h->lattice == LBM_D2Q9)
-                lbmk::k_collide<0><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, dst,
-                                                             h->rp, h->u, h->gflux);
-            else
-                lbmk::k_collide<1><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, dst,
-                                                             h->rp, h->u, h->gflux);
+            if (h->lattice == LBM_D2Q9) launch_collide64<0>(h, h->stream, src, dst);
+            else                        launch_collide64<1>(h, h->stream, src, dst);
             h->launches += 2;
         }
         CU(h, cudaEventRecord(ev[3 * k + 2], h->stream));

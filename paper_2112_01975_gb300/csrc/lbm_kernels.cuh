@@ -1,7 +1,7 @@
 // Device code of the two-phase lattice Boltzmann step (arXiv 2112.01975).
 //
 // Storage: populations SoA f[i * N + n] (FP64), node n = x + nx (y + ny z);
-// side fields written once per step by k_macro and read by k_collide:
+// side fields written once per step by k_macro and read by the collision:
 //   rp[n] = (rho, s psi)   double2; s = +1 where P > P0, else -1 (Sec. 2.3.4)
 //   u[a * N + n]           bare velocity sum c f / rho (Sec. 2.3.3)
 //   g[a * N + n]           rho u_a^3, the flux differenced by Phi (Eq. correction)
@@ -21,11 +21,14 @@ struct Geo {
 struct Phys {
     int eos;
     double a, b, RT, alpha;   // EOS constants at the run's temperature (R = 1)
+    double aalpha;            // a alpha
     double kappa;             // capillary coefficient kappa~
     double omega;             // 1 / tau
     double phi_pref;          // -(1 - omega/2), or 0 with the correction off
     double rho_w;             // virtual solid density
     double g[3];              // body acceleration; rho g joins the force (Sec. 4.1)
+    int body;                 // g is not zero
+    double kr;                // -kappa / 36 (D3Q27) or -kappa / 6 (D2Q9), see force_of_sums
     // density-dependent relaxation (var_visc): nu linear in rho from nu_l at
     // visc_rl to nu_v at visc_rv, constant beyond; phi_sign = -1, or 0 with
     // the correction off
@@ -49,108 +52,276 @@ __host__ __device__ constexpr int cxi(int i) { return i % 3 - 1; }
 __host__ __device__ constexpr int cyi(int i) { return (i / 3) % 3 - 1; }
 __host__ __device__ constexpr int czi(int i) { return i / 9 - 1; }
 
-// Pressure of the equations of state of Sec. 3.1 and Appendix G (gas constant 1).
-__device__ __forceinline__ double eos_pressure(const Phys &p, double rho)
+// An FP64 instruction (a comparison or a conversion too) takes 64 cycles of
+// one SM sub-partition and 19 of the SM's shared pipe, whatever the number of
+// active lanes (measured): as long as 76 issue slots. The FP64 kernels are
+// bound by how many they execute per node, so what can be shared between
+// neighbours is, signs and finiteness are tested on the bit patterns, and
+// one reciprocal serves the equation of state and 1/rho.
+
+// P - rho/3 of the equations of state of Sec. 3.1 and Appendix G (gas
+// constant 1) and 1/rho, from one reciprocal where the EOS has a denominator:
+// P = rho n / D, 1/(rho D) gives both.
+__device__ __forceinline__ double excess_pressure(const Phys &p, double rho, double &inv)
 {
+    double n, D;   // P / rho + m = n / D
+    double m = 0.0;
     switch (p.eos) {
     case 0:  // van der Waals
-        return rho * p.RT / (1.0 - p.b * rho) - p.a * rho * rho;
-    case 1: {  // Peng-Robinson, one division
-        const double d1 = 1.0 - p.b * rho, d2 = 1.0 + 2.0 * p.b * rho - p.b * p.b * rho * rho;
-        return (rho * p.RT * d2 - p.a * p.alpha * rho * rho * d1) / (d1 * d2);
+        n = p.RT;
+        D = fma(-p.b, rho, 1.0);
+        m = p.a * rho;
+        break;
+    case 1: {  // Peng-Robinson
+        const double br = p.b * rho, d1 = 1.0 - br, d2 = fma(br, 2.0 - br, 1.0);
+        n = fma(p.RT, d2, -(p.aalpha * rho) * d1);
+        D = d1 * d2;
+        break;
     }
-    case 2: {  // Redlich-Kwong-Soave, one division
-        const double d1 = 1.0 - p.b * rho, d2 = 1.0 + p.b * rho;
-        return (rho * p.RT * d2 - p.a * p.alpha * rho * rho * d1) / (d1 * d2);
+    case 2: {  // Redlich-Kwong-Soave
+        const double br = p.b * rho, d1 = 1.0 - br, d2 = 1.0 + br;
+        n = fma(p.RT, d2, -(p.aalpha * rho) * d1);
+        D = d1 * d2;
+        break;
     }
     case 3: {  // Carnahan-Starling
-        const double e = 0.25 * p.b * rho;
-        const double om = 1.0 - e;
-        return rho * p.RT * (1.0 + e + e * e - e * e * e) / (om * om * om) - p.a * rho * rho;
+        const double e = 0.25 * p.b * rho, om = 1.0 - e;
+        n = p.RT * fma(e * e, om, 1.0 + e);
+        D = om * om * om;
+        m = p.a * rho;
+        break;
     }
     case 4: {  // Shan-Chen, psi_SC = 1 - exp(-rho); RT holds the coupling G
         const double q = 1.0 - exp(-rho);
-        return rho * (1.0 / 3.0) + p.RT * (1.0 / 6.0) * q * q;
+        inv = 1.0 / rho;
+        return p.RT * (1.0 / 6.0) * q * q;
     }
     default: {  // Shan-Chen, psi_SC = exp(-1/rho)
-        const double q = exp(-1.0 / rho);
-        return rho * (1.0 / 3.0) + p.RT * (1.0 / 6.0) * q * q;
+        inv = 1.0 / rho;
+        const double q = exp(-inv);
+        return p.RT * (1.0 / 6.0) * q * q;
     }
     }
+    const double r = 1.0 / (rho * D);
+    inv = r * D;
+    return rho * (fma(n, r * rho, -m) - 1.0 / 3.0);
+}
+
+// d > 0 by its bits (false for NaN, as the comparison is).
+__device__ __forceinline__ bool positive(double d)
+{
+    const long long v = __double_as_longlong(d);
+    return v > 0 && v <= 0x7ff0000000000000ll;
+}
+
+__device__ __forceinline__ bool finite_bits(double d)
+{
+    return (__double2hiint(d) & 0x7ff00000) != 0x7ff00000;
 }
 
 // Signed pseudo-potential s psi with psi = sqrt|P - P0|, P0 = rho/3.
+__device__ __forceinline__ double signed_psi_of(double d)
+{
+    const double r = sqrt(fabs(d));
+    return positive(d) ? r : -r;
+}
+
 __device__ __forceinline__ double signed_psi(const Phys &p, double rho)
 {
-    const double d = eos_pressure(p, rho) - rho * (1.0 / 3.0);
-    return d > 0.0 ? sqrt(d) : -sqrt(-d);
+    double inv;
+    return signed_psi_of(excess_pressure(p, rho, inv));
 }
 
 __device__ __forceinline__ int wrapm(int v, int n) { return v < 0 ? v + n : v; }
 __device__ __forceinline__ int wrapp(int v, int n) { return v >= n ? v - n : v; }
 
-// Korteweg force acting on the fluid at one node, plus the body force rho g:
+// ---- the Korteweg force of every node ---------------------------------
 //   F = -2 (s psi)_c S_psi - kappa rho_c S_rho + rho_c g,
 //   S_psi = sum_i (w_i/cs2) c_i [4/3 psi(r+c_i) - 1/6 psi(r+2c_i)],
 //   S_rho = sum_i (w_i/cs2) c_i [2 rho(r+c_i) - rho(r+2c_i)]   (Eq. Kforce_final).
-// w_i/cs2 c_ia = 1/2 W(c_ib) W(c_ic) c_ia with the 1D weights W(0) = 2/3,
-// W(+-1) = 1/6 of Eq. wi, so each ring sums neighbours by their number of
-// nonzero transverse components (centre, edge, corner) before weighting.
+// With the 1D weights W(0) = 2/3, W(+-1) = 1/6 of Eq. wi, w_i/cs2 c_ia =
+// 1/2 c_ia W(c_ib) W(c_ic): a central difference along a times [1, 4, 1]/6
+// smoothings along the other axes. Summed node by node that is 208 FP64
+// operations (D3Q27; both fields, both rings), more than half of the step;
+// one axis at a time, with each axis's sums shared by the nodes of a tile
+// through shared memory, it is 64. sum_a below are the sums without their
+// common factor: ring 1 plus RING2 times ring 2,
+//   S_psi = sum_psi / 54 (D2Q9: / 9),  S_rho = sum_rho / 36 (D2Q9: / 6).
+constexpr double RING2_PSI = -1.0 / 8.0, RING2_RHO = -1.0 / 2.0;
+
 template <int LAT>
-__device__ __forceinline__ void korteweg_force(const Geo &g, const Phys &p,
-                                               const double2 *__restrict__ rp, int x, int y,
-                                               int z, double rho_c, double spsi_c, double *F)
+__device__ __forceinline__ void force_of_sums(const Phys &p, double rho, double spsi, const double *sp,
+                                              const double *sr, double *F)
 {
     constexpr int D = Lattice<LAT>::D;
-    double Spsi[3] = {0.0, 0.0, 0.0}, Srho[3] = {0.0, 0.0, 0.0};
+    const double cp = spsi * (D == 3 ? -1.0 / 27.0 : -2.0 / 9.0);
+    const double cr = rho * p.kr;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        F[a] = fma(cp, sp[a], cr * sr[a]);
+        if (p.body) F[a] = fma(rho, p.g[a], F[a]);
+    }
+}
+
+// Tiles of 32 x 8 nodes; D3Q27 marches along z through `chunk` planes.
+// Per plane of the 36 x 12 halo tile: |psi| and rho to shared memory, the
+// x-sums of its 12 rows (smoothed and differenced, rings 1 and 2), and each
+// node's y-sums from them; the z-sums build up in registers as the planes
+// pass. The two barriers per plane and the loads are hidden by the second
+// block of the SM: the FP64 pipe is what is busy.
+// Body: what is done with a node's sums: body(p, n, x, y, z, sp, sr).
+constexpr int SWX = 32, SWY = 8;
+
+struct SweepSmem {
+    double raw[2][SWY + 4][SWX + 4];       // |psi|, rho
+    double xs[2][4][SWY + 4][SWX];         // x-sums: smooth 1, difference 1, smooth 2, difference 2
+};
+
+__device__ __forceinline__ int wrap_any(int v, int n)
+{
+    v = v < 0 ? v + n : v;
+    if (v >= n) {
+        v -= n;
+        if (v >= n) v %= n;
+    }
+    return v;
+}
+
+// x-sums of row r (of the halo tile) of field q.
+__device__ __forceinline__ void x_sums(SweepSmem &sm, int q, int r, int tx)
+{
+    const double *a = &sm.raw[q][r][tx + 2];
 #pragma unroll
     for (int s = 1; s <= 2; ++s) {
-        const int xm = wrapm(x - s, g.nx), xp = wrapp(x + s, g.nx);
-        const int ym = wrapm(y - s, g.ny), yp = wrapp(y + s, g.ny);
-        int zm = 0, zp = 0;
-        if (D == 3) { zm = wrapm(z - s, g.nz); zp = wrapp(z + s, g.nz); }
-        const int X[3] = {xm, x, xp}, Y[3] = {ym, y, yp}, Z[3] = {zm, z, zp};
-        double ap[3][3], ar[3][3];  // [component][0 centre, 1 edge, 2 corner]
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) { ap[a][k] = 0.0; ar[a][k] = 0.0; }
-        // each pair (c_i, -c_i) once: differences of the two neighbours, added
-        // with the sign of c_ia to every component where c_ia != 0
-#pragma unroll
-        for (int i = Lattice<LAT>::Q / 2 + 1; i < Lattice<LAT>::Q; ++i) {
-            const int c[3] = {cxi(i), cyi(i), D == 3 ? czi(i) : 0};
-            const unsigned np_ = X[c[0] + 1] + g.nx * (Y[c[1] + 1] + g.ny * Z[c[2] + 1]);
-            const unsigned nm_ = X[1 - c[0]] + g.nx * (Y[1 - c[1]] + g.ny * Z[1 - c[2]]);
-            const double2 vp = rp[np_], vm = rp[nm_];
-            const double dps = fabs(vp.y) - fabs(vm.y);
-            const double drh = vp.x - vm.x;
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                if (c[a] == 0) continue;
-                const int k = (a != 0 && c[0] != 0) + (a != 1 && c[1] != 0) + (a != 2 && c[2] != 0);
-                if (c[a] > 0) { ap[a][k] += dps; ar[a][k] += drh; }
-                else          { ap[a][k] -= dps; ar[a][k] -= drh; }
-            }
-        }
-        const double gp = s == 1 ? 4.0 / 3.0 : -1.0 / 6.0;
-        const double gr = s == 1 ? 2.0 : -1.0;
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            double dp, dr;
-            if (D == 3) {
-                dp = (2.0 / 9.0) * ap[a][0] + (1.0 / 18.0) * ap[a][1] + (1.0 / 72.0) * ap[a][2];
-                dr = (2.0 / 9.0) * ar[a][0] + (1.0 / 18.0) * ar[a][1] + (1.0 / 72.0) * ar[a][2];
-            } else {
-                dp = (1.0 / 3.0) * ap[a][0] + (1.0 / 12.0) * ap[a][1];
-                dr = (1.0 / 3.0) * ar[a][0] + (1.0 / 12.0) * ar[a][1];
-            }
-            Spsi[a] += gp * dp;
-            Srho[a] += gr * dr;
-        }
+        const double lo = a[-s], hi = a[s];
+        sm.xs[q][2 * s - 2][r][tx] = fma(4.0, a[0], lo + hi);
+        sm.xs[q][2 * s - 1][r][tx] = hi - lo;
     }
+}
+
+template <typename Body>
+__global__ void __launch_bounds__(SWX *SWY, 2)
+k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body body)
+{
+    __shared__ SweepSmem sm;
+    constexpr int NT = SWX * SWY, HX = SWX + 4, NH = HX * (SWY + 4);
+    const int tid = threadIdx.x, tx = tid % SWX, ty = tid / SWX;
+    const int x = blockIdx.x * SWX + tx, y = blockIdx.y * SWY + ty;
+    const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, g.nz);
+    const bool inside = x < g.nx && y < g.ny;
+    const unsigned plane = (unsigned)g.nx * (unsigned)g.ny;
+    // this thread's one or two halo nodes
+    const bool two = tid + NT < NH;
+    int hr[2], hc[2];
+    unsigned off[2];
 #pragma unroll
-    for (int a = 0; a < D; ++a) F[a] = -2.0 * spsi_c * Spsi[a] - p.kappa * rho_c * Srho[a] + rho_c * p.g[a];
+    for (int k = 0; k < 2; ++k) {
+        const int h = k == 0 || two ? tid + k * NT : 0;
+        hr[k] = h / HX;
+        hc[k] = h - hr[k] * HX;
+        off[k] = (unsigned)wrap_any((int)blockIdx.x * SWX - 2 + hc[k], g.nx) +
+                 (unsigned)g.nx * (unsigned)wrap_any((int)blockIdx.y * SWY - 2 + hr[k], g.ny);
+    }
+    int zq = z0 - 2 < 0 ? z0 - 2 + g.nz : z0 - 2;
+    double2 v0 = rp[off[0] + plane * (unsigned)zq], v1 = two ? rp[off[1] + plane * (unsigned)zq] : v0;
+    // sums under way, per field (|psi|, rho) and component, after plane q:
+    // n2 (ring 2 part of plane q + 2, without its factor), a1 (q + 1), a0 (q), m1 (q - 1)
+    double n2[2][3] = {}, a1[2][3] = {}, a0[2][3] = {}, m1[2][3] = {};
+    for (int q = z0 - 2; q < z1 + 2; ++q) {
+        sm.raw[0][hr[0]][hc[0]] = fabs(v0.y);
+        sm.raw[1][hr[0]][hc[0]] = v0.x;
+        if (two) {
+            sm.raw[0][hr[1]][hc[1]] = fabs(v1.y);
+            sm.raw[1][hr[1]][hc[1]] = v1.x;
+        }
+        zq = zq + 1 == g.nz ? 0 : zq + 1;
+        if (q + 1 < z1 + 2) {   // the next plane, while this one is summed
+            v0 = rp[off[0] + plane * (unsigned)zq];
+            if (two) v1 = rp[off[1] + plane * (unsigned)zq];
+        }
+        __syncthreads();
+        x_sums(sm, 0, ty, tx);
+        x_sums(sm, 1, ty, tx);
+        if (ty < 4) {
+            x_sums(sm, 0, ty + SWY, tx);
+            x_sums(sm, 1, ty + SWY, tx);
+        }
+        __syncthreads();
+        double done[2][3];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const double r2 = k == 0 ? RING2_PSI : RING2_RHO;
+            double X1[3], X2[3];   // ring 1 and 2 sums of the plane: x, y differences, smoothed
+#pragma unroll
+            for (int s = 1; s <= 2; ++s) {
+                double *X = s == 1 ? X1 : X2;
+                const auto &S = sm.xs[k][2 * s - 2], &Dx = sm.xs[k][2 * s - 1];
+                const double lo = S[ty + 2 - s][tx], hi = S[ty + 2 + s][tx];
+                X[0] = fma(4.0, Dx[ty + 2][tx], Dx[ty + 2 - s][tx] + Dx[ty + 2 + s][tx]);
+                X[1] = hi - lo;
+                X[2] = fma(4.0, S[ty + 2][tx], lo + hi);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                done[k][a] = fma(r2, X2[a], m1[k][a]);
+                m1[k][a] = a0[k][a] + X1[a];
+                if (a < 2) {
+                    a0[k][a] = fma(4.0, fma(r2, X2[a], X1[a]), a1[k][a]);
+                    a1[k][a] = fma(r2, n2[k][a], X1[a]);
+                } else {
+                    a0[k][a] = a1[k][a];
+                    a1[k][a] = fma(-r2, n2[k][a], -X1[a]);
+                }
+                n2[k][a] = X2[a];
+            }
+        }
+        if (q - 2 >= z0 && inside)
+            body(g, p, (unsigned)x + (unsigned)g.nx * (unsigned)y + plane * (unsigned)(q - 2), x, y, q - 2,
+                 done[0], done[1]);
+    }
+}
+
+// D2Q9: one tile of 32 x ROWS nodes per block, one shot; NW warps share the
+// x-sums of the ROWS + 4 rows, ROWS of them go on to the nodes. A lattice
+// with too few tiles of 8 rows for the SMs takes tiles of 2 rows, 4 warps: a
+// warp alone on its sub-partition is bound by its own chain of FP64
+// instructions, so the tile with fewer of them per warp on more SMs wins.
+template <int ROWS, int NW, typename Body>
+__global__ void __launch_bounds__(32 * NW)
+k_force_sweep2(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
+{
+    __shared__ SweepSmem sm;
+    static_assert(ROWS <= SWY && ROWS <= NW, "a warp per row of the tile");
+    constexpr int NT = 32 * NW, HX = SWX + 4, NH = HX * (ROWS + 4);
+    const int tid = threadIdx.x, tx = tid % 32, w = tid / 32;
+    const int x0 = blockIdx.x * SWX, y0 = blockIdx.y * ROWS;
+    for (int h = tid; h < NH; h += NT) {
+        const int r = h / HX, c = h - r * HX;
+        const double2 v = rp[(unsigned)wrap_any(x0 - 2 + c, g.nx) +
+                             (unsigned)g.nx * (unsigned)wrap_any(y0 - 2 + r, g.ny)];
+        sm.raw[0][r][c] = fabs(v.y);
+        sm.raw[1][r][c] = v.x;
+    }
+    __syncthreads();
+    for (int t = w; t < 2 * (ROWS + 4); t += NW) x_sums(sm, t & 1, t >> 1, tx);
+    __syncthreads();
+    const int x = x0 + tx, y = y0 + w;
+    if (w >= ROWS || x >= g.nx || y >= g.ny) return;
+    double sum[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double r2 = k == 0 ? RING2_PSI : RING2_RHO;
+        double X[2][2];
+#pragma unroll
+        for (int s = 1; s <= 2; ++s) {
+            const auto &S = sm.xs[k][2 * s - 2], &Dx = sm.xs[k][2 * s - 1];
+            X[s - 1][0] = fma(4.0, Dx[w + 2][tx], Dx[w + 2 - s][tx] + Dx[w + 2 + s][tx]);
+            X[s - 1][1] = S[w + 2 + s][tx] - S[w + 2 - s][tx];
+        }
+        sum[k][0] = fma(r2, X[1][0], X[0][0]);
+        sum[k][1] = fma(r2, X[1][1], X[0][1]);
+    }
+    body(g, p, (unsigned)x + (unsigned)g.nx * (unsigned)y, x, y, 0, sum[0], sum[1]);
 }
 
 // Moments, EOS and pseudo-potential of every fluid node; flags bad densities.
@@ -187,128 +358,146 @@ __global__ void k_macro(Geo g, Phys p, const uint8_t *__restrict__ mask,
         if (cy > 0) jy += row[r]; else if (cy < 0) jy -= row[r];
         if (D == 3) { if (cz > 0) jz += row[r]; else if (cz < 0) jz -= row[r]; }
     }
-    const double inv = 1.0 / rho;
-    const double ux = jx * inv, uy = jy * inv, uz = jz * inv;
-    if (!(rho > 0.0) || !isfinite(rho) || !isfinite(ux) || !isfinite(uy) || !isfinite(uz))
-        atomicOr(status, 1);
-    rp[n] = make_double2(rho, signed_psi(p, rho));
-    u[n] = ux;
-    u[g.N + n] = uy;
-    gflux[n] = rho * ux * ux * ux;
-    gflux[g.N + n] = rho * uy * uy * uy;
-    if (D == 3) {
-        u[2 * g.N + n] = uz;
-        gflux[2 * g.N + n] = rho * uz * uz * uz;
+    double inv;
+    const double d = excess_pressure(p, rho, inv);
+    const double j[3] = {jx, jy, jz};
+    bool ok = positive(rho) && finite_bits(rho);
+    rp[n] = make_double2(rho, signed_psi_of(d));
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const double ua = j[a] * inv;
+        u[a * g.N + n] = ua;
+        gflux[a * g.N + n] = j[a] * ua * ua;   // rho u_a^3
+        ok = ok && finite_bits(ua);
     }
+    if (!ok) atomicOr(status, 1);
 }
 
 // Force, correction, product-form collision and push streaming with
-// halfway bounce-back, one fluid node per thread (Eqs. LBGK, LBMeq, LBMstar).
-template <int LAT>
-__global__ void k_collide(Geo g, Phys p, const uint8_t *__restrict__ mask,
-                          const double *__restrict__ f, double *__restrict__ fout,
-                          const double2 *__restrict__ rp, const double *__restrict__ u,
-                          const double *__restrict__ gflux)
-{
-    constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= g.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
-    if (mask[n]) return;
-    const double2 c = rp[n];
-    const double rho = c.x;
-    double F[3] = {0.0, 0.0, 0.0};
-    korteweg_force<LAT>(g, p, rp, x, y, z, rho, c.y, F);
-    // Phi_aa = -(1 - omega/2) (g_a(r + e_a) - g_a(r - e_a)) / 2, the node's omega
-    const double om = omega_at(p, rho);
-    const double pref = p.var_visc ? p.phi_sign * (1.0 - 0.5 * om) : p.phi_pref;
-    const int xm = wrapm(x - 1, g.nx), xp = wrapp(x + 1, g.nx);
-    const int ym = wrapm(y - 1, g.ny), yp = wrapp(y + 1, g.ny);
-    double Phi[3];
-    Phi[0] = pref * 0.5 * (gflux[xp + g.nx * (y + g.ny * z)] - gflux[xm + g.nx * (y + g.ny * z)]);
-    Phi[1] = pref * 0.5 * (gflux[g.N + x + g.nx * (yp + g.ny * z)] -
-                                 gflux[g.N + x + g.nx * (ym + g.ny * z)]);
-    int zm = 0, zp = 0;
-    if (D == 3) {
-        zm = wrapm(z - 1, g.nz);
-        zp = wrapp(z + 1, g.nz);
-        Phi[2] = pref * 0.5 * (gflux[2 * g.N + x + g.nx * (y + g.ny * zp)] -
-                                     gflux[2 * g.N + x + g.nx * (y + g.ny * zm)]);
-    }
-    // Product-form factors: equilibrium (xi = u, zeta = 1/3 + u^2) and
-    // extended (xi* = u + F/rho, zeta* = 1/3 + xi*^2 + Phi/rho).
-    const double inv_rho = 1.0 / rho;
-    double E[3][3], S[3][3];
+// halfway bounce-back (Eqs. LBGK, LBMeq, LBMstar): the body of the force
+// sweep for the FP64 step. REST: relaxation time 1, where post = f* and
+// neither f nor feq is needed.
+template <int LAT, bool REST>
+struct CollideBody {
+    const uint8_t *mask;
+    const double *f;
+    double *fout;
+    const double2 *rp;
+    const double *u, *gflux;
+
+    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int x, int y, int z,
+                                               const double *sp, const double *sr) const
+    {
+        constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
+        if (mask[n]) return;
+        const double2 c = rp[n];
+        const double rho = c.x;
+        double F[3];
+        force_of_sums<LAT>(p, rho, c.y, sp, sr, F);
+        // Phi_aa = -(1 - omega/2) (g_a(r + e_a) - g_a(r - e_a)) / 2, the node's omega
+        const double om = REST ? 1.0 : omega_at(p, rho);
+        const double pref = p.var_visc ? p.phi_sign * (1.0 - 0.5 * om) : p.phi_pref;
+        const int X[3] = {wrapm(x - 1, g.nx), x, wrapp(x + 1, g.nx)};
+        const int Y[3] = {wrapm(y - 1, g.ny), y, wrapp(y + 1, g.ny)};
+        const int Z[3] = {D == 3 ? wrapm(z - 1, g.nz) : 0, z, D == 3 ? wrapp(z + 1, g.nz) : 0};
+        const auto at = [&](int cx, int cy, int cz) {
+            return X[cx + 1] + g.nx * (Y[cy + 1] + g.ny * Z[cz + 1]);
+        };
+        // Product-form factors: equilibrium (xi = u, zeta = 1/3 + u^2) and
+        // extended (xi* = u + F/rho, zeta* = 1/3 + xi*^2 + Phi/rho), as
+        // (zeta -+ xi)/2 and 1 - zeta.
+        const double inv = 1.0 / rho, ph = 0.25 * pref * inv;
+        double E[3][3], S[3][3];
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const double ua = u[a * g.N + n];
-        const double ze = 1.0 / 3.0 + ua * ua;
-        E[a][0] = 0.5 * (ze - ua);
-        E[a][1] = 1.0 - ze;
-        E[a][2] = 0.5 * (ze + ua);
-        const double xs = ua + F[a] * inv_rho;
-        const double zs = 1.0 / 3.0 + xs * xs + Phi[a] * inv_rho;
-        S[a][0] = 0.5 * (zs - xs);
-        S[a][1] = 1.0 - zs;
-        S[a][2] = 0.5 * (zs + xs);
-    }
-    const int X[3] = {xm, x, xp}, Y[3] = {ym, y, yp}, Z[3] = {zm, z, zp};
-    // post = f* + (1 - omega)(f - feq); feq and f* by x-y partial products
-    const double omw = 1.0 - om;
-    double Ae[3][3], As[3][3];
+        for (int a = 0; a < D; ++a) {
+            const double ua = u[a * (size_t)g.N + n];
+            const double dg = gflux[a * (size_t)g.N + at(a == 0, a == 1, a == 2)] -
+                              gflux[a * (size_t)g.N + at(-(a == 0), -(a == 1), -(a == 2))];
+            if (!REST) {
+                const double t = 0.5 * ua, h = fma(t, ua, 1.0 / 6.0);
+                E[a][0] = h - t;
+                E[a][1] = fma(-2.0, h, 1.0);
+                E[a][2] = h + t;
+            }
+            const double xs = fma(F[a], inv, ua), t = 0.5 * xs;
+            const double h = fma(ph, dg, fma(t, xs, 1.0 / 6.0));
+            S[a][0] = h - t;
+            S[a][1] = fma(-2.0, h, 1.0);
+            S[a][2] = h + t;
+        }
+        // post = (1 - omega) f + (f* - (1 - omega) feq); feq and f* by x-y
+        // partial products, the factor 1 - omega taken into feq's
+        const double omw = 1.0 - om, ro = REST ? 0.0 : rho * omw;
+        double Ae[3][3], As[3][3];
 #pragma unroll
-    for (int cx = 0; cx < 3; ++cx) {
-        const double ex = rho * E[0][cx], sx = rho * S[0][cx];
+        for (int cx = 0; cx < 3; ++cx) {
+            const double sx = rho * S[0][cx], ex = REST ? 0.0 : ro * E[0][cx];
 #pragma unroll
-        for (int cy = 0; cy < 3; ++cy) { Ae[cx][cy] = ex * E[1][cy]; As[cx][cy] = sx * S[1][cy]; }
-    }
+            for (int cy = 0; cy < 3; ++cy) {
+                As[cx][cy] = sx * S[1][cy];
+                Ae[cx][cy] = REST ? 0.0 : ex * E[1][cy];
+            }
+        }
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = cxi(i), cy = cyi(i), cz = D == 3 ? czi(i) : 0;
-        double eq = Ae[cx + 1][cy + 1];
-        double st = As[cx + 1][cy + 1];
-        if (D == 3) { eq *= E[2][cz + 1]; st *= S[2][cz + 1]; }
-        const double fi = f[(size_t)i * g.N + n];
-        const double post = fma(omw, fi - eq, st);
-        const unsigned dst = X[cx + 1] + g.nx * (Y[cy + 1] + g.ny * Z[cz + 1]);
-        if (mask[dst]) fout[(size_t)(Q - 1 - i) * g.N + n] = post;
-        else           fout[(size_t)i * g.N + dst] = post;
+        for (int i = 0; i < Q; ++i) {
+            const int cx = cxi(i), cy = cyi(i), cz = D == 3 ? czi(i) : 0;
+            double post = D == 3 ? As[cx + 1][cy + 1] * S[2][cz + 1] : As[cx + 1][cy + 1];
+            if (!REST) {
+                post = D == 3 ? fma(-Ae[cx + 1][cy + 1], E[2][cz + 1], post) : post - Ae[cx + 1][cy + 1];
+                post = fma(omw, f[(size_t)i * g.N + n], post);
+            }
+            const unsigned dst = at(cx, cy, cz);
+            if (mask[dst]) fout[(size_t)(Q - 1 - i) * g.N + n] = post;
+            else           fout[(size_t)i * g.N + dst] = post;
+        }
     }
-}
+};
 
 // Output moments: rho, bare u and U = u + F/(2 rho) (Sec. 2.3.5).
+// Without U no force is needed.
 template <int LAT>
 __global__ void k_moments_out(Geo g, Phys p, const uint8_t *__restrict__ mask,
                               const double2 *__restrict__ rp, const double *__restrict__ u,
-                              double *__restrict__ rho_out, double *__restrict__ u_out,
-                              double *__restrict__ U_out)
+                              double *__restrict__ rho_out, double *__restrict__ u_out)
 {
     constexpr int D = Lattice<LAT>::D;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
     const unsigned n = x + g.nx * (y + g.ny * z);
-    if (mask[n]) {
-        if (rho_out) rho_out[n] = p.rho_w;
+    const bool solid = mask[n];
+    if (rho_out) rho_out[n] = solid ? p.rho_w : rp[n].x;
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+        if (u_out) u_out[a * (size_t)g.N + n] = solid ? 0.0 : u[a * (size_t)g.N + n];
+}
+
+// The same with U: the body of the force sweep.
+template <int LAT>
+struct MomentsBody {
+    const uint8_t *mask;
+    const double2 *rp;
+    const double *u;
+    double *rho_out, *u_out, *U_out;
+
+    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int, int, int,
+                                               const double *sp, const double *sr) const
+    {
+        constexpr int D = Lattice<LAT>::D;
+        const bool solid = mask[n];
+        const double2 c = solid ? make_double2(p.rho_w, 0.0) : rp[n];
+        double F[3];
+        force_of_sums<LAT>(p, c.x, c.y, sp, sr, F);
+        const double half = 0.5 / c.x;
+        if (rho_out) rho_out[n] = c.x;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            if (u_out) u_out[a * g.N + n] = 0.0;
-            if (U_out) U_out[a * g.N + n] = 0.0;
+            const double ua = solid ? 0.0 : u[a * (size_t)g.N + n];
+            if (u_out) u_out[a * (size_t)g.N + n] = ua;
+            U_out[a * (size_t)g.N + n] = solid ? 0.0 : fma(F[a], half, ua);
         }
-        return;
     }
-    const double2 c = rp[n];
-    double F[3] = {0.0, 0.0, 0.0};
-    if (U_out) korteweg_force<LAT>(g, p, rp, x, y, z, c.x, c.y, F);
-    if (rho_out) rho_out[n] = c.x;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const double ua = u[a * g.N + n];
-        if (u_out) u_out[a * g.N + n] = ua;
-        if (U_out) U_out[a * g.N + n] = ua + F[a] / (2.0 * c.x);
-    }
-}
+};
 
 // Interpolated (linear Bouzidi) bounce-back, after a push step with halfway
 // bounce-back, one boundary node per thread. For each active link of node n
@@ -434,41 +623,44 @@ __global__ void k_init_density(Geo g, Phys p, const uint8_t *__restrict__ mask,
 // the bare velocity u = U0 - F/(2 rho0), F the Korteweg force of the initial
 // density (rp, filled by k_init_density and k_fill_solid), so that
 // U = u + F/(2 rho) of Sec. 2.3.5 equals U0 at t = 0. Zero at solid nodes.
+// The body of the force sweep.
 template <int LAT, typename T = double>
-__global__ void k_init(Geo g, Phys p, const uint8_t *__restrict__ mask,
-                       const double2 *__restrict__ rp, const double *__restrict__ u0,
-                       T *__restrict__ f)
-{
-    constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= g.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
-    if (mask[n]) {
+struct InitBody {
+    const uint8_t *mask;
+    const double2 *rp;
+    const double *u0;
+    T *f;
+
+    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int, int, int,
+                                               const double *sp, const double *sr) const
+    {
+        constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
+        if (mask[n]) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + n] = (T)0;
-        return;
-    }
-    const double2 c = rp[n];
-    const double rho = c.x;
-    double F[3] = {0.0, 0.0, 0.0};
-    korteweg_force<LAT>(g, p, rp, x, y, z, rho, c.y, F);
-    double E[3][3];
+            for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + n] = (T)0;
+            return;
+        }
+        const double2 c = rp[n];
+        const double rho = c.x, half = 0.5 / rho;
+        double F[3];
+        force_of_sums<LAT>(p, rho, c.y, sp, sr, F);
+        double E[3][3];
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const double ua = (u0 ? u0[a * g.N + n] : 0.0) - F[a] / (2.0 * rho);
-        const double ze = 1.0 / 3.0 + ua * ua;
-        E[a][0] = 0.5 * (ze - ua);
-        E[a][1] = 1.0 - ze;
-        E[a][2] = 0.5 * (ze + ua);
-    }
+        for (int a = 0; a < D; ++a) {
+            const double ua = fma(-F[a], half, u0 ? u0[a * (size_t)g.N + n] : 0.0);
+            const double t = 0.5 * ua, h = fma(t, ua, 1.0 / 6.0);
+            E[a][0] = h - t;
+            E[a][1] = fma(-2.0, h, 1.0);
+            E[a][2] = h + t;
+        }
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        double eq = rho * E[0][cxi(i) + 1] * E[1][cyi(i) + 1];
-        if (D == 3) eq *= E[2][czi(i) + 1];
-        f[(size_t)i * g.N + n] = (T)eq;
+        for (int i = 0; i < Q; ++i) {
+            double eq = rho * E[0][cxi(i) + 1] * E[1][cyi(i) + 1];
+            if (D == 3) eq *= E[2][czi(i) + 1];
+            f[(size_t)i * g.N + n] = (T)eq;
+        }
     }
-}
+};
 
 template <int LAT>
 __global__ void k_fill_solid(Geo g, Phys p, const uint8_t *__restrict__ mask,
