@@ -697,9 +697,7 @@ template <int LAT>
 int encode_from(lbm_ctx *h, const double *f)
 {
     const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    // both buffers' source densities: -1 at solid nodes stays for good
-    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->mask, f, h->rs[0]);
-    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->mask, f, h->rs[1]);
+    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->mask, f, h->rs[0], h->rs[1]);
     if (h->storage == LBM_F16S)
         lbmk::k_encode_shifted<LAT, __half><<<gr, bl, 0, h->stream>>>(
             h->geo, f, h->rs[0], static_cast<__half *>(h->fv[0]));
@@ -707,7 +705,7 @@ int encode_from(lbm_ctx *h, const double *f)
         lbmk::k_encode_shifted<LAT, __nv_bfloat16><<<gr, bl, 0, h->stream>>>(
             h->geo, f, h->rs[0], static_cast<__nv_bfloat16 *>(h->fv[0]));
     CU(h, cudaGetLastError());
-    h->launches += 3;
+    h->launches += 2;
     h->cur = 0;
     return LBM_OK;
 }
@@ -774,29 +772,37 @@ int check_ready(lbm_ctx *h)
     return LBM_OK;
 }
 
+// fn(populations of buffer k) with their storage's type.
+template <typename Fn>
+void with_pops(const lbm_ctx *h, int k, const Fn &fn)
+{
+    switch (h->storage) {
+    case LBM_F64: fn(static_cast<const double *>(h->fv[k])); break;
+    case LBM_F32: fn(static_cast<const float *>(h->fv[k])); break;
+    case LBM_F16S: fn(lbmk::Shifted<__half>{static_cast<const __half *>(h->fv[k]), h->rs[k]}); break;
+    default: fn(lbmk::Shifted<__nv_bfloat16>{static_cast<const __nv_bfloat16 *>(h->fv[k]), h->rs[k]});
+    }
+}
+
+// Side fields (rho, s psi), u and rho u_a^3 of the current state.
+template <int LAT>
+void launch_macro(lbm_ctx *h)
+{
+    with_pops(h, h->cur, [&](auto f) {
+        lbmk::k_macro<LAT><<<node_grid(h->geo), node_block(h->geo), 0, h->stream>>>(
+            h->geo, h->phys, h->mask, f, h->rp, h->u, h->gflux, h->status);
+    });
+}
+
 template <int LAT>
 int launch_macro_and_out(lbm_ctx *h, double *rho, double *u, double *U)
 {
-    const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    if (shifted(h->storage)) {
-        TempF64 t;
-        int rc = temp_alloc(h, t);
-        if (!rc) rc = decode_to<LAT>(h, h->cur, t.p);
-        if (rc) return rc;
-        lbmk::k_macro<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, t.p, h->rp, h->u,
-                                                     h->gflux, h->status);
-        CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
-    } else if (h->storage == LBM_F32)
-        lbmk::k_macro<LAT, float><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask,
-                                                            f32(h, h->cur), h->rp, h->u,
-                                                            h->gflux, h->status);
-    else
-        lbmk::k_macro<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, f64(h, h->cur),
-                                                     h->rp, h->u, h->gflux, h->status);
+    launch_macro<LAT>(h);
     if (U)
         launch_sweep<LAT>(h, h->stream, lbmk::MomentsBody<LAT>{h->mask, h->rp, h->u, rho, u, U});
     else
-        lbmk::k_moments_out<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, h->u, rho, u);
+        lbmk::k_moments_out<LAT><<<node_grid(h->geo), node_block(h->geo), 0, h->stream>>>(
+            h->geo, h->phys, h->mask, h->rp, h->u, rho, u);
     CU(h, cudaGetLastError());
     h->launches += 2;
     return LBM_OK;
@@ -805,28 +811,11 @@ int launch_macro_and_out(lbm_ctx *h, double *rho, double *u, double *U)
 template <int LAT>
 int launch_pressure(lbm_ctx *h, double *out)
 {
-    const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    if (shifted(h->storage)) {
-        TempF64 t;
-        int rc = temp_alloc(h, t);
-        if (!rc) rc = decode_to<LAT>(h, h->cur, t.p);
-        if (rc) return rc;
-        lbmk::k_macro<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, t.p, h->rp, h->u,
-                                                     h->gflux, h->status);
-        lbmk::k_pressure_tensor<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, t.p, h->rp, out);
-        CU(h, cudaGetLastError());
-        CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
-    } else if (h->storage == LBM_F32) {
-        lbmk::k_macro<LAT, float><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, f32(h, h->cur),
-                                                            h->rp, h->u, h->gflux, h->status);
-        lbmk::k_pressure_tensor<LAT, float><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask,
-                                                                      f32(h, h->cur), h->rp, out);
-    } else {
-        lbmk::k_macro<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, f64(h, h->cur), h->rp,
-                                                     h->u, h->gflux, h->status);
-        lbmk::k_pressure_tensor<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask,
-                                                               f64(h, h->cur), h->rp, out);
-    }
+    launch_macro<LAT>(h);
+    with_pops(h, h->cur, [&](auto f) {
+        lbmk::k_pressure_tensor<LAT><<<node_grid(h->geo), node_block(h->geo), 0, h->stream>>>(
+            h->geo, h->phys, h->mask, f, h->rp, out);
+    });
     CU(h, cudaGetLastError());
     h->launches += 2;
     return LBM_OK;
@@ -874,25 +863,10 @@ int launch_fill_solid(lbm_ctx *h)
 template <int LAT>
 int launch_reduce(lbm_ctx *h)
 {
-    if (shifted(h->storage)) {
-        TempF64 t;
-        int rc = temp_alloc(h, t);
-        if (!rc) rc = decode_to<LAT>(h, h->cur, t.p);
-        if (rc) return rc;
-        lbmk::k_reduce_partial<LAT><<<lbmk::RED_BLOCKS, lbmk::RED_THREADS, 0, h->stream>>>(
-            h->geo, h->mask, t.p, h->partial);
-        lbmk::k_reduce_final<<<1, lbmk::RED_BLOCKS, 0, h->stream>>>(h->partial, h->sums);
-        CU(h, cudaGetLastError());
-        CU(h, cudaStreamSynchronize(h->stream));
-        h->launches += 2;
-        return LBM_OK;
-    }
-    if (h->storage == LBM_F32)
-        lbmk::k_reduce_partial<LAT, float><<<lbmk::RED_BLOCKS, lbmk::RED_THREADS, 0, h->stream>>>(
-            h->geo, h->mask, f32(h, h->cur), h->partial);
-    else
-        lbmk::k_reduce_partial<LAT><<<lbmk::RED_BLOCKS, lbmk::RED_THREADS, 0, h->stream>>>(
-            h->geo, h->mask, f64(h, h->cur), h->partial);
+    with_pops(h, h->cur, [&](auto f) {
+        lbmk::k_reduce_partial<LAT><<<lbmk::RED_BLOCKS, lbmk::RED_THREADS, 0, h->stream>>>(h->geo, h->mask, f,
+                                                                                           h->partial);
+    });
     lbmk::k_reduce_final<<<1, lbmk::RED_BLOCKS, 0, h->stream>>>(h->partial, h->sums);
     CU(h, cudaGetLastError());
     h->launches += 2;
@@ -1289,13 +1263,17 @@ int lbm_get_populations(lbm_handle h, double *f, int on_device)
     if (!f) return LBM_EINVAL;
     const size_t N = h->geo.N, QN = (size_t)h->Q * N;
     if (shifted(h->storage)) {
-        TempF64 t;
-        rc = temp_alloc(h, t);
-        if (!rc) rc = h->lattice == LBM_D2Q9 ? decode_to<0>(h, h->cur, t.p) : decode_to<1>(h, h->cur, t.p);
+        TempF64 t;   // of a host buffer; an aligned device buffer is written in place
+        const bool direct = on_device && reinterpret_cast<uintptr_t>(f) % sizeof(double) == 0;
+        if (!direct && (rc = temp_alloc(h, t))) return rc;
+        double *out = direct ? f : t.p;
+        rc = h->lattice == LBM_D2Q9 ? decode_to<0>(h, h->cur, out) : decode_to<1>(h, h->cur, out);
         if (rc) return rc;
-        CU(h, cudaMemcpyAsync(f, t.p, sizeof(double) * QN,
-                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
-        CU(h, cudaStreamSynchronize(h->stream));
+        if (!direct) {
+            CU(h, cudaMemcpyAsync(f, t.p, sizeof(double) * QN,
+                                  on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+            CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
+        }
     } else if (h->storage == LBM_F32) {
         if (on_device) {
             lbmk::k_convert<float, double><<<1024, 256, 0, h->stream>>>(QN, f32(h, h->cur), f);
@@ -1329,14 +1307,17 @@ int lbm_set_populations(lbm_handle h, const double *f, int on_device)
     const size_t QN = (size_t)h->Q * h->geo.N;
     h->cur = 0;
     if (shifted(h->storage)) {
-        TempF64 t;
-        rc = temp_alloc(h, t);
+        TempF64 t;   // of a host buffer; an aligned device buffer is read in place
+        const bool direct = on_device && reinterpret_cast<uintptr_t>(f) % sizeof(double) == 0;
+        if (!direct) {
+            if ((rc = temp_alloc(h, t))) return rc;
+            CU(h, cudaMemcpyAsync(t.p, f, sizeof(double) * QN,
+                                  on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
+        }
+        const double *in = direct ? f : t.p;
+        rc = h->lattice == LBM_D2Q9 ? encode_from<0>(h, in) : encode_from<1>(h, in);
         if (rc) return rc;
-        CU(h, cudaMemcpyAsync(t.p, f, sizeof(double) * QN,
-                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
-        rc = h->lattice == LBM_D2Q9 ? encode_from<0>(h, t.p) : encode_from<1>(h, t.p);
-        if (rc) return rc;
-        CU(h, cudaStreamSynchronize(h->stream));
+        if (!direct) CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
     } else if (h->storage == LBM_F32) {
         if (on_device) {
             lbmk::k_convert<double, float><<<1024, 256, 0, h->stream>>>(QN, f, f32(h, 0));

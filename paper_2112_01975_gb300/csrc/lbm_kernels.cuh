@@ -135,6 +135,26 @@ __device__ __forceinline__ double signed_psi(const Phys &p, double rho)
 __device__ __forceinline__ int wrapm(int v, int n) { return v < 0 ? v + n : v; }
 __device__ __forceinline__ int wrapp(int v, int n) { return v >= n ? v - n : v; }
 
+// Of shifted 16-bit storage: the weight and the node that pushed population i.
+__device__ __forceinline__ double weight_d(int i, int D)
+{
+    const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
+    return w1[cxi(i) + 1] * w1[cyi(i) + 1] * (D == 3 ? w1[czi(i) + 1] : 1.0);
+}
+
+__device__ __forceinline__ unsigned source_node(const Geo &g, int D, int i, int x, int y, int z)
+{
+    const int sx = (x - cxi(i) + g.nx) % g.nx, sy = (y - cyi(i) + g.ny) % g.ny;
+    const int sz = D == 3 ? (z - czi(i) + g.nz) % g.nz : 0;
+    return sx + g.nx * (sy + g.ny * sz);
+}
+
+}  // namespace lbmk
+
+#include "lbm_fixed.cuh"
+
+namespace lbmk {
+
 // ---- the Korteweg force of every node ---------------------------------
 //   F = -2 (s psi)_c S_psi - kappa rho_c S_rho + rho_c g,
 //   S_psi = sum_i (w_i/cs2) c_i [4/3 psi(r+c_i) - 1/6 psi(r+2c_i)],
@@ -325,42 +345,22 @@ k_force_sweep2(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
 }
 
 // Moments, EOS and pseudo-potential of every fluid node; flags bad densities.
-// Populations are stored as T (double, or float for FP32 storage); the
-// arithmetic here is FP64 either way.
-template <int LAT, typename T = double>
-__global__ void k_macro(Geo g, Phys p, const uint8_t *__restrict__ mask,
-                        const T *__restrict__ f, double2 *__restrict__ rp,
-                        double *__restrict__ u, double *__restrict__ gflux,
-                        int *__restrict__ status)
+// P: the populations' storage (double, float or Shifted); the moments are
+// FP64 either way.
+template <int LAT, typename P>
+__global__ void k_macro(Geo g, Phys p, const uint8_t *__restrict__ mask, P f, double2 *__restrict__ rp,
+                        double *__restrict__ u, double *__restrict__ gflux, int *__restrict__ status)
 {
-    constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
+    constexpr int D = Lattice<LAT>::D;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
     const unsigned n = x + g.nx * (y + g.ny * z);
     if (mask[n]) return;
-    // Row sums along x for each (cy, cz), then the moments from them.
-    double fi[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) fi[i] = (double)f[(size_t)i * g.N + n];
-    constexpr int R = Q / 3;
-    double row[R], jx = 0.0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        row[r] = fi[3 * r] + fi[3 * r + 1] + fi[3 * r + 2];
-        jx += fi[3 * r + 2] - fi[3 * r];
-    }
-    double rho = 0.0, jy = 0.0, jz = 0.0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        rho += row[r];
-        const int cy = r % 3 - 1, cz = r / 3 - 1;
-        if (cy > 0) jy += row[r]; else if (cy < 0) jy -= row[r];
-        if (D == 3) { if (cz > 0) jz += row[r]; else if (cz < 0) jz -= row[r]; }
-    }
+    double rho, j[3];
+    node_sums<LAT, false>(g, f, n, x, y, z, rho, j);
     double inv;
     const double d = excess_pressure(p, rho, inv);
-    const double j[3] = {jx, jy, jz};
     bool ok = positive(rho) && finite_bits(rho);
     rp[n] = make_double2(rho, signed_psi_of(d));
 #pragma unroll
@@ -549,10 +549,14 @@ __global__ void k_interp_bounce_back(Geo g, const unsigned *__restrict__ bn,
 // X[v] = sum_i (w_i/cs2) c_ia c_ib v(r - c_i) v(r + c_i).
 // Needs rp of the current state (k_macro). Components xx, yy[, zz],
 // xy[, xz, yz] as N-planes; 0 at solid nodes.
-template <int LAT, typename T = double>
-__global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mask,
-                                  const T *__restrict__ f, const double2 *__restrict__ rp,
-                                  double *__restrict__ out)
+// All terms but the populations' are linear in what a pair of opposite
+// neighbours gives with the weight w_i c_ia c_ib, so each of the 13 (4)
+// pairs forms its sum T of all terms once (12 FP64 operations) and the T are
+// added by weight class: about 220 operations per node where term by term
+// and component by component took 1200 (160^3: 11.1 ms).
+template <int LAT, typename P>
+__global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mask, P f,
+                                  const double2 *__restrict__ rp, double *__restrict__ out)
 {
     constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q, NA = D == 3 ? 6 : 3;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -566,42 +570,55 @@ __global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mas
         for (int k = 0; k < NA; ++k) out[(size_t)k * g.N + n] = 0.0;
         return;
     }
-    double kin[NA], pa[NA], pb1[NA], pb2[NA], pc[NA], pd1[NA], pd2[NA];
+    double rho, j[3], kin[6];
+    node_sums<LAT, true>(g, f, n, x, y, z, rho, j, kin);
+    const double2 c0 = rp[n];
+    const double r = c0.x, sps = c0.y;   // s psi; s = +1 where P > P0, else -1
+    const double s6 = positive(sps) ? -1.0 / 3.0 : 1.0 / 3.0;
+    const double c1 = 4.0 / 3.0 * sps, c2 = -1.0 / 6.0 * sps;
+    const double c3 = p.kappa * r, c4 = -0.5 * c3;
+    int X[5], Y[5], Z[5];
 #pragma unroll
-    for (int k = 0; k < NA; ++k) kin[k] = pa[k] = pb1[k] = pb2[k] = pc[k] = pd1[k] = pd2[k] = 0.0;
+    for (int k = -2; k <= 2; ++k) {
+        X[k + 2] = k < 0 ? wrapm(x + k, g.nx) : wrapp(x + k, g.nx);
+        Y[k + 2] = k < 0 ? wrapm(y + k, g.ny) : wrapp(y + k, g.ny);
+        Z[k + 2] = D == 2 ? 0 : k < 0 ? wrapm(z + k, g.nz) : wrapp(z + k, g.nz);
+    }
+    // sums of T by component and weight class (nonzero components of c less one)
+    double acc[6][3];
+    bool set[6][3] = {};
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
+    for (int i = Q / 2 + 1; i < Q; ++i) {
         const int c[3] = {cxi(i), cyi(i), D == 3 ? czi(i) : 0};
-        const double fi = (double)f[(size_t)i * g.N + n];
         const auto at = [&](int k) {
-            const int xx = (x + k * c[0] + 2 * g.nx) % g.nx;
-            const int yy = (y + k * c[1] + 2 * g.ny) % g.ny;
-            const int zz = D == 3 ? (z + k * c[2] + 2 * g.nz) % g.nz : 0;
-            return rp[xx + g.nx * (yy + g.ny * zz)];
+            return rp[X[k * c[0] + 2] + g.nx * (Y[k * c[1] + 2] + g.ny * Z[k * c[2] + 2])];
         };
-        const double2 v1 = at(1), v2 = at(2), vm = at(-1);
-        const double wi = (D == 3 ? (c[0] ? 1.0 / 6.0 : 2.0 / 3.0) * (c[1] ? 1.0 / 6.0 : 2.0 / 3.0) *
-                                        (c[2] ? 1.0 / 6.0 : 2.0 / 3.0)
-                                  : (c[0] ? 1.0 / 6.0 : 2.0 / 3.0) * (c[1] ? 1.0 / 6.0 : 2.0 / 3.0)) * 3.0;
+        const double2 p1 = at(1), m1 = at(-1), p2 = at(2), m2 = at(-2);
+        double T = c1 * (fabs(p1.y) + fabs(m1.y));
+        T = fma(c2, fabs(p2.y) + fabs(m2.y), T);
+        T = fma(s6, fabs(p1.y * m1.y), T);
+        T = fma(c3, p1.x + m1.x, T);
+        T = fma(c4, p2.x + m2.x, T);
+        T = fma(-p.kappa, p1.x * m1.x, T);
+        const int cls = (c[0] != 0) + (c[1] != 0) + (c[2] != 0) - 1;
 #pragma unroll
         for (int k = 0; k < NA; ++k) {
-            const double cc = (double)(c[CA[k]] * c[CB[k]]);
-            kin[k] += cc * fi;
-            const double wc = wi * cc;
-            pa[k] += wc * fabs(v1.y);
-            pb1[k] += wc * fabs(v2.y);
-            pb2[k] += wc * fabs(vm.y) * fabs(v1.y);
-            pc[k] += wc * v1.x;
-            pd1[k] += wc * v2.x;
-            pd2[k] += wc * vm.x * v1.x;
+            const int cc = c[CA[k]] * c[CB[k]];
+            if (cc == 0) continue;
+            acc[k][cls] = !set[k][cls] ? (cc > 0 ? T : -T) : cc > 0 ? acc[k][cls] + T : acc[k][cls] - T;
+            set[k][cls] = true;
         }
     }
-    const double2 c0 = rp[n];
-    const double sg = c0.y > 0.0 ? 1.0 : -1.0, ps = fabs(c0.y), r = c0.x;
+    // 3 w_i of the classes
+    const double w[3] = {D == 3 ? 2.0 / 9.0 : 1.0 / 3.0, D == 3 ? 1.0 / 18.0 : 1.0 / 12.0, 1.0 / 72.0};
 #pragma unroll
-    for (int k = 0; k < NA; ++k)
-        out[(size_t)k * g.N + n] = kin[k] + sg * (4.0 / 3.0) * ps * pa[k] - sg * (1.0 / 6.0) * (ps * pb1[k] + pb2[k]) +
-                                   p.kappa * r * pc[k] - 0.5 * p.kappa * (r * pd1[k] + pd2[k]);
+    for (int k = 0; k < NA; ++k) {
+        double v = kin[k];
+#pragma unroll
+        for (int cls = 0; cls < D; ++cls)
+            if (set[k][cls]) v = fma(w[cls], acc[k][cls], v);
+        out[(size_t)k * g.N + n] = v;
+    }
 }
 
 // Side field of the initial density: rp = (rho0, s psi(rho0)) at fluid nodes
@@ -690,24 +707,22 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-template <int LAT, typename T = double>
+template <int LAT, typename P>
 __global__ void __launch_bounds__(RED_THREADS)
-k_reduce_partial(Geo g, const uint8_t *__restrict__ mask, const T *__restrict__ f,
-                 double *__restrict__ partial)
+k_reduce_partial(Geo g, const uint8_t *__restrict__ mask, P f, double *__restrict__ partial)
 {
-    constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
+    constexpr int D = Lattice<LAT>::D;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const unsigned plane = (unsigned)g.nx * (unsigned)g.ny;
     for (unsigned n = blockIdx.x * RED_THREADS + threadIdx.x; n < g.N;
          n += RED_THREADS * RED_BLOCKS) {
         if (mask[n]) continue;
+        const unsigned z = n / plane, y = (n - z * plane) / g.nx, x = n - z * plane - y * g.nx;
+        double rho, j[3];
+        node_sums<LAT, false>(g, f, n, x, y, z, rho, j);
+        acc[0] += rho;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const double fi = (double)f[(size_t)i * g.N + n];
-            acc[0] += fi;
-            if (cxi(i)) acc[1] += cxi(i) * fi;
-            if (cyi(i)) acc[2] += cyi(i) * fi;
-            if (D == 3 && czi(i)) acc[3] += czi(i) * fi;
-        }
+        for (int a = 0; a < D; ++a) acc[1 + a] += j[a];
     }
     __shared__ double sh[4][RED_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -749,19 +764,6 @@ k_reduce_final(const double *__restrict__ partial, double *__restrict__ out)
 
 // Shifted 16-bit storage (h_i = f_i / rho(src) - w_i, src = r - c_i, or r itself
 // when r - c_i is solid): decode to FP64, per-node densities, encode.
-__device__ __forceinline__ double weight_d(int i, int D)
-{
-    const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
-    return w1[cxi(i) + 1] * w1[cyi(i) + 1] * (D == 3 ? w1[czi(i) + 1] : 1.0);
-}
-
-__device__ __forceinline__ unsigned source_node(const Geo &g, int D, int i, int x, int y, int z)
-{
-    const int sx = (x - cxi(i) + g.nx) % g.nx, sy = (y - cyi(i) + g.ny) % g.ny;
-    const int sz = D == 3 ? (z - czi(i) + g.nz) % g.nz : 0;
-    return sx + g.nx * (sy + g.ny * sz);
-}
-
 template <int LAT, typename ST>
 __global__ void k_decode_shifted(Geo g, const ST *__restrict__ h, const float *__restrict__ rho_src,
                                  double *__restrict__ f)
@@ -776,29 +778,37 @@ __global__ void k_decode_shifted(Geo g, const ST *__restrict__ h, const float *_
         // a solid source (density -1) means a population bounced by n itself
         float src = rho_src[source_node(g, D, i, x, y, z)];
         if (src < 0.0f) src = rho_src[n];
-        f[(size_t)i * g.N + n] = (weight_d(i, D) + (double)lbmf::to_f(h[(size_t)i * g.N + n])) * (double)src;
+        f[(size_t)i * g.N + n] = (weight_d(i, D) + widen(lbmf::to_f(h[(size_t)i * g.N + n]))) * widen(src);
     }
 }
 
-// The source-density field of shifted storage: each fluid node's density,
-// -1 at solid nodes (their populations' sources are the fluid nodes that
-// bounced them; see the decoders).
+// The source-density field of shifted storage, written to both buffers (-1 at
+// solid nodes stays for good): each fluid node's density, -1 at solid nodes
+// (their populations' sources are the fluid nodes that bounced them; see the
+// decoders).
 template <int LAT>
 __global__ void k_density(Geo g, const uint8_t *__restrict__ mask, const double *__restrict__ f,
-                          float *__restrict__ rho)
+                          float *__restrict__ rho0, float *__restrict__ rho1)
 {
-    constexpr int Q = Lattice<LAT>::Q;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const unsigned n = x + g.nx * (blockIdx.y + g.ny * blockIdx.z);
-    if (mask[n]) {
-        rho[n] = -1.0f;
-        return;
+    float v = -1.0f;
+    if (!mask[n]) {
+        double s, j[3];
+        node_sums<LAT, false>(g, f, n, x, blockIdx.y, blockIdx.z, s, j);
+        v = (float)s;
     }
-    double s = 0.0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) s += f[(size_t)i * g.N + n];
-    rho[n] = (float)s;
+    rho0[n] = rho1[n] = v;
+}
+
+// 1/v of a float in FP64, to 2^-46: a Newton step on its FP32 reciprocal (the
+// division below goes on to 16 bits; in full it is 8 FP64 operations).
+__device__ __forceinline__ double reciprocal_of(float v)
+{
+    const float r = __frcp_rn(v);
+    const double a = widen(v), b = widen(r);
+    return r > 0.0f && r < 3.0e38f ? fma(b, fma(-a, b, 1.0), b) : 1.0 / a;
 }
 
 template <int LAT, typename ST>
@@ -820,7 +830,7 @@ __global__ void k_encode_shifted(Geo g, const double *__restrict__ f, const floa
         float src = rho[source_node(g, D, i, x, y, z)];
         if (src < 0.0f) src = rho[n];   // bounced by n itself
         h[(size_t)i * g.N + n] =
-            lbmf::from_f<ST>((float)(f[(size_t)i * g.N + n] / (double)src - weight_d(i, D)));
+            lbmf::from_f<ST>((float)fma(f[(size_t)i * g.N + n], reciprocal_of(src), -weight_d(i, D)));
     }
 }
 
@@ -830,7 +840,8 @@ __global__ void k_convert(size_t n, const A *__restrict__ in, B *__restrict__ ou
 {
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x)
-        out[k] = (B)in[k];
+        if constexpr (sizeof(A) == 4) out[k] = widen(in[k]);
+        else                          out[k] = (B)in[k];
 }
 
 // FP64 throughput probe: eight independent fused multiply-add chains per
