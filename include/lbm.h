@@ -268,13 +268,16 @@ int lbm_selftest_wait_timeout(long long limit_cycles, int *status_bits, double *
 int lbm_time_kernels(lbm_handle h, int64_t n, double *ms);
 
 /* Planes per CTA along the march axis (z; the 2D y axis for D2Q9) of the
- * fused FP32 step, >= 1 (default 16 for D3Q27, 64 for D2Q9). A tuning knob:
- * results do not depend on it; D2Q9 steps, which march along nothing, take
+ * fused FP32 step, >= 1. A tuning knob: results do not depend on it. Until
+ * the form, tile or chunk is set or tuned, a D3Q27 handle takes the form and
+ * the chunk that suit its lattice; once one of them is set, the others are
+ * the plain form's (LBM_FUSED_PLAIN, 8 rows, chunk 16). D2Q9 steps, which march along nothing, take
  * it and run the same. */
 int lbm_set_chunk(lbm_handle h, int chunk);
 
 /* Pick the chunk of the fused FP32 step by timing candidates (4 to 128
- * planes and, on a longer march axis, 10/16 to 16/16 of it) on the
+ * planes, on a longer march axis 10/16 to 16/16 of it, and the chunks that
+ * handles left open take) on the
  * handle's own state (saved to a temporary device buffer and restored
  * afterwards, so the state is unchanged). Sets and returns it in
  * *chunk_out (0 for FP64 storage, which has no tile parameter; D2Q9, whose
@@ -305,8 +308,11 @@ int lbm_set_tile(lbm_handle h, int tile_y);
 /* Forms of the fused step of the reduced storages (LBM_F32 all but
  * LBM_FUSED_TM_TMA; LBM_F16S and LBM_BF16S all but
  * LBM_FUSED_WARP_SPECIALISED); the same arithmetic in the same order, so
- * results are bitwise the same whichever runs.
- *   LBM_FUSED_PLAIN (default): one thread group per tile; each entering
+ * results are bitwise the same whichever runs. A D3Q27 handle whose form,
+ * tile and chunk were neither set nor tuned runs the TMA-staged form of its
+ * storage from its first use of device memory on (LBM_FUSED_TMEM where there
+ * is none, LBM_FUSED_PLAIN with LBM_FLAG_EOS_F64).
+ *   LBM_FUSED_PLAIN: one thread group per tile; each entering
  *     plane's densities, pseudo-potentials and velocities are formed, the
  *     block synchronises, and the plane two behind collides and streams,
  *     reading its node's populations again (an L2 hit).
@@ -361,7 +367,8 @@ enum {
  * maps. */
 int lbm_set_fused_variant(lbm_handle h, int variant);
 
-/* *variant = the form of the fused step in use. */
+/* *variant = the form of the fused step in use (LBM_FUSED_PLAIN before the
+ * device memory is laid out, if none was set). */
 int lbm_get_fused_variant(lbm_handle h, int *variant);
 
 /* ---- Batches: many lattices advanced by one persistent launch ----------

@@ -32,7 +32,10 @@ struct lbm_ctx {
     GeoF geof;     // FP32 fused step: 3D frame (D2Q9: ny = 1, nz = 2D y extent)
     PhysF physf;
     int tile_rows = 8;   // D3Q27 FP32 step: 32 x 8 (lbmf) or 32 x 7 (lbmf7) tiles
-    int variant = LBM_FUSED_PLAIN;   // FP32 step: plain, warp-specialised or Tensor Memory form
+    int variant = LBM_FUSED_PLAIN;   // form of the fused step
+    // D3Q27 reduced storage: the form and chunk follow the lattice
+    // (choose_form) until the caller sets or tunes any of them
+    bool auto_form = true;
     bool e64 = false;    // reduced storage: EOS, psi and force sums in FP64 (LBM_FLAG_EOS_F64)
     int storage, flags;
     double t_over_tc, tau;
@@ -226,6 +229,83 @@ dim3 node_grid(const Geo &g)
 
 void make_tensor_maps(lbm_ctx *h);
 
+// Makespan of n_full blocks of cost cf, then n_tail of cost ct <= cf, each
+// taken by the first of `slots` that is free.
+double makespan(long long n_full, double cf, long long n_tail, double ct, long long slots)
+{
+    const long long k = n_full / slots, r = n_full % slots;
+    const double lo = k * cf, hi = r ? lo + cf : lo;   // slots - r end at lo, r at hi
+    if (n_tail == 0) return hi;
+    double a = hi, b = hi + (n_tail / slots + 1) * ct;   // n_tail fit before b
+    for (int it = 0; it < 40; ++it) {
+        const double t = 0.5 * (a + b);
+        const long long fit = (slots - r) * (long long)((t - lo) / ct + 1e-9) + r * (long long)((t - hi) / ct + 1e-9);
+        if (fit >= n_tail) b = t;
+        else               a = t;
+    }
+    return b;
+}
+
+// The chunk of planes per block that ends the step first: a block of c planes
+// marches through c + 4. `resident` blocks share an SM; two together take
+// 1.31 times as long per plane as one alone (measured: 5.4 against 4.1 us,
+// shifted storage at 128^3). The last, shorter chunk of each column fills the
+// SMs that the whole ones leave. Measured, TMA-staged forms, the choice here
+// against the best chunk of a scan: FP32 64^3 24.8 us (chunk 7; 8: 26.6),
+// 128^3 110.8 (56; 64: 122.7, 16: 145), 160^3 200 (108; 54: 205), 256^3 786
+// (223; 64: 828); FP16-shifted 128^3 177 (29; 32: 192), 256^3 1161 (223).
+int best_chunk(const GeoF &g, int rows, int sms, int resident)
+{
+    const long long tiles = (long long)((g.nx + 31) / 32) * ((g.ny + rows - 1) / rows);
+    int best = 1;
+    double cost = 1e300;
+    for (int c = 1; c <= g.nz; ++c) {
+        const long long full = tiles * (g.nz / c), tail = g.nz % c ? tiles : 0;
+        const double cf = c + 4.5, ct = g.nz % c + 4.5;
+        double t = makespan(full, cf, tail, ct, sms);
+        if (resident == 2 && full + tail > sms) t = 1.31 * makespan(full, cf, tail, ct, 2ll * sms);
+        if (t <= cost) {
+            cost = t;
+            best = c;
+        }
+    }
+    return best;
+}
+
+constexpr int kDefaultChunk3 = 16;
+
+// Form and chunk of a D3Q27 handle of reduced storage that the caller has
+// left open: with tensor maps the TMA-staged form of the storage, the
+// fastest of the forms at every size measured, each at its best chunk (FP32
+// 64^3 25 us against 29 for the next, 128^3 111 against 160, 256^3 786
+// against 1177; FP16-shifted 128^3 177 against 203, 256^3 1161 against
+// 1404), without them the Tensor Memory form (97 x 61 x 75 FP32: 58 us, plain
+// 60), with the FP64 EOS the plain one. The fixed default before, plain at
+// chunk 16: FP32 64^3 62, 128^3 184, 256^3 1208; FP16-shifted 258, 1649.
+void choose_form(lbm_ctx *h)
+{
+    if (!h->auto_form || h->lattice != LBM_D3Q27 || h->storage == LBM_F64) return;
+    if (h->e64) h->variant = LBM_FUSED_PLAIN;
+    else if (!h->tmap_ready) h->variant = LBM_FUSED_TMEM;
+    else h->variant = h->storage == LBM_F32 ? LBM_FUSED_WS_TMA : LBM_FUSED_TM_TMA;
+    h->geof.chunk = best_chunk(h->geof, 8, h->sms, h->variant == LBM_FUSED_WS_TMA ? 1 : 2);
+}
+
+// The caller sets one of form, tile and chunk: the others start from the
+// plain form's.
+void leave_auto_form(lbm_ctx *h)
+{
+    if (!h->auto_form) return;
+    h->auto_form = false;
+    if (h->lattice != LBM_D3Q27 || h->storage == LBM_F64) return;
+    h->variant = LBM_FUSED_PLAIN;
+    h->geof.chunk = kDefaultChunk3;
+    if (h->graph) {   // the captured graph holds the chosen form
+        cudaGraphExecDestroy(h->graph);
+        h->graph = nullptr;
+    }
+}
+
 int ensure_memory(lbm_ctx *h)
 {
     if (h->fv[0]) return LBM_OK;
@@ -270,6 +350,7 @@ int ensure_memory(lbm_ctx *h)
     make_tensor_maps(h);
     if (h->variant == LBM_FUSED_WS_TMA && !h->tmap_ready) h->variant = LBM_FUSED_WS_TMEM;
     if (h->variant == LBM_FUSED_TM_TMA && !h->tmap_ready) h->variant = LBM_FUSED_TMEM;
+    choose_form(h);
     return LBM_OK;
 }
 
@@ -994,7 +1075,7 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
     h->geof.ny = lattice == LBM_D2Q9 ? 1 : ny;
     h->geof.nz = lattice == LBM_D2Q9 ? ny : nz;
     h->geof.N = h->geo.N;
-    h->geof.chunk = lattice == LBM_D2Q9 ? 64 : 16;
+    h->geof.chunk = lattice == LBM_D2Q9 ? 64 : kDefaultChunk3;
     PhysF &pf = h->physf;
     pf.eos = eos;
     pf.a = (float)ph.a;
@@ -1553,10 +1634,12 @@ int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
         // D3Q27: 32 x 8 columns by z-chunks; D2Q9: 32 x 8 tiles of the (x, 2D y) plane
         const int tx = (h->geof.nx + 31) / 32;
         const int ty = ((lattice == LBM_D2Q9 ? h->geof.nz : h->geof.ny) + 7) / 8;
-        const int tz = lattice == LBM_D2Q9 ? 1 : (h->geof.nz + h->geof.chunk - 1) / h->geof.chunk;
+        GeoF geof = h->geof;
+        if (h->auto_form && lattice == LBM_D3Q27) geof.chunk = kDefaultChunk3;   // the batch runs the plain form
+        const int tz = lattice == LBM_D2Q9 ? 1 : (geof.nz + geof.chunk - 1) / geof.chunk;
         for (int par = 0; par < 2; ++par) {
             lbmf::MemberF m;
-            m.g = h->geof;
+            m.g = geof;
             m.p = h->physf;
             m.mask = h->any_solid ? h->mask : nullptr;
             m.src = h->fv[h->cur ^ par];
@@ -1746,7 +1829,11 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
     std::vector<int> cands = {4, 6, 8, 11, 13, 16, 22, 26, 32, 43, 64, 128};
     if (nz > 128)
         for (int k = 10; k <= 16; ++k) cands.push_back(std::max(129, nz * k / 16));
+    for (int resident : {1, 2}) cands.push_back(best_chunk(h->geof, 8, h->sms, resident));
+    std::sort(cands.begin(), cands.end());
     const int chunk0 = h->geof.chunk, rows0 = h->tile_rows;   // restored on failure
+    const bool auto0 = h->auto_form;
+    h->auto_form = false;
     // FP32: the plain, warp-specialised and Tensor Memory kernels; D3Q27 FP32
     // also 32 x 8 and 32 x 7 tiles (the shifted and batched steps use plain
     // 32 x 8)
@@ -1783,6 +1870,7 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
     h->tile_rows = rc == LBM_OK ? best_rows : rows0;
     h->geof.chunk = rc == LBM_OK ? best : chunk0;
     h->variant = rc == LBM_OK ? best_variant : variant0;
+    if (rc != LBM_OK) h->auto_form = auto0;
     if (h->graph) {
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
@@ -1821,8 +1909,9 @@ int lbm_set_tile(lbm_handle h, int tile_y)
         return fail(h, LBM_EINVAL, "the tile height is a parameter of the D3Q27 FP32 step only");
     if (tile_y != 7 && tile_y != 8) return fail(h, LBM_EINVAL, "tile height must be 7 or 8");
     if (tile_y == 7 && h->e64) return fail(h, LBM_EINVAL, "the FP64-EOS step runs 8-row tiles");
-    if (tile_y == 7 && h->variant >= LBM_FUSED_WS_TMEM)
+    if (tile_y == 7 && !h->auto_form && h->variant >= LBM_FUSED_WS_TMEM)
         return fail(h, LBM_EINVAL, "the warp-specialised Tensor Memory forms run 8-row tiles");
+    leave_auto_form(h);
     if (h->tile_rows != tile_y && h->graph) {   // the captured graph holds the other kernel
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
@@ -1851,6 +1940,7 @@ int lbm_set_fused_variant(lbm_handle h, int variant)
         return fail(h, LBM_EINVAL, "the FP64-EOS step has one form");
     if (shifted(h->storage) && variant == LBM_FUSED_WARP_SPECIALISED)
         return fail(h, LBM_EINVAL, "shifted storage has the plain and the Tensor Memory forms");
+    leave_auto_form(h);
     if (h->variant != variant && h->graph) {   // the captured graph holds the other kernel
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
@@ -1870,6 +1960,7 @@ int lbm_set_chunk(lbm_handle h, int chunk)
 {
     if (!h) return LBM_EINVAL;
     if (chunk < 1) return fail(h, LBM_EINVAL, "chunk must be >= 1");
+    leave_auto_form(h);
     if (h->geof.chunk != chunk && h->graph) {
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
