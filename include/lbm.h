@@ -151,7 +151,9 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos,
                const lbm_params *p);
 
 /* Device bytes a handle of this shape and storage needs (populations,
- * side fields, mask, reduction partials), or 0 for invalid arguments. */
+ * side fields, mask, reduction partials), or 0 for invalid arguments. In D3Q27
+ * reduced storage each row of nx nodes takes a multiple of 16 bytes of
+ * populations (4 FP32 or 8 16-bit ones); callers' arrays never do. */
 size_t lbm_required_bytes(int lattice, int nx, int ny, int nz, int storage);
 
 /* Use caller-owned device memory (e.g. a torch tensor) of at least
@@ -311,7 +313,10 @@ int lbm_set_tile(lbm_handle h, int tile_y);
  * results are bitwise the same whichever runs. A D3Q27 handle whose form,
  * tile and chunk were neither set nor tuned runs the TMA-staged form of its
  * storage from its first use of device memory on (LBM_FUSED_TMEM where there
- * is none, LBM_FUSED_PLAIN with LBM_FLAG_EOS_F64).
+ * is none, where nx leaves remainder 1 by 4 (FP32) or 8 (shifted), or where
+ * the tiles of shifted storage hang far over the lattice; LBM_FUSED_PLAIN
+ * with LBM_FLAG_EOS_F64). For other nx that are not a multiple of 4 or 8 the
+ * TMA-staged forms run only by that choice or lbm_autotune's.
  *   LBM_FUSED_PLAIN: one thread group per tile; each entering
  *     plane's densities, pseudo-potentials and velocities are formed, the
  *     block synchronises, and the plane two behind collides and streams,

@@ -133,6 +133,21 @@ Layout layout_for(int D, int Q, size_t N, int storage, size_t planes)
     return L;
 }
 
+// Row alignment of the TMA-staged forms: rows of 16 bytes, 4 FP32 or 8 16-bit
+// populations.
+int tma_nx_multiple(int storage) { return storage == LBM_F32 ? 4 : shifted(storage) ? 8 : 0; }
+
+// Entries per row of the library's own fields: nx, in D3Q27 reduced storage
+// rounded up so that every row starts on 16 bytes and lattices of any width
+// have a TMA-staged form (unless entry numbers then leave 32 bits).
+int row_pitch(int lattice, int nx, int ny, int nz, int storage)
+{
+    const int mult = tma_nx_multiple(storage);
+    if (lattice != LBM_D3Q27 || !mult) return nx;
+    const int px = (nx + mult - 1) / mult * mult;
+    return (double)px * ny * nz * 27.0 <= 4.2e9 ? px : nx;
+}
+
 bool valid_shape(int lattice, int nx, int ny, int nz)
 {
     if (lattice != LBM_D2Q9 && lattice != LBM_D3Q27) return false;
@@ -279,14 +294,22 @@ constexpr int kDefaultChunk3 = 16;
 // fastest of the forms at every size measured, each at its best chunk (FP32
 // 64^3 25 us against 29 for the next, 128^3 111 against 160, 256^3 786
 // against 1177; FP16-shifted 128^3 177 against 203, 256^3 1161 against
-// 1404), without them the Tensor Memory form (97 x 61 x 75 FP32: 58 us, plain
-// 60), with the FP64 EOS the plain one. The fixed default before, plain at
-// chunk 16: FP32 64^3 62, 128^3 184, 256^3 1208; FP16-shifted 258, 1649.
+// 1404). The Tensor Memory form without tensor maps, where a column of the
+// halo lies in no box (box_pos; 153 x 145 x 131 FP32: 215 us against 290) and,
+// in shifted storage, where the tiles hang over the lattice by more than a
+// tenth: there it reads less, while the TMA-staged form's nine copies cost the
+// same (98 x 61 x 75: 71 against 80 us, 45 x 37 x 60: 36 against 41, 150^3: 309
+// against 300; FP32 98 x 61 x 75: 53 against 47). With the FP64 EOS the plain
+// one. The fixed default before, plain at chunk 16: FP32 64^3 62, 128^3 184,
+// 256^3 1208; FP16-shifted 258, 1649.
 void choose_form(lbm_ctx *h)
 {
     if (!h->auto_form || h->lattice != LBM_D3Q27 || h->storage == LBM_F64) return;
+    const Geo &g = h->geo;
+    const bool stray = g.nx % tma_nx_multiple(h->storage) == 1;   // a halo column in no box
+    const double use = (double)g.nx * g.ny / (((g.nx + 31) / 32 * 32.0) * ((g.ny + 7) / 8 * 8.0));
     if (h->e64) h->variant = LBM_FUSED_PLAIN;
-    else if (!h->tmap_ready) h->variant = LBM_FUSED_TMEM;
+    else if (!h->tmap_ready || stray || (shifted(h->storage) && use < 0.9)) h->variant = LBM_FUSED_TMEM;
     else h->variant = h->storage == LBM_F32 ? LBM_FUSED_WS_TMA : LBM_FUSED_TM_TMA;
     h->geof.chunk = best_chunk(h->geof, 8, h->sms, h->variant == LBM_FUSED_WS_TMA ? 1 : 2);
 }
@@ -336,11 +359,19 @@ int ensure_memory(lbm_ctx *h)
     h->partial = reinterpret_cast<double *>(b + L.partial);
     h->sums = reinterpret_cast<double *>(b + L.sums);
     h->status = reinterpret_cast<int *>(b + L.status);
-    CU(h, cudaMemcpyAsync(h->mask, h->mask_host.data(), h->geo.N, cudaMemcpyHostToDevice, h->stream));
+    // the mask with the rows' padding, if any, marked solid
+    std::vector<uint8_t> padded;
+    if (h->geo.px != h->geo.nx) {
+        padded.assign(h->geo.N, 1);
+        for (size_t r = 0; r < (size_t)h->geo.ny * h->geo.nz; ++r)
+            memcpy(&padded[r * h->geo.px], &h->mask_host[r * h->geo.nx], h->geo.nx);
+    }
+    CU(h, cudaMemcpyAsync(h->mask, padded.empty() ? h->mask_host.data() : padded.data(), h->geo.N,
+                          cudaMemcpyHostToDevice, h->stream));
     {   // planes of the fused step's march axis (z; the 2D y axis for D2Q9) that hold a solid
         const size_t plane = (size_t)h->geof.nx * h->geof.ny;
         h->zsolid_host.assign(h->geof.nz, 0);
-        for (size_t n = 0; n < h->geo.N; ++n)
+        for (size_t n = 0; n < h->geo.M; ++n)
             if (h->mask_host[n]) h->zsolid_host[n / plane] = 1;
         CU(h, cudaMemcpyAsync(const_cast<uint8_t *>(h->geof.zsolid), h->zsolid_host.data(), h->geof.nz,
                               cudaMemcpyHostToDevice, h->stream));
@@ -356,23 +387,18 @@ int ensure_memory(lbm_ctx *h)
 
 bool has_solid(const lbm_ctx *h) { return h->any_solid; }
 
-// Row alignment the TMA-staged form needs: nx a multiple of 4 (FP32) or 8
-// (16-bit shifted storage), so that rows start on 16 bytes.
-int tma_nx_multiple(int storage) { return storage == LBM_F32 ? 4 : shifted(storage) ? 8 : 0; }
-
 // The two population buffers of a D3Q27 FP32 or shifted-storage handle as
 // 4D tensors (x, y, z, i) of the stored type, each with the five box shapes
 // of the TMA-staged forms (32 x 8, 32 x 2, W x 8, W x 2 and the one-copy
 // (32 + 2 W) x 12 nodes of one plane, all 27 populations; W = 16 bytes of
-// the type). Needs nx a multiple
-// of tma_nx_multiple (16-byte row strides) and the CUDA driver's tensor-map
+// the type). Needs rows that start on 16 bytes (row_pitch) and the CUDA driver's tensor-map
 // encoder, found through the runtime's entry-point query; leaves tmap_ready
 // false when either is missing.
 void make_tensor_maps(lbm_ctx *h)
 {
     h->tmap_ready = false;
     const int mult = tma_nx_multiple(h->storage);
-    if (h->lattice != LBM_D3Q27 || !mult || h->geo.nx % mult || !h->fv[0]) return;
+    if (h->lattice != LBM_D3Q27 || !mult || h->geo.px % mult || !h->fv[0]) return;
     using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
                                 CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
@@ -392,7 +418,7 @@ void make_tensor_maps(lbm_ctx *h)
                                                             : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const cuuint32_t w = (cuuint32_t)(16 / es);
     const cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz, 27};
-    const cuuint64_t strides[3] = {(cuuint64_t)g.nx * es, (cuuint64_t)g.nx * g.ny * es, (cuuint64_t)g.N * es};
+    const cuuint64_t strides[3] = {(cuuint64_t)g.px * es, (cuuint64_t)g.px * g.ny * es, (cuuint64_t)g.N * es};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     for (int k = 0; k < 2; ++k) {
         CUtensorMap *m[5] = {&h->tmaps[k].mc, &h->tmaps[k].tc, &h->tmaps[k].ml, &h->tmaps[k].tl,
@@ -775,20 +801,29 @@ int decode_to(lbm_ctx *h, int k, double *out)
 }
 
 template <int LAT>
-int encode_from(lbm_ctx *h, const double *f)
+int encode_from(lbm_ctx *h, const Geo &gf, const double *f)   // gf: the layout of f
 {
     const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->mask, f, h->rs[0], h->rs[1]);
+    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, gf, h->mask, f, h->rs[0], h->rs[1]);
     if (h->storage == LBM_F16S)
         lbmk::k_encode_shifted<LAT, __half><<<gr, bl, 0, h->stream>>>(
-            h->geo, f, h->rs[0], static_cast<__half *>(h->fv[0]));
+            h->geo, gf, f, h->rs[0], static_cast<__half *>(h->fv[0]));
     else
         lbmk::k_encode_shifted<LAT, __nv_bfloat16><<<gr, bl, 0, h->stream>>>(
-            h->geo, f, h->rs[0], static_cast<__nv_bfloat16 *>(h->fv[0]));
+            h->geo, gf, f, h->rs[0], static_cast<__nv_bfloat16 *>(h->fv[0]));
     CU(h, cudaGetLastError());
     h->launches += 2;
     h->cur = 0;
     return LBM_OK;
+}
+
+// Every node's populations from layout ga and type A to gb and B.
+template <typename A, typename B>
+void convert_pops(lbm_ctx *h, const Geo &ga, const Geo &gb, const A *in, B *out)
+{
+    const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
+    if (h->lattice == LBM_D2Q9) lbmk::k_convert<0><<<gr, bl, 0, h->stream>>>(ga, gb, in, out);
+    else                        lbmk::k_convert<1><<<gr, bl, 0, h->stream>>>(ga, gb, in, out);
 }
 
 int temp_alloc(lbm_ctx *h, TempF64 &t)
@@ -916,7 +951,7 @@ int launch_init(lbm_ctx *h, const double *rho0, const double *u0)
         int rc = temp_alloc(h, t);
         if (rc) return rc;
         launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT>{h->mask, h->rp, u0, t.p});
-        rc = encode_from<LAT>(h, t.p);
+        rc = encode_from<LAT>(h, h->geo, t.p);
         if (rc) return rc;
         CU(h, cudaGetLastError());
         CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
@@ -1018,7 +1053,8 @@ size_t lbm_required_bytes(int lattice, int nx, int ny, int nz, int storage)
 {
     if (!valid_shape(lattice, nx, ny, nz) || storage < LBM_F64 || storage > LBM_BF16S) return 0;
     const int D = lattice == LBM_D2Q9 ? 2 : 3, Q = lattice == LBM_D2Q9 ? 9 : 27;
-    return layout_for(D, Q, (size_t)nx * ny * nz, storage, lattice == LBM_D2Q9 ? ny : nz).total;
+    return layout_for(D, Q, (size_t)row_pitch(lattice, nx, ny, nz, storage) * ny * nz, storage,
+                      lattice == LBM_D2Q9 ? ny : nz).total;
 }
 
 int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, double t_over_tc,
@@ -1045,7 +1081,9 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
     h->D = lattice == LBM_D2Q9 ? 2 : 3;
     h->Q = lattice == LBM_D2Q9 ? 9 : 27;
     h->geo.nx = nx; h->geo.ny = ny; h->geo.nz = nz;
-    h->geo.N = (unsigned)((size_t)nx * ny * nz);
+    h->geo.M = (unsigned)((size_t)nx * ny * nz);
+    h->geo.px = row_pitch(lattice, nx, ny, nz, prm.storage);
+    h->geo.N = (unsigned)((size_t)h->geo.px * ny * nz);
     h->storage = prm.storage;
     h->flags = prm.flags;
     h->t_over_tc = t_over_tc;
@@ -1075,6 +1113,7 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
     h->geof.ny = lattice == LBM_D2Q9 ? 1 : ny;
     h->geof.nz = lattice == LBM_D2Q9 ? ny : nz;
     h->geof.N = h->geo.N;
+    h->geof.px = h->geo.px;
     h->geof.chunk = lattice == LBM_D2Q9 ? 64 : kDefaultChunk3;
     PhysF &pf = h->physf;
     pf.eos = eos;
@@ -1130,9 +1169,9 @@ int lbm_create(lbm_handle *out, int lattice, int nx, int ny, int nz, int eos, do
         pf.spsi_w = d;
         if (h->e64) pf.spsi_w = (float)excess_pressure_host(eos, ph.a, ph.b, ph.RT, ph.a * ph.alpha, prm.rho_w);
     }
-    h->mask_host.assign(h->geo.N, 0);
+    h->mask_host.assign(h->geo.M, 0);
     if (solid_mask)
-        for (size_t n = 0; n < h->geo.N; ++n) {
+        for (size_t n = 0; n < h->geo.M; ++n) {
             h->mask_host[n] = solid_mask[n] ? 1 : 0;
             h->any_solid = h->any_solid || solid_mask[n];
         }
@@ -1175,7 +1214,7 @@ int lbm_init(lbm_handle h, const double *rho0, const double *u0, int on_device)
     if (!h || !rho0) return LBM_EINVAL;
     int rc = ensure_memory(h);
     if (rc) return rc;
-    const size_t N = h->geo.N;
+    const size_t N = h->geo.M;
     h->cur = 0;
     const double *r = rho0, *v = u0;
     if (!on_device) {
@@ -1229,7 +1268,7 @@ int lbm_moments(lbm_handle h, double *rho, double *u, double *U, int on_device)
 {
     int rc = check_ready(h);
     if (rc) return rc;
-    const size_t N = h->geo.N, D = h->D;
+    const size_t N = h->geo.M, D = h->D;
     double *dr = rho, *du = u, *dU = U;
     if (!on_device) {
         double *st = static_cast<double *>(h->fv[h->cur ^ 1]);  // dead between steps
@@ -1251,7 +1290,7 @@ int lbm_moments(lbm_handle h, double *rho, double *u, double *U, int on_device)
 int lbm_set_wall_distances(lbm_handle h, const double *q)
 {
     if (!h) return LBM_EINVAL;
-    const size_t N = h->geo.N;
+    const size_t N = h->geo.M;
     const int Q = h->Q, D = h->D;
     const Geo &g = h->geo;
     std::vector<unsigned> bn, bm;
@@ -1311,7 +1350,7 @@ int lbm_pressure_tensor(lbm_handle h, double *P, int on_device)
     int rc = check_ready(h);
     if (rc) return rc;
     if (!P) return fail(h, LBM_EINVAL, "null output");
-    const size_t N = h->geo.N, na = h->D == 3 ? 6 : 3;
+    const size_t N = h->geo.M, na = h->D == 3 ? 6 : 3;
     // the dead population buffer holds (1 + 2D) N >= na N doubles
     double *out = on_device ? P : static_cast<double *>(h->fv[h->cur ^ 1]);
     rc = h->lattice == LBM_D2Q9 ? launch_pressure<0>(h, out) : launch_pressure<1>(h, out);
@@ -1342,7 +1381,7 @@ int lbm_get_populations(lbm_handle h, double *f, int on_device)
     int rc = check_ready(h);
     if (rc) return rc;
     if (!f) return LBM_EINVAL;
-    const size_t N = h->geo.N, QN = (size_t)h->Q * N;
+    const size_t N = h->geo.M, QN = (size_t)h->Q * N;
     if (shifted(h->storage)) {
         TempF64 t;   // of a host buffer; an aligned device buffer is written in place
         const bool direct = on_device && reinterpret_cast<uintptr_t>(f) % sizeof(double) == 0;
@@ -1357,15 +1396,17 @@ int lbm_get_populations(lbm_handle h, double *f, int on_device)
         }
     } else if (h->storage == LBM_F32) {
         if (on_device) {
-            lbmk::k_convert<float, double><<<1024, 256, 0, h->stream>>>(QN, f32(h, h->cur), f);
+            convert_pops(h, h->geo, lbmk::flat(h->geo), f32(h, h->cur), f);
             CU(h, cudaGetLastError());
             h->launches += 1;
         } else {
-            std::vector<float> tmp(QN);
-            CU(h, cudaMemcpyAsync(tmp.data(), f32(h, h->cur), sizeof(float) * QN,
+            std::vector<float> tmp((size_t)h->Q * h->geo.N);
+            CU(h, cudaMemcpyAsync(tmp.data(), f32(h, h->cur), sizeof(float) * tmp.size(),
                                   cudaMemcpyDeviceToHost, h->stream));
             CU(h, cudaStreamSynchronize(h->stream));
-            for (size_t k = 0; k < QN; ++k) f[k] = tmp[k];
+            const size_t nx = h->geo.nx, px = h->geo.px;
+            for (size_t r = 0; r < QN / nx; ++r)   // rows, without their padding
+                for (size_t x = 0; x < nx; ++x) f[r * nx + x] = tmp[r * px + x];
         }
     } else {
         CU(h, cudaMemcpyAsync(f, f64(h, h->cur), sizeof(double) * QN,
@@ -1385,7 +1426,7 @@ int lbm_set_populations(lbm_handle h, const double *f, int on_device)
     if (!h || !f) return LBM_EINVAL;
     int rc = ensure_memory(h);
     if (rc) return rc;
-    const size_t QN = (size_t)h->Q * h->geo.N;
+    const size_t QN = (size_t)h->Q * h->geo.M;
     h->cur = 0;
     if (shifted(h->storage)) {
         TempF64 t;   // of a host buffer; an aligned device buffer is read in place
@@ -1396,18 +1437,21 @@ int lbm_set_populations(lbm_handle h, const double *f, int on_device)
                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
         }
         const double *in = direct ? f : t.p;
-        rc = h->lattice == LBM_D2Q9 ? encode_from<0>(h, in) : encode_from<1>(h, in);
+        const Geo gu = lbmk::flat(h->geo);
+        rc = h->lattice == LBM_D2Q9 ? encode_from<0>(h, gu, in) : encode_from<1>(h, gu, in);
         if (rc) return rc;
         if (!direct) CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
     } else if (h->storage == LBM_F32) {
         if (on_device) {
-            lbmk::k_convert<double, float><<<1024, 256, 0, h->stream>>>(QN, f, f32(h, 0));
+            convert_pops(h, lbmk::flat(h->geo), h->geo, f, f32(h, 0));
             CU(h, cudaGetLastError());
             h->launches += 1;
         } else {
-            std::vector<float> tmp(QN);
-            for (size_t k = 0; k < QN; ++k) tmp[k] = (float)f[k];
-            CU(h, cudaMemcpyAsync(f32(h, 0), tmp.data(), sizeof(float) * QN,
+            std::vector<float> tmp((size_t)h->Q * h->geo.N);
+            const size_t nx = h->geo.nx, px = h->geo.px;
+            for (size_t r = 0; r < QN / nx; ++r)
+                for (size_t x = 0; x < nx; ++x) tmp[r * px + x] = (float)f[r * nx + x];
+            CU(h, cudaMemcpyAsync(f32(h, 0), tmp.data(), sizeof(float) * tmp.size(),
                                   cudaMemcpyHostToDevice, h->stream));
             CU(h, cudaStreamSynchronize(h->stream));
         }

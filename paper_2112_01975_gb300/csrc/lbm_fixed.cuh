@@ -121,7 +121,7 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const Shifted<ST> &f, u
     for (int i = 0; i < Q; ++i) h[i] = lbmf::to_f(f.h[(size_t)i * g.N + n]);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const unsigned src = X[cxi(i) + 1] + g.nx * (Y[cyi(i) + 1] + g.ny * Z[D == 3 ? czi(i) + 1 : 1]);
+        const unsigned src = entry(g, X[cxi(i) + 1], Y[cyi(i) + 1], Z[D == 3 ? czi(i) + 1 : 1]);
         s[i] = __float_as_uint(f.rho_src[src]);
     }
     const unsigned own = s[Q / 2];

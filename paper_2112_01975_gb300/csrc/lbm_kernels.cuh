@@ -13,10 +13,28 @@
 
 namespace lbmk {
 
+// A lattice of M = nx ny nz nodes. The library's own fields have rows of px >=
+// nx entries (px = nx except in D3Q27 reduced storage, whose rows start on 16
+// bytes): node (x, y, z) is entry x + px (y + ny z) of a field of N = px ny nz
+// entries. The caller's fields have no padding: see flat().
 struct Geo {
     int nx, ny, nz;
     unsigned N;
+    int px;
+    unsigned M;
 };
+
+__host__ __device__ __forceinline__ Geo flat(Geo g)
+{
+    g.px = g.nx;
+    g.N = g.M;
+    return g;
+}
+
+__device__ __forceinline__ unsigned entry(const Geo &g, int x, int y, int z)
+{
+    return (unsigned)x + (unsigned)g.px * ((unsigned)y + (unsigned)g.ny * (unsigned)z);
+}
 
 struct Phys {
     int eos;
@@ -146,7 +164,7 @@ __device__ __forceinline__ unsigned source_node(const Geo &g, int D, int i, int 
 {
     const int sx = (x - cxi(i) + g.nx) % g.nx, sy = (y - cyi(i) + g.ny) % g.ny;
     const int sz = D == 3 ? (z - czi(i) + g.nz) % g.nz : 0;
-    return sx + g.nx * (sy + g.ny * sz);
+    return entry(g, sx, sy, sz);
 }
 
 }  // namespace lbmk
@@ -229,7 +247,7 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
     const int x = blockIdx.x * SWX + tx, y = blockIdx.y * SWY + ty;
     const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, g.nz);
     const bool inside = x < g.nx && y < g.ny;
-    const unsigned plane = (unsigned)g.nx * (unsigned)g.ny;
+    const unsigned plane = (unsigned)g.px * (unsigned)g.ny;
     // this thread's one or two halo nodes
     const bool two = tid + NT < NH;
     int hr[2], hc[2];
@@ -240,7 +258,7 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
         hr[k] = h / HX;
         hc[k] = h - hr[k] * HX;
         off[k] = (unsigned)wrap_any((int)blockIdx.x * SWX - 2 + hc[k], g.nx) +
-                 (unsigned)g.nx * (unsigned)wrap_any((int)blockIdx.y * SWY - 2 + hr[k], g.ny);
+                 (unsigned)g.px * (unsigned)wrap_any((int)blockIdx.y * SWY - 2 + hr[k], g.ny);
     }
     int zq = z0 - 2 < 0 ? z0 - 2 + g.nz : z0 - 2;
     double2 v0 = rp[off[0] + plane * (unsigned)zq], v1 = two ? rp[off[1] + plane * (unsigned)zq] : v0;
@@ -296,8 +314,7 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
             }
         }
         if (q - 2 >= z0 && inside)
-            body(g, p, (unsigned)x + (unsigned)g.nx * (unsigned)y + plane * (unsigned)(q - 2), x, y, q - 2,
-                 done[0], done[1]);
+            body(g, p, entry(g, x, y, q - 2), x, y, q - 2, done[0], done[1]);
     }
 }
 
@@ -318,7 +335,7 @@ k_force_sweep2(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
     for (int h = tid; h < NH; h += NT) {
         const int r = h / HX, c = h - r * HX;
         const double2 v = rp[(unsigned)wrap_any(x0 - 2 + c, g.nx) +
-                             (unsigned)g.nx * (unsigned)wrap_any(y0 - 2 + r, g.ny)];
+                             (unsigned)g.px * (unsigned)wrap_any(y0 - 2 + r, g.ny)];
         sm.raw[0][r][c] = fabs(v.y);
         sm.raw[1][r][c] = v.x;
     }
@@ -341,7 +358,7 @@ k_force_sweep2(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
         sum[k][0] = fma(r2, X[1][0], X[0][0]);
         sum[k][1] = fma(r2, X[1][1], X[0][1]);
     }
-    body(g, p, (unsigned)x + (unsigned)g.nx * (unsigned)y, x, y, 0, sum[0], sum[1]);
+    body(g, p, entry(g, x, y, 0), x, y, 0, sum[0], sum[1]);
 }
 
 // Moments, EOS and pseudo-potential of every fluid node; flags bad densities.
@@ -355,7 +372,7 @@ __global__ void k_macro(Geo g, Phys p, const uint8_t *__restrict__ mask, P f, do
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z);
     if (mask[n]) return;
     double rho, j[3];
     node_sums<LAT, false>(g, f, n, x, y, z, rho, j);
@@ -401,7 +418,7 @@ struct CollideBody {
         const int Y[3] = {wrapm(y - 1, g.ny), y, wrapp(y + 1, g.ny)};
         const int Z[3] = {D == 3 ? wrapm(z - 1, g.nz) : 0, z, D == 3 ? wrapp(z + 1, g.nz) : 0};
         const auto at = [&](int cx, int cy, int cz) {
-            return X[cx + 1] + g.nx * (Y[cy + 1] + g.ny * Z[cz + 1]);
+            return entry(g, X[cx + 1], Y[cy + 1], Z[cz + 1]);
         };
         // Product-form factors: equilibrium (xi = u, zeta = 1/3 + u^2) and
         // extended (xi* = u + F/rho, zeta* = 1/3 + xi*^2 + Phi/rho), as
@@ -464,12 +481,13 @@ __global__ void k_moments_out(Geo g, Phys p, const uint8_t *__restrict__ mask,
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z);
+    const unsigned m = entry(flat(g), x, y, z);
     const bool solid = mask[n];
-    if (rho_out) rho_out[n] = solid ? p.rho_w : rp[n].x;
+    if (rho_out) rho_out[m] = solid ? p.rho_w : rp[n].x;
 #pragma unroll
     for (int a = 0; a < D; ++a)
-        if (u_out) u_out[a * (size_t)g.N + n] = solid ? 0.0 : u[a * (size_t)g.N + n];
+        if (u_out) u_out[a * (size_t)g.M + m] = solid ? 0.0 : u[a * (size_t)g.N + n];
 }
 
 // The same with U: the body of the force sweep.
@@ -480,21 +498,22 @@ struct MomentsBody {
     const double *u;
     double *rho_out, *u_out, *U_out;
 
-    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int, int, int,
+    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int x, int y, int z,
                                                const double *sp, const double *sr) const
     {
         constexpr int D = Lattice<LAT>::D;
+        const unsigned m = entry(flat(g), x, y, z);
         const bool solid = mask[n];
         const double2 c = solid ? make_double2(p.rho_w, 0.0) : rp[n];
         double F[3];
         force_of_sums<LAT>(p, c.x, c.y, sp, sr, F);
         const double half = 0.5 / c.x;
-        if (rho_out) rho_out[n] = c.x;
+        if (rho_out) rho_out[m] = c.x;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             const double ua = solid ? 0.0 : u[a * (size_t)g.N + n];
-            if (u_out) u_out[a * (size_t)g.N + n] = ua;
-            U_out[a * (size_t)g.N + n] = solid ? 0.0 : fma(F[a], half, ua);
+            if (u_out) u_out[a * (size_t)g.M + m] = ua;
+            U_out[a * (size_t)g.M + m] = solid ? 0.0 : fma(F[a], half, ua);
         }
     }
 };
@@ -517,8 +536,9 @@ __global__ void k_interp_bounce_back(Geo g, const unsigned *__restrict__ bn,
     constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
-    const unsigned n = bn[b], m = bmask[b];
-    const int x = n % g.nx, y = (n / g.nx) % g.ny, z = n / (g.nx * g.ny);
+    const unsigned id = bn[b], m = bmask[b];   // id: without row padding
+    const int x = id % g.nx, y = (id / g.nx) % g.ny, z = id / (g.nx * g.ny);
+    const unsigned n = entry(g, x, y, z);
     T excess = T(0);
     for (int i = 0; i < Q; ++i) {
         if (!((m >> i) & 1u)) continue;
@@ -531,7 +551,7 @@ __global__ void k_interp_bounce_back(Geo g, const unsigned *__restrict__ bn,
         } else {
             const int xm = (x - cxi(i) + g.nx) % g.nx, ym = (y - cyi(i) + g.ny) % g.ny;
             const int zm = D == 3 ? (z - czi(i) + g.nz) % g.nz : 0;
-            const unsigned nm = xm + g.nx * (ym + g.ny * zm);
+            const unsigned nm = entry(g, xm, ym, zm);
             v = a / (T(2) * q) + (T(2) * q - T(1)) / (T(2) * q) * f[(size_t)ib * g.N + nm];
         }
         f[(size_t)ib * g.N + n] = v;
@@ -562,12 +582,12 @@ __global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mas
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z), m = entry(flat(g), x, y, z);
     constexpr int CA[6] = {0, 1, D == 3 ? 2 : 0, 0, 0, 1};
     constexpr int CB[6] = {0, 1, D == 3 ? 2 : 1, 1, 2, 2};
     if (mask[n]) {
 #pragma unroll
-        for (int k = 0; k < NA; ++k) out[(size_t)k * g.N + n] = 0.0;
+        for (int k = 0; k < NA; ++k) out[(size_t)k * g.M + m] = 0.0;
         return;
     }
     double rho, j[3], kin[6];
@@ -591,7 +611,7 @@ __global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mas
     for (int i = Q / 2 + 1; i < Q; ++i) {
         const int c[3] = {cxi(i), cyi(i), D == 3 ? czi(i) : 0};
         const auto at = [&](int k) {
-            return rp[X[k * c[0] + 2] + g.nx * (Y[k * c[1] + 2] + g.ny * Z[k * c[2] + 2])];
+            return rp[entry(g, X[k * c[0] + 2], Y[k * c[1] + 2], Z[k * c[2] + 2])];
         };
         const double2 p1 = at(1), m1 = at(-1), p2 = at(2), m2 = at(-2);
         double T = c1 * (fabs(p1.y) + fabs(m1.y));
@@ -617,7 +637,7 @@ __global__ void k_pressure_tensor(Geo g, Phys p, const uint8_t *__restrict__ mas
 #pragma unroll
         for (int cls = 0; cls < D; ++cls)
             if (set[k][cls]) v = fma(w[cls], acc[k][cls], v);
-        out[(size_t)k * g.N + n] = v;
+        out[(size_t)k * g.M + m] = v;
     }
 }
 
@@ -630,9 +650,9 @@ __global__ void k_init_density(Geo g, Phys p, const uint8_t *__restrict__ mask,
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z);
     if (mask[n]) return;
-    const double rho = rho0[n];
+    const double rho = rho0[entry(flat(g), x, y, z)];
     rp[n] = make_double2(rho, signed_psi(p, rho));
 }
 
@@ -648,7 +668,7 @@ struct InitBody {
     const double *u0;
     T *f;
 
-    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int, int, int,
+    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int x, int y, int z,
                                                const double *sp, const double *sr) const
     {
         constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
@@ -657,6 +677,7 @@ struct InitBody {
             for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + n] = (T)0;
             return;
         }
+        const unsigned m = entry(flat(g), x, y, z);
         const double2 c = rp[n];
         const double rho = c.x, half = 0.5 / rho;
         double F[3];
@@ -664,7 +685,7 @@ struct InitBody {
         double E[3][3];
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            const double ua = fma(-F[a], half, u0 ? u0[a * (size_t)g.N + n] : 0.0);
+            const double ua = fma(-F[a], half, u0 ? u0[a * (size_t)g.M + m] : 0.0);
             const double t = 0.5 * ua, h = fma(t, ua, 1.0 / 6.0);
             E[a][0] = h - t;
             E[a][1] = fma(-2.0, h, 1.0);
@@ -688,7 +709,7 @@ __global__ void k_fill_solid(Geo g, Phys p, const uint8_t *__restrict__ mask,
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z);
     if (!mask[n]) return;
     rp[n] = make_double2(p.rho_w, signed_psi(p, p.rho_w));
 #pragma unroll
@@ -713,11 +734,11 @@ k_reduce_partial(Geo g, const uint8_t *__restrict__ mask, P f, double *__restric
 {
     constexpr int D = Lattice<LAT>::D;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    const unsigned plane = (unsigned)g.nx * (unsigned)g.ny;
+    const unsigned plane = (unsigned)g.px * (unsigned)g.ny;
     for (unsigned n = blockIdx.x * RED_THREADS + threadIdx.x; n < g.N;
          n += RED_THREADS * RED_BLOCKS) {
-        if (mask[n]) continue;
-        const unsigned z = n / plane, y = (n - z * plane) / g.nx, x = n - z * plane - y * g.nx;
+        if (mask[n]) continue;   // the rows' padding too: its mask is 1
+        const unsigned z = n / plane, y = (n - z * plane) / g.px, x = n - z * plane - y * g.px;
         double rho, j[3];
         node_sums<LAT, false>(g, f, n, x, y, z, rho, j);
         acc[0] += rho;
@@ -772,13 +793,13 @@ __global__ void k_decode_shifted(Geo g, const ST *__restrict__ h, const float *_
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z), m = entry(flat(g), x, y, z);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         // a solid source (density -1) means a population bounced by n itself
         float src = rho_src[source_node(g, D, i, x, y, z)];
         if (src < 0.0f) src = rho_src[n];
-        f[(size_t)i * g.N + n] = (weight_d(i, D) + widen(lbmf::to_f(h[(size_t)i * g.N + n]))) * widen(src);
+        f[(size_t)i * g.M + m] = (weight_d(i, D) + widen(lbmf::to_f(h[(size_t)i * g.N + n]))) * widen(src);
     }
 }
 
@@ -786,17 +807,19 @@ __global__ void k_decode_shifted(Geo g, const ST *__restrict__ h, const float *_
 // solid nodes stays for good): each fluid node's density, -1 at solid nodes
 // (their populations' sources are the fluid nodes that bounced them; see the
 // decoders).
+// gf: the layout of f (the caller's or the library's).
 template <int LAT>
-__global__ void k_density(Geo g, const uint8_t *__restrict__ mask, const double *__restrict__ f,
+__global__ void k_density(Geo g, Geo gf, const uint8_t *__restrict__ mask, const double *__restrict__ f,
                           float *__restrict__ rho0, float *__restrict__ rho1)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
-    const unsigned n = x + g.nx * (blockIdx.y + g.ny * blockIdx.z);
+    const int y = blockIdx.y, z = blockIdx.z;
+    const unsigned n = entry(g, x, y, z);
     float v = -1.0f;
     if (!mask[n]) {
         double s, j[3];
-        node_sums<LAT, false>(g, f, n, x, blockIdx.y, blockIdx.z, s, j);
+        node_sums<LAT, false>(gf, f, entry(gf, x, y, z), x, y, z, s, j);
         v = (float)s;
     }
     rho0[n] = rho1[n] = v;
@@ -812,14 +835,14 @@ __device__ __forceinline__ double reciprocal_of(float v)
 }
 
 template <int LAT, typename ST>
-__global__ void k_encode_shifted(Geo g, const double *__restrict__ f, const float *__restrict__ rho,
+__global__ void k_encode_shifted(Geo g, Geo gf, const double *__restrict__ f, const float *__restrict__ rho,
                                  ST *__restrict__ h)
 {
     constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned n = x + g.nx * (y + g.ny * z);
+    const unsigned n = entry(g, x, y, z), m = entry(gf, x, y, z);
     if (rho[n] < 0.0f) {   // solid: no populations
 #pragma unroll
         for (int i = 0; i < Q; ++i) h[(size_t)i * g.N + n] = lbmf::from_f<ST>(0.0f);
@@ -830,18 +853,25 @@ __global__ void k_encode_shifted(Geo g, const double *__restrict__ f, const floa
         float src = rho[source_node(g, D, i, x, y, z)];
         if (src < 0.0f) src = rho[n];   // bounced by n itself
         h[(size_t)i * g.N + n] =
-            lbmf::from_f<ST>((float)fma(f[(size_t)i * g.N + n], reciprocal_of(src), -weight_d(i, D)));
+            lbmf::from_f<ST>((float)fma(f[(size_t)i * gf.N + m], reciprocal_of(src), -weight_d(i, D)));
     }
 }
 
-// Element-wise type conversion (population I/O of FP32 storage).
-template <typename A, typename B>
-__global__ void k_convert(size_t n, const A *__restrict__ in, B *__restrict__ out)
+// Population I/O of FP32 storage: every node's populations from the layout of
+// ga and type A to that of gb and B.
+template <int LAT, typename A, typename B>
+__global__ void k_convert(Geo ga, Geo gb, const A *__restrict__ in, B *__restrict__ out)
 {
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
-         k += (size_t)gridDim.x * blockDim.x)
-        if constexpr (sizeof(A) == 4) out[k] = widen(in[k]);
-        else                          out[k] = (B)in[k];
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= ga.nx) return;
+    const int y = blockIdx.y, z = blockIdx.z;
+    const unsigned a = entry(ga, x, y, z), b = entry(gb, x, y, z);
+#pragma unroll
+    for (int i = 0; i < Lattice<LAT>::Q; ++i) {
+        const A v = in[(size_t)i * ga.N + a];
+        if constexpr (sizeof(A) == 4) out[(size_t)i * gb.N + b] = widen(v);
+        else                          out[(size_t)i * gb.N + b] = (B)v;
+    }
 }
 
 // FP64 throughput probe: eight independent fused multiply-add chains per

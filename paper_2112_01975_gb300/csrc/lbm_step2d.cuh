@@ -93,7 +93,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
         int r, c;
         halo2(live[u] ? k : 0, r, c);
         const int x = wrap_any(x0 - 2 + c, nx), y = wrap_any(y0 - 2 + r, ny);
-        const unsigned n = (unsigned)x + (unsigned)nx * (unsigned)y;
+        const unsigned n = (unsigned)x + (unsigned)g.px * (unsigned)y;
         solid[u] = MASK && live[u] && mask[n];
         if (!live[u] || solid[u]) continue;
         if constexpr (SHIFT) {
@@ -104,7 +104,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
             float src[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                src[i] = __ldg(rho_src + ((unsigned)X[L::cx(i) + 1] + (unsigned)nx * (unsigned)Y[L::cz(i) + 1]));
+                src[i] = __ldg(rho_src + ((unsigned)X[L::cx(i) + 1] + (unsigned)g.px * (unsigned)Y[L::cz(i) + 1]));
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const float own = MASK && src[i] < 0.0f ? src[Q / 2] : src[i];
@@ -144,7 +144,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
     __syncthreads();
     const int tx = tid & 31, ty = tid >> 5, x = x0 + tx, y = y0 + ty;
     if (x >= nx || y >= ny || solid[0]) return;
-    const unsigned n = (unsigned)x + (unsigned)nx * (unsigned)y;
+    const unsigned n = (unsigned)x + (unsigned)g.px * (unsigned)y;
     const float rho = own.rho, spsi = (own.d > 0.0f ? 1.0f : -1.0f) * psi0;
     if (!(rho > 0.0f) || !isfinite(rho)) atomicOr(status, 1);
     if constexpr (SHIFT) rho_dst[n] = rho;   // source density of what this node pushes
@@ -170,7 +170,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
         const float2 es = __fmul2_rn(A[L::cx(i) + 1][1], ES[2][L::cz(i) + 1]);   // (feq, f*)
         const float post = SHIFT ? fmaf(fmaf(omw, fi[0][i] - es.x, es.y), inv, -weight_f<0>(i))
                                  : fmaf(omw, fi[0][i] - es.x, es.y);
-        const unsigned dst = (unsigned)X[L::cx(i) + 1] + (unsigned)nx * (unsigned)Y[L::cz(i) + 1];
+        const unsigned dst = (unsigned)X[L::cx(i) + 1] + (unsigned)g.px * (unsigned)Y[L::cz(i) + 1];
         if (MASK && mask[dst]) fout[(Q - 1 - i) * N + n] = from_f<ST>(post);
         else                   fout[i * N + dst] = from_f<ST>(post);
     }
