@@ -381,8 +381,8 @@ int lbm_get_fused_variant(lbm_handle h, int *variant);
  * storage (LBM_F32, LBM_F16S or LBM_BF16S, not LBM_F64) and the same lattice
  * type, of any sizes and parameters; otherwise LBM_EINVAL. Each
  * lbm_batch_step launch gives every member one time step (the fused step of
- * that storage over all members' tiles: D3Q27 spread over a persistent grid
- * of two CTAs per SM, D2Q9 one CTA per tile); steps after the first replay a CUDA graph of two launches. Each
+ * that storage over all members' tiles, in the TMA-staged form for D3Q27;
+ * a step of more than 32 D3Q27 members takes a launch for each 32); steps after the first replay a CUDA graph of two launches. Each
  * member's result is bitwise the same as stepping it alone. While the batch
  * exists the members' work is ordered on the batch's stream (members must
  * not be stepped, initialised or written individually); lbm_batch_destroy
@@ -400,7 +400,7 @@ int lbm_batch_step(lbm_batch b, int64_t n);
  * (lbm_moments, lbm_reduce, lbm_get_populations). */
 int lbm_batch_sync(lbm_batch b);
 
-/* Launches issued by the batch (one per step). */
+/* Steps launched by the batch. */
 int64_t lbm_batch_launch_count(lbm_batch b);
 
 void lbm_batch_destroy(lbm_batch b);

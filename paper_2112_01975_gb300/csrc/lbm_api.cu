@@ -9,6 +9,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <thread>
 #include <vector>
@@ -362,7 +363,11 @@ int ensure_memory(lbm_ctx *h)
     // the mask with the rows' padding, if any, marked solid
     std::vector<uint8_t> padded;
     if (h->geo.px != h->geo.nx) {
-        padded.assign(h->geo.N, 1);
+        try {
+            padded.assign(h->geo.N, 1);
+        } catch (const std::bad_alloc &) {
+            return fail(h, LBM_ENOMEM, "no host memory for the padded mask");
+        }
         for (size_t r = 0; r < (size_t)h->geo.ny * h->geo.nz; ++r)
             memcpy(&padded[r * h->geo.px], &h->mask_host[r * h->geo.nx], h->geo.nx);
     }
@@ -1580,8 +1585,17 @@ struct lbm_batch_ctx {
     int lattice = 0, storage = LBM_F32;
     cudaStream_t stream = nullptr;
     lbmf::MemberF *d_members[2] = {nullptr, nullptr};   // step parity 0 and 1
-    lbmf::WorkItem *d_items = nullptr;
-    int n_items = 0, grid = 0, parity = 0;
+    lbmf::WorkItem *d_items = nullptr;   // of the launches below, one after the other
+    lbmf::BoxMaps *d_maps = nullptr;     // [member][buffer], TMA-staged launches
+    // a step: launches of up to kBatchMembers TMA-staged D3Q27 members, and
+    // one of all members that have no such form (or of all D2Q9 members)
+    struct Launch {
+        bool tma, solid;
+        int first, n_items, eos;
+        lbmf::BatchT args[2];   // TMA-staged: by step parity
+    };
+    std::vector<Launch> steps;
+    int grid = 0, parity = 0;   // blocks of the plain launch
     cudaGraphExec_t graph = nullptr;
     int64_t launches = 0;
 };
@@ -1589,40 +1603,93 @@ struct lbm_batch_ctx {
 namespace {
 
 template <typename ST>
-void launch_batch_shifted(lbm_batch_ctx *b, int parity, cudaStream_t s)
+void launch_batch_plain_shifted(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
     const int bytes = (int)sizeof(lbmf::SharedS<1>);
     smem_opt_in(lbmf::k_step_shifted_batch<1, ST>, bytes, done);
     lbmf::k_step_shifted_batch<1, ST><<<b->grid, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(
-        b->d_members[parity], b->d_items, b->n_items);
+        b->d_members[parity], items, n);
 }
 
-void launch_batch(lbm_batch_ctx *b, int parity, cudaStream_t s)
+void launch_batch_plain(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
 {
-    if (b->storage == LBM_F16S) launch_batch_shifted<__half>(b, parity, s);
-    else if (b->storage == LBM_BF16S) launch_batch_shifted<__nv_bfloat16>(b, parity, s);
+    if (b->storage == LBM_F16S) launch_batch_plain_shifted<__half>(b, items, n, parity, s);
+    else if (b->storage == LBM_BF16S) launch_batch_plain_shifted<__nv_bfloat16>(b, items, n, parity, s);
     else {
         static std::atomic<unsigned long long> done{0};   // devices already opted in
         const int bytes = (int)sizeof(lbmf::SharedF<1>);
         smem_opt_in(lbmf::k_step_f32_batch<1>, bytes, done);
         lbmf::k_step_f32_batch<1><<<b->grid, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(
-            b->d_members[parity], b->d_items, b->n_items);
+            b->d_members[parity], items, n);
     }
 }
 
 template <typename ST>
-void launch_batch_2d(lbm_batch_ctx *b, int parity, cudaStream_t s)
+void launch_batch_2d(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
 {
-    lbmf2::k_step2d_batch<ST><<<b->n_items, lbmf2::NT, 0, s>>>(b->d_members[parity], b->d_items);
+    lbmf2::k_step2d_batch<ST><<<n, lbmf2::NT, 0, s>>>(b->d_members[parity], items);
 }
 
+// One step of every member.
 void batch_launch(lbm_batch_ctx *b, int parity, cudaStream_t s)
 {
-    if (b->lattice != LBM_D2Q9) launch_batch(b, parity, s);
-    else if (b->storage == LBM_F32) launch_batch_2d<float>(b, parity, s);
-    else if (b->storage == LBM_F16S) launch_batch_2d<__half>(b, parity, s);
-    else launch_batch_2d<__nv_bfloat16>(b, parity, s);
+    for (const lbm_batch_ctx::Launch &l : b->steps) {
+        const lbmf::WorkItem *items = b->d_items + l.first;
+        if (l.tma) {
+            if (b->storage == LBM_F32) lbmtma::launch_batch(l.args[parity], items, l.n_items, l.eos, l.solid, s);
+            else if (b->storage == LBM_F16S)
+                lbmtma::launch_batch_shifted<__half>(l.args[parity], items, l.n_items, l.solid, s);
+            else
+                lbmtma::launch_batch_shifted<__nv_bfloat16>(l.args[parity], items, l.n_items, l.solid, s);
+        } else if (b->lattice != LBM_D2Q9) launch_batch_plain(b, items, l.n_items, parity, s);
+        else if (b->storage == LBM_F32) launch_batch_2d<float>(b, items, l.n_items, parity, s);
+        else if (b->storage == LBM_F16S) launch_batch_2d<__half>(b, items, l.n_items, parity, s);
+        else launch_batch_2d<__nv_bfloat16>(b, items, l.n_items, parity, s);
+    }
+}
+
+// Chunks of the members (by number) of one TMA-staged launch, and its items,
+// longest first: members' march axes in equal parts of at most `cap` planes,
+// with the cap that ends first when each free slot (SM, or half of one) takes
+// the next item.
+std::vector<lbmf::WorkItem> batch_items(const std::vector<lbm_ctx *> &members, const std::vector<int> &which,
+                                        int slots, std::vector<int> &chunks)
+{
+    std::vector<lbmf::WorkItem> best;
+    double best_cost = 1e300;
+    for (int cap : {1 << 30, 96, 64, 40, 24, 12}) {
+        struct Part { int k, chunk, len, bz; };
+        std::vector<Part> parts;
+        std::vector<int> ch;
+        for (size_t k = 0; k < which.size(); ++k) {
+            const int nz = members[which[k]]->geof.nz, n = (nz + cap - 1) / cap, c = (nz + n - 1) / n;
+            ch.push_back(c);
+            for (int bz = 0; bz * c < nz; ++bz) parts.push_back({(int)k, c, std::min(c, nz - bz * c), bz});
+        }
+        std::stable_sort(parts.begin(), parts.end(), [](const Part &a, const Part &b) { return a.len > b.len; });
+        std::vector<lbmf::WorkItem> items;
+        std::vector<double> busy(slots, 0.0);   // a heap: the slot that is free first on top
+        double cost = 0.0;
+        for (const Part &q : parts) {
+            const GeoF &g = members[which[q.k]]->geof;
+            const int tx = (g.nx + 31) / 32, ty = (g.ny + 7) / 8;
+            for (int by = 0; by < ty; ++by)
+                for (int bx = 0; bx < tx; ++bx) {
+                    items.push_back({q.k, bx, by, q.bz});
+                    std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+                    busy.back() += q.len + 4.5;
+                    cost = std::max(cost, busy.back());
+                    std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+                }
+        }
+        if (cost < best_cost) {
+            best_cost = cost;
+            best.swap(items);
+            chunks.swap(ch);
+        }
+    }
+    return best;
 }
 
 void batch_free(lbm_batch_ctx *b)
@@ -1631,20 +1698,16 @@ void batch_free(lbm_batch_ctx *b)
     if (b->graph) cudaGraphExecDestroy(b->graph);
     for (auto *m : b->d_members) if (m) cudaFree(m);
     if (b->d_items) cudaFree(b->d_items);
+    if (b->d_maps) cudaFree(b->d_maps);
     for (size_t k = 0; k < b->prev.size(); ++k) b->members[k]->stream = b->prev[k];
     if (b->stream) cudaStreamDestroy(b->stream);
     cudaGetLastError();
     delete b;
 }
 
-}  // namespace
-
-extern "C" {
-
-int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
+// b: the batch under construction, freed by the caller if this fails.
+int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
 {
-    if (!out || !members || count < 1) return LBM_EINVAL;
-    *out = nullptr;
     const int lattice = members[0] ? members[0]->lattice : -1;
     const int storage = members[0] ? members[0]->storage : -1;
     if (storage == LBM_F64) return LBM_EINVAL;
@@ -1657,8 +1720,7 @@ int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
         for (int j = 0; j < k; ++j)
             if (members[j] == h) return LBM_EINVAL;   // a lattice at most once
     }
-    lbm_batch_ctx *b = new (std::nothrow) lbm_batch_ctx();
-    if (!b) return LBM_ENOMEM;
+    b = new lbm_batch_ctx();
     b->lattice = lattice;
     b->storage = storage;
     b->members.assign(members, members + count);
@@ -1667,19 +1729,25 @@ int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
         b->prev.push_back(h->stream);
     }
     for (lbm_ctx *h : b->members) cudaStreamSynchronize(h->stream);
-    if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
-        batch_free(b);
-        return LBM_ECUDA;
-    }
+    if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) return LBM_ECUDA;
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, 1);
     std::vector<lbmf::MemberF> desc[2];
-    std::vector<lbmf::WorkItem> items;
+    std::vector<lbmf::WorkItem> items, plain;
+    std::vector<lbmf::BoxMaps> maps;
+    std::vector<int> staged;   // members with a TMA-staged form
     for (int k = 0; k < count; ++k) {
         lbm_ctx *h = b->members[k];
+        const bool tma = lattice == LBM_D3Q27 && h->tmap_ready;
+        if (tma) staged.push_back(k);
+        for (int par = 0; par < 2; ++par) maps.push_back(h->tmaps[par]);
         // D3Q27: 32 x 8 columns by z-chunks; D2Q9: 32 x 8 tiles of the (x, 2D y) plane
         const int tx = (h->geof.nx + 31) / 32;
         const int ty = ((lattice == LBM_D2Q9 ? h->geof.nz : h->geof.ny) + 7) / 8;
         GeoF geof = h->geof;
-        if (h->auto_form && lattice == LBM_D3Q27) geof.chunk = kDefaultChunk3;   // the batch runs the plain form
+        if (h->auto_form && lattice == LBM_D3Q27) geof.chunk = kDefaultChunk3;   // the plain form's
         const int tz = lattice == LBM_D2Q9 ? 1 : (geof.nz + geof.chunk - 1) / geof.chunk;
         for (int par = 0; par < 2; ++par) {
             lbmf::MemberF m;
@@ -1695,30 +1763,83 @@ int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
             m.tiles_y = ty;
             desc[par].push_back(m);
         }
-        for (int bz = 0; bz < tz; ++bz)
-            for (int by = 0; by < ty; ++by)
-                for (int bx = 0; bx < tx; ++bx) items.push_back({k, bx, by, bz});
+        if (!tma)
+            for (int bz = 0; bz < tz; ++bz)
+                for (int by = 0; by < ty; ++by)
+                    for (int bx = 0; bx < tx; ++bx) plain.push_back({k, bx, by, bz});
         h->stream = b->stream;   // members' later work is ordered after the batch
     }
-    b->n_items = (int)items.size();
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = std::min(b->n_items, 2 * std::max(sms, 1));
-    const size_t db = sizeof(lbmf::MemberF) * count, ib = sizeof(lbmf::WorkItem) * items.size();
+    const size_t db = sizeof(lbmf::MemberF) * count;
     if (cudaMalloc(&b->d_members[0], db) != cudaSuccess || cudaMalloc(&b->d_members[1], db) != cudaSuccess ||
-        cudaMalloc(&b->d_items, ib) != cudaSuccess) {
-        batch_free(b);
-        return LBM_ENOMEM;
+        (!staged.empty() && cudaMalloc(&b->d_maps, sizeof(lbmf::BoxMaps) * maps.size()) != cudaSuccess)) return LBM_ENOMEM;
+    for (size_t first = 0; first < staged.size(); first += lbmf::kBatchMembers) {
+        const std::vector<int> which(staged.begin() + first,
+                                     staged.begin() + std::min(staged.size(), first + lbmf::kBatchMembers));
+        std::vector<int> chunks;
+        const std::vector<lbmf::WorkItem> part =
+            batch_items(b->members, which, storage == LBM_F32 ? sms : 2 * sms, chunks);
+        lbm_batch_ctx::Launch l = {};
+        l.tma = true;
+        l.first = (int)items.size();
+        l.n_items = (int)part.size();
+        l.eos = b->members[which[0]]->physf.eos;
+        for (size_t k = 0; k < which.size(); ++k) {
+            const lbm_ctx *h = b->members[which[k]];
+            l.solid = l.solid || h->any_solid;
+            if (h->physf.eos != l.eos) l.eos = -1;
+            for (int par = 0; par < 2; ++par) {
+                lbmf::MemberT &m = l.args[par].m[k];
+                m.g = h->geof;
+                m.g.chunk = chunks[k];
+                m.p = h->physf;
+                m.mask = h->mask;
+                m.src = h->fv[h->cur ^ par];
+                m.dst = h->fv[h->cur ^ par ^ 1];
+                m.rho_src = h->rs[h->cur ^ par];
+                m.rho_dst = h->rs[h->cur ^ par ^ 1];
+                m.status = h->status;
+                m.maps = b->d_maps + 2 * which[k] + (h->cur ^ par);
+            }
+        }
+        items.insert(items.end(), part.begin(), part.end());
+        b->steps.push_back(l);
     }
+    if (!plain.empty()) {
+        lbm_batch_ctx::Launch l = {};
+        l.first = (int)items.size();
+        l.n_items = (int)plain.size();
+        b->grid = std::min(l.n_items, 2 * sms);
+        items.insert(items.end(), plain.begin(), plain.end());
+        b->steps.push_back(l);
+    }
+    const size_t ib = sizeof(lbmf::WorkItem) * items.size();
+    if (cudaMalloc(&b->d_items, ib) != cudaSuccess) return LBM_ENOMEM;
     if (cudaMemcpy(b->d_members[0], desc[0].data(), db, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_members[1], desc[1].data(), db, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_items, items.data(), ib, cudaMemcpyHostToDevice) != cudaSuccess) {
-        batch_free(b);
-        return LBM_ECUDA;
-    }
-    *out = b;
+        (b->d_maps && cudaMemcpy(b->d_maps, maps.data(), sizeof(lbmf::BoxMaps) * maps.size(),
+                                 cudaMemcpyHostToDevice) != cudaSuccess) ||
+        cudaMemcpy(b->d_items, items.data(), ib, cudaMemcpyHostToDevice) != cudaSuccess) return LBM_ECUDA;
     return LBM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int lbm_batch_create(lbm_batch *out, const lbm_handle *members, int count)
+{
+    if (!out || !members || count < 1) return LBM_EINVAL;
+    *out = nullptr;
+    lbm_batch_ctx *b = nullptr;
+    int rc;
+    try {
+        rc = batch_build(b, members, count);
+    } catch (const std::bad_alloc &) {
+        rc = LBM_ENOMEM;
+    }
+    if (rc == LBM_OK) *out = b;
+    else              batch_free(b);
+    return rc;
 }
 
 int lbm_batch_step(lbm_batch b, int64_t n)

@@ -7,6 +7,38 @@
 namespace lbmtma {
 namespace {
 
+// Opt a kernel in to its dynamic shared memory, once per device.
+template <typename Kern>
+void opt_in(Kern kernel, int bytes, std::atomic<unsigned long long> &done)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load() & bit) return;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    done.fetch_or(bit);
+}
+
+template <bool MASK, int EOSK>
+void launch_b(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
+    const int bytes = (int)sizeof(lbmf::SharedWT<1>);
+    opt_in(lbmf::k_step_f32_wstma_batch<MASK, EOSK>, bytes, done);
+    lbmf::k_step_f32_wstma_batch<MASK, EOSK>
+        <<<n_items, 2 * lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(batch, items);
+}
+
+template <typename ST, bool MASK>
+void launch_bs(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
+    const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
+    opt_in(lbmf::k_step_shifted_tmtma_batch<ST, MASK>, bytes, done);
+    lbmf::k_step_shifted_tmtma_batch<ST, MASK>
+        <<<n_items, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(batch, items);
+}
+
 template <bool MASK, int EOSK>
 void launch_k(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, const lbmf::BoxMaps &maps,
               const float *src, float *dst, int *status, cudaStream_t s)
@@ -14,14 +46,7 @@ void launch_k(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     using L = lbmf::LatF<1>;
     const int bytes = (int)sizeof(lbmf::SharedWT<1>);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (!(done.load() & bit)) {   // more than 48 KB of dynamic shared memory
-        cudaFuncSetAttribute(lbmf::k_step_f32_wstma<1, MASK, EOSK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
-        done.fetch_or(bit);
-    }
+    opt_in(lbmf::k_step_f32_wstma<1, MASK, EOSK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
     lbmf::k_step_f32_wstma<1, MASK, EOSK><<<grid, 2 * L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
                                                                                  status);
@@ -48,14 +73,7 @@ void launch_s(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     using L = lbmf::LatF<1>;
     const int bytes = (int)sizeof(lbmf::SharedSWT<1, ST>);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (!(done.load() & bit)) {
-        cudaFuncSetAttribute(lbmf::k_step_shifted_wstma<1, ST, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
-        done.fetch_or(bit);
-    }
+    opt_in(lbmf::k_step_shifted_wstma<1, ST, MASK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
     lbmf::k_step_shifted_wstma<1, ST, MASK><<<grid, 2 * L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
                                                                                    rho_src, rho_dst, status);
@@ -68,14 +86,7 @@ void launch_t(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     using L = lbmf::LatF<1>;
     const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (!(done.load() & bit)) {
-        cudaFuncSetAttribute(lbmf::k_step_shifted_tmtma<1, ST, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
-        done.fetch_or(bit);
-    }
+    opt_in(lbmf::k_step_shifted_tmtma<1, ST, MASK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
     lbmf::k_step_shifted_tmtma<1, ST, MASK><<<grid, L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
                                                                               rho_src, rho_dst, status);
@@ -121,5 +132,28 @@ void launch(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, cons
     if (solid) launch_m<true>(g, p, mask, maps, src, dst, status, s);
     else       launch_m<false>(g, p, mask, maps, src, dst, status, s);
 }
+
+// The sweep's equations of state fixed at compile time (van der Waals, its
+// only one, and Peng-Robinson), the others and mixtures at run time.
+void launch_batch(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, int eos, bool solid,
+                  cudaStream_t s)
+{
+    if (solid) launch_b<true, -1>(batch, items, n_items, s);
+    else if (eos == 0) launch_b<false, 0>(batch, items, n_items, s);
+    else if (eos == 1) launch_b<false, 1>(batch, items, n_items, s);
+    else launch_b<false, -1>(batch, items, n_items, s);
+}
+
+template <typename ST>
+void launch_batch_shifted(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, bool solid,
+                          cudaStream_t s)
+{
+    if (solid) launch_bs<ST, true>(batch, items, n_items, s);
+    else       launch_bs<ST, false>(batch, items, n_items, s);
+}
+
+template void launch_batch_shifted<__half>(const lbmf::BatchT &, const lbmf::WorkItem *, int, bool, cudaStream_t);
+template void launch_batch_shifted<__nv_bfloat16>(const lbmf::BatchT &, const lbmf::WorkItem *, int, bool,
+                                                  cudaStream_t);
 
 }  // namespace lbmtma

@@ -34,4 +34,12 @@ void launch_shifted_tm(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t 
                        const ST *src, ST *dst, const float *rho_src, float *rho_dst, int *status, bool solid,
                        cudaStream_t s);
 
+// One step of the n_items items over the members of a batch (`solid`: one of
+// them has solid nodes; eos: that of all of them, or -1).
+void launch_batch(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, int eos, bool solid,
+                  cudaStream_t s);
+template <typename ST>
+void launch_batch_shifted(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, bool solid,
+                          cudaStream_t s);
+
 }  // namespace lbmtma
