@@ -43,7 +43,7 @@ struct lbm_ctx {
     std::vector<uint8_t> mask_host, zsolid_host;
     bool any_solid = false;
     int sms = 148;         // SMs of the device
-    int sweep_chunk = 16;  // planes per block of the D3Q27 force sweep (FP64 kernels)
+    int sweep_chunk = 16;  // planes per block of the D3Q27 force sweep (FP64 kernels); 0: direct sums
     int device;
     cudaStream_t own_stream = nullptr, stream = nullptr, cap_stream = nullptr;
     // device memory
@@ -58,7 +58,8 @@ struct lbm_ctx {
     int *status = nullptr;
     int cur = 0;
     bool initialised = false, bad = false;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr;        // two steps
+    cudaGraphExec_t graph_long = nullptr;   // kLongSteps steps
     int64_t launches = 0;
     // status polling of long lbm_step calls: a pinned copy of the status word
     // and the event that marks its arrival
@@ -78,6 +79,14 @@ struct lbm_ctx {
 };
 
 namespace {
+
+// Forget the captured steps (the form, chunk or kernels of a step change).
+void drop_graphs(lbm_ctx *h)
+{
+    if (h->graph) cudaGraphExecDestroy(h->graph);
+    if (h->graph_long) cudaGraphExecDestroy(h->graph_long);
+    h->graph = h->graph_long = nullptr;
+}
 
 // Opt a kernel in to more than 48 KB of dynamic shared memory, once per
 // device (the attribute belongs to the device the call runs on).
@@ -324,10 +333,7 @@ void leave_auto_form(lbm_ctx *h)
     if (h->lattice != LBM_D3Q27 || h->storage == LBM_F64) return;
     h->variant = LBM_FUSED_PLAIN;
     h->geof.chunk = kDefaultChunk3;
-    if (h->graph) {   // the captured graph holds the chosen form
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    drop_graphs(h);  // the captured graph holds the chosen form
 }
 
 int ensure_memory(lbm_ctx *h)
@@ -441,6 +447,14 @@ void make_tensor_maps(lbm_ctx *h)
     h->tmap_ready = true;
 }
 
+// Whether the two kernels of the FP64 step overlap at their ends: D2Q9
+// lattices of so few 32 x 2 tiles that both kernels' blocks have an SM each.
+bool overlap64(const lbm_ctx *h)
+{
+    const Geo &g = h->geo;
+    return h->lattice == LBM_D2Q9 && 2ll * ((g.nx + 31) / 32) * ((g.ny + 1) / 2) <= h->sms;
+}
+
 // The force sweep over the lattice (lbm_kernels.cuh) with the given body.
 template <int LAT, typename Body>
 void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
@@ -449,18 +463,29 @@ void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
     const int tx = (g.nx + lbmk::SWX - 1) / lbmk::SWX;
     if constexpr (LAT == 1) {
         const int chunk = h->sweep_chunk;
+        if (chunk == 0) {
+            lbmpdl::launch_step(false, lbmk::k_force_direct3<Body>, node_grid(g), node_block(g), 0, s, g, h->phys,
+                                h->rp, body);
+            return;
+        }
         const dim3 grid(tx, (g.ny + lbmk::SWY - 1) / lbmk::SWY, (g.nz + chunk - 1) / chunk);
-        lbmk::k_force_sweep3<<<grid, lbmk::SWX * lbmk::SWY, 0, s>>>(g, h->phys, h->rp, chunk, body);
+        lbmpdl::launch_step(false, lbmk::k_force_sweep3<Body>, grid, lbmk::SWX * lbmk::SWY, 0, s, g, h->phys, h->rp, chunk,
+                            body);
     } else if (tx * ((g.ny + 7) / 8) < h->sms) {
-        lbmk::k_force_sweep2<2, 4><<<dim3(tx, (g.ny + 1) / 2), 128, 0, s>>>(g, h->phys, h->rp, body);
+        lbmpdl::launch_step(overlap64(h), lbmk::k_force_sweep2<2, 4, Body>, dim3(tx, (g.ny + 1) / 2), 128, 0, s, g, h->phys, h->rp,
+                            body);
     } else {
-        lbmk::k_force_sweep2<8, 8><<<dim3(tx, (g.ny + 7) / 8), 256, 0, s>>>(g, h->phys, h->rp, body);
+        lbmpdl::launch_step(false, lbmk::k_force_sweep2<8, 8, Body>, dim3(tx, (g.ny + 7) / 8), 256, 0, s, g, h->phys, h->rp,
+                            body);
     }
 }
 
-// Planes per block of the D3Q27 force sweep: its blocks share each SM's FP64
-// pipe, so the SM with the most blocks sets the time; a block of c planes
-// also sums 4 more (64 of about 200 operations per node).
+// Planes per block of the D3Q27 force sweep, or 0 for the direct sums of small
+// lattices: a block's 8 warps share their SM's FP64 pipe (19 cycles an
+// instruction), so the SM with the most blocks sets the time; a block of c
+// planes also sums 4 more (64 of about 200 operations per node). Directly it
+// is about 290 operations per node, but every SM has its share (32^3: 20 us
+// against 39 a step, 48^3 about equal).
 int sweep_chunk(const Geo &g, int sms)
 {
     const long long tiles = (long long)((g.nx + lbmk::SWX - 1) / lbmk::SWX) *
@@ -475,7 +500,9 @@ int sweep_chunk(const Geo &g, int sms)
             best = c;
         }
     }
-    return best;
+    const long long warps = (long long)g.ny * g.nz * ((g.nx + 31) / 32);
+    const double direct = std::max(19.0 * ((warps + sms - 1) / sms), 64.0) * 290.0;
+    return direct < 19.0 * 8.0 * cost ? 0 : best;
 }
 
 double *f64(lbm_ctx *h, int k) { return static_cast<double *>(h->fv[k]); }
@@ -580,9 +607,12 @@ void launch_2d_m(lbm_ctx *h, cudaStream_t s, int k)
 {
     const GeoF &g = h->geof;
     const dim3 grid((g.nx + lbmf2::TX - 1) / lbmf2::TX, (g.nz + lbmf2::TY - 1) / lbmf2::TY);
-    lbmf2::k_step2d<MASK, ST, E64><<<grid, lbmf2::NT, 0, s>>>(
-        g, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]), h->rs[k],
-        h->rs[k ^ 1], h->status);
+    // (five blocks per SM are resident: more of them leave a successor no room)
+    const long long blocks = (long long)grid.x * grid.y;
+    const bool overlap = lbmpdl::side_by_side(blocks, h->sms) || blocks > 5 * h->sms;
+    lbmpdl::launch_step(overlap, lbmf2::k_step2d<MASK, ST, E64>, grid, lbmf2::NT, 0, s, g, h->physf, h->mask,
+                        static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]), h->rs[k], h->rs[k ^ 1],
+                        h->status);
 }
 
 template <typename ST>
@@ -753,8 +783,8 @@ int launch_step(lbm_ctx *h, cudaStream_t s, int *nk)
         const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
         const double *src = f64(h, h->cur);
         double *dst = f64(h, h->cur ^ 1);
-        lbmk::k_macro<LAT><<<gr, bl, 0, s>>>(h->geo, h->phys, h->mask, src, h->rp, h->u,
-                                             h->gflux, h->status);
+        lbmpdl::launch_step(overlap64(h), lbmk::k_macro<LAT, const double *>, gr, bl, 0, s, h->geo, h->phys, h->mask, src, h->rp,
+                            h->u, h->gflux, h->status);
         launch_collide64<LAT>(h, s, src, dst);
         *nk = 2;
     }
@@ -842,18 +872,18 @@ int temp_alloc(lbm_ctx *h, TempF64 &t)
     return LBM_OK;
 }
 
-// Two steps (state buffer 0 -> 1 -> 0) captured once on the library's own
-// stream; replayed on the handle's stream.
-int ensure_graph(lbm_ctx *h)
+// An even number of steps (state buffer 0 -> 1 -> 0 ...) captured once on the
+// library's own stream; replayed on the handle's stream.
+int ensure_graph(lbm_ctx *h, cudaGraphExec_t &graph, int steps)
 {
-    if (h->graph) return LBM_OK;
+    if (graph) return LBM_OK;
     if (!h->cap_stream) CU(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
     CU(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     const int saved = h->cur;
-    int rc = step_plain(h, h->cap_stream);
-    if (rc == LBM_OK) rc = step_plain(h, h->cap_stream);
-    h->launches -= 2 * kernels_per_step(h);  // captured, not launched
+    int rc = LBM_OK;
+    for (int k = 0; k < steps && rc == LBM_OK; ++k) rc = step_plain(h, h->cap_stream);
+    h->launches -= steps * kernels_per_step(h);  // captured, not launched
     h->cur = saved;
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
     if (rc != LBM_OK) {
@@ -861,10 +891,10 @@ int ensure_graph(lbm_ctx *h)
         return rc;
     }
     if (e != cudaSuccess) return fail(h, LBM_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&h->graph, g, 0);
+    e = cudaGraphInstantiate(&graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        h->graph = nullptr;
+        graph = nullptr;
         return fail(h, LBM_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     }
     return LBM_OK;
@@ -994,12 +1024,18 @@ int launch_reduce(lbm_ctx *h)
     return LBM_OK;
 }
 
-// Status polling of long step sequences: every kPollReplays graph replays
-// (2 steps each) the status word is copied to pinned host memory behind an
+// Between two graph replays the GPU idles for 1 to 3 us, as long as a step of a
+// small lattice (64^2 FP32: 4.3 us a step with graphs of two steps, 2.9 with
+// 16, 2.8 with 32). Sequences of at least twice that on lattices whose step is
+// short (under about 50 us) replay graphs of kLongSteps steps.
+constexpr int kLongSteps = 16;
+constexpr unsigned kLongNodes = 1u << 20;
+
+// Status polling of long step sequences: every kPollSteps steps the status word is copied to pinned host memory behind an
 // event; before the next copy is queued the previous one is awaited, so the
 // host runs at most one polling interval ahead of the device and a diverged
 // lattice stops within two intervals.
-constexpr int64_t kPollReplays = 32;
+constexpr int64_t kPollSteps = 64;
 
 int ensure_poll(lbm_ctx *h)
 {
@@ -1253,16 +1289,22 @@ int lbm_step(lbm_handle h, int64_t n)
             if ((rc = step_plain(h, h->stream))) return rc;
             --n;
         }
-        if ((rc = ensure_graph(h))) return rc;
-        const int64_t reps = n / 2;
-        if (reps > kPollReplays && (rc = ensure_poll(h))) return rc;
+        const bool longer = n >= 2 * kLongSteps && h->geo.M <= kLongNodes;
+        if ((rc = ensure_graph(h, h->graph, 2))) return rc;
+        if (longer && (rc = ensure_graph(h, h->graph_long, kLongSteps))) return rc;
+        if (n / 2 * 2 > kPollSteps && (rc = ensure_poll(h))) return rc;
         h->poll_pending = false;
-        for (int64_t k = 0; k < reps; ++k) {
-            if (k > 0 && k % kPollReplays == 0 && (rc = poll_status(h))) return rc;
-            CU(h, cudaGraphLaunch(h->graph, h->stream));
-            h->launches += 2 * kernels_per_step(h);
+        for (int64_t unpolled = 0; n >= 2;) {
+            const int k = longer && n >= kLongSteps ? kLongSteps : 2;
+            if (unpolled >= kPollSteps) {
+                if ((rc = poll_status(h))) return rc;
+                unpolled = 0;
+            }
+            CU(h, cudaGraphLaunch(k == 2 ? h->graph : h->graph_long, h->stream));
+            h->launches += k * kernels_per_step(h);
+            unpolled += k;
+            n -= k;
         }
-        n %= 2;
     }
     for (int64_t k = 0; k < n; ++k)
         if ((rc = step_plain(h, h->stream))) return rc;
@@ -1335,10 +1377,7 @@ int lbm_set_wall_distances(lbm_handle h, const double *q)
     h->bn = h->bmask = nullptr;
     h->bq = nullptr;
     h->nb = 0;
-    if (h->graph) {   // the captured steps change
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    drop_graphs(h);  // the captured steps change
     if (bn.empty()) return LBM_OK;
     CU(h, cudaMalloc(&h->bn, sizeof(unsigned) * bn.size()));
     CU(h, cudaMalloc(&h->bmask, sizeof(unsigned) * bm.size()));
@@ -1596,7 +1635,8 @@ struct lbm_batch_ctx {
     };
     std::vector<Launch> steps;
     int grid = 0, parity = 0;   // blocks of the plain launch
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr, graph_long = nullptr;   // two steps, kLongSteps steps
+    long long nodes = 0;   // of all members
     int64_t launches = 0;
 };
 
@@ -1628,7 +1668,7 @@ void launch_batch_plain(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, in
 template <typename ST>
 void launch_batch_2d(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
 {
-    lbmf2::k_step2d_batch<ST><<<n, lbmf2::NT, 0, s>>>(b->d_members[parity], items);
+    lbmpdl::launch_step(n > 5 * b->members[0]->sms, lbmf2::k_step2d_batch<ST>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
 }
 
 // One step of every member.
@@ -1692,10 +1732,32 @@ std::vector<lbmf::WorkItem> batch_items(const std::vector<lbm_ctx *> &members, c
     return best;
 }
 
+// `steps` (even) steps from parity 0, captured once.
+int batch_graph(lbm_batch_ctx *b, cudaGraphExec_t &graph, int steps)
+{
+    if (graph) return LBM_OK;
+    cudaStream_t cap = nullptr;
+    if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return LBM_ECUDA;
+    cudaGraph_t gr = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int k = 0; k < steps; ++k) batch_launch(b, k & 1, cap);
+        e = cudaStreamEndCapture(cap, &gr);
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&graph, gr, 0);
+    if (gr) cudaGraphDestroy(gr);
+    cudaStreamDestroy(cap);
+    if (e == cudaSuccess) return LBM_OK;
+    graph = nullptr;
+    cudaGetLastError();
+    return LBM_ECUDA;
+}
+
 void batch_free(lbm_batch_ctx *b)
 {
     if (!b) return;
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    if (b->graph_long) cudaGraphExecDestroy(b->graph_long);
     for (auto *m : b->d_members) if (m) cudaFree(m);
     if (b->d_items) cudaFree(b->d_items);
     if (b->d_maps) cudaFree(b->d_maps);
@@ -1727,6 +1789,7 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
     for (lbm_ctx *h : b->members) {
         b->cur0.push_back(h->cur);
         b->prev.push_back(h->stream);
+        b->nodes += h->geo.M;
     }
     for (lbm_ctx *h : b->members) cudaStreamSynchronize(h->stream);
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) return LBM_ECUDA;
@@ -1854,29 +1917,16 @@ int lbm_batch_step(lbm_batch b, int64_t n)
             ++b->launches;
             --n;
         }
-        if (!b->graph) {
-            cudaStream_t cap = nullptr;
-            if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return LBM_ECUDA;
-            cudaGraph_t gr = nullptr;
-            cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                batch_launch(b, 0, cap);
-                batch_launch(b, 1, cap);
-                e = cudaStreamEndCapture(cap, &gr);
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, gr, 0);
-            if (gr) cudaGraphDestroy(gr);
-            cudaStreamDestroy(cap);
-            if (e != cudaSuccess) {
-                b->graph = nullptr;
-                cudaGetLastError();
-                return LBM_ECUDA;
-            }
+        const bool longer = n >= 2 * kLongSteps && b->nodes <= (long long)kLongNodes;
+        int rc = batch_graph(b, b->graph, 2);
+        if (rc == LBM_OK && longer) rc = batch_graph(b, b->graph_long, kLongSteps);
+        if (rc != LBM_OK) return rc;
+        while (n >= 2) {
+            const int k = longer && n >= kLongSteps ? kLongSteps : 2;
+            if (cudaGraphLaunch(k == 2 ? b->graph : b->graph_long, b->stream) != cudaSuccess) return LBM_ECUDA;
+            b->launches += k;
+            n -= k;
         }
-        for (int64_t k = 0; k < n / 2; ++k)
-            if (cudaGraphLaunch(b->graph, b->stream) != cudaSuccess) return LBM_ECUDA;
-        b->launches += 2 * (n / 2);
-        n %= 2;
     }
     for (int64_t k = 0; k < n; ++k) {
         batch_launch(b, b->parity, b->stream);
@@ -2036,10 +2086,7 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
     h->geof.chunk = rc == LBM_OK ? best : chunk0;
     h->variant = rc == LBM_OK ? best_variant : variant0;
     if (rc != LBM_OK) h->auto_form = auto0;
-    if (h->graph) {
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    drop_graphs(h);
     cudaError_t e = cudaMemcpyAsync(h->fv[0], save, bytes, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess && rbytes)
         e = cudaMemcpyAsync(h->rs[0], static_cast<char *>(save) + bytes, rbytes,
@@ -2077,10 +2124,7 @@ int lbm_set_tile(lbm_handle h, int tile_y)
     if (tile_y == 7 && !h->auto_form && h->variant >= LBM_FUSED_WS_TMEM)
         return fail(h, LBM_EINVAL, "the warp-specialised Tensor Memory forms run 8-row tiles");
     leave_auto_form(h);
-    if (h->tile_rows != tile_y && h->graph) {   // the captured graph holds the other kernel
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    if (h->tile_rows != tile_y) drop_graphs(h);  // the captured graph holds the other kernel
     h->tile_rows = tile_y;
     return LBM_OK;
 }
@@ -2106,10 +2150,7 @@ int lbm_set_fused_variant(lbm_handle h, int variant)
     if (shifted(h->storage) && variant == LBM_FUSED_WARP_SPECIALISED)
         return fail(h, LBM_EINVAL, "shifted storage has the plain and the Tensor Memory forms");
     leave_auto_form(h);
-    if (h->variant != variant && h->graph) {   // the captured graph holds the other kernel
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    if (h->variant != variant) drop_graphs(h);  // the captured graph holds the other kernel
     h->variant = variant;
     return LBM_OK;
 }
@@ -2126,10 +2167,7 @@ int lbm_set_chunk(lbm_handle h, int chunk)
     if (!h) return LBM_EINVAL;
     if (chunk < 1) return fail(h, LBM_EINVAL, "chunk must be >= 1");
     leave_auto_form(h);
-    if (h->geof.chunk != chunk && h->graph) {
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-    }
+    if (h->geof.chunk != chunk) drop_graphs(h);
     h->geof.chunk = chunk;
     return LBM_OK;
 }
@@ -2140,7 +2178,7 @@ void lbm_destroy(lbm_handle h)
 {
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
-    if (h->graph) cudaGraphExecDestroy(h->graph);
+    drop_graphs(h);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->owns_base && h->base) cudaFree(h->base);
     if (h->bn) cudaFree(h->bn);

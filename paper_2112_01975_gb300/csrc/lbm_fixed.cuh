@@ -58,16 +58,18 @@ __device__ __forceinline__ long long shift_down(unsigned long long v, int k)
     return (long long)((v + (1ull << (k - 1))) >> k);
 }
 
-// Node n = (x, y, z): q[i] 2^e2 = population i.
+// Node n = (x, y, z): q[i] 2^e2 = population i. skip: nothing is formed (the
+// populations have been requested by then, beside what `skip` waits for).
 template <int LAT>
 __device__ __forceinline__ bool fixed_pops(const Geo &g, const double *__restrict__ f, unsigned n, int, int, int,
-                                           long long *q, int &e2)
+                                           long long *q, int &e2, bool skip)
 {
     constexpr int Q = Lattice<LAT>::Q;
     double v[Q];
     unsigned top = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i] = f[(size_t)i * g.N + n];
+    if (skip) return true;
 #pragma unroll
     for (int i = 0; i < Q; ++i) top = max(top, (unsigned)__double2hiint(v[i]));
     const int E = (int)(top >> 20);
@@ -85,12 +87,13 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const double *__restric
 
 template <int LAT>
 __device__ __forceinline__ bool fixed_pops(const Geo &g, const float *__restrict__ f, unsigned n, int, int, int,
-                                           long long *q, int &e2)
+                                           long long *q, int &e2, bool skip)
 {
     constexpr int Q = Lattice<LAT>::Q;
     unsigned b[Q], top = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) b[i] = __float_as_uint(f[(size_t)i * g.N + n]);
+    if (skip) return true;
 #pragma unroll
     for (int i = 0; i < Q; ++i) top = max(top, b[i]);
     const int E = (int)(top >> 23);
@@ -108,7 +111,7 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const float *__restrict
 // multiple of 2^-25 and the rest), times the 31-bit mantissa of the density.
 template <int LAT, typename ST>
 __device__ __forceinline__ bool fixed_pops(const Geo &g, const Shifted<ST> &f, unsigned n, int x, int y, int z,
-                                           long long *q, int &e2)
+                                           long long *q, int &e2, bool skip)
 {
     constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
     constexpr double W1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
@@ -124,6 +127,7 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const Shifted<ST> &f, u
         const unsigned src = entry(g, X[cxi(i) + 1], Y[cyi(i) + 1], Z[D == 3 ? czi(i) + 1 : 1]);
         s[i] = __float_as_uint(f.rho_src[src]);
     }
+    if (skip) return true;
     const unsigned own = s[Q / 2];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -174,14 +178,15 @@ __device__ __forceinline__ double pop_f64(const Geo &g, const Shifted<ST> &f, in
 // sum c_a c_b f (xx, yy[, zz], xy[, xz, yz]).
 template <int LAT, bool SECOND, typename P>
 __device__ __forceinline__ void node_sums(const Geo &g, const P &f, unsigned n, int x, int y, int z, double &rho,
-                                          double *j, double *second = nullptr)
+                                          double *j, double *second = nullptr, bool skip = false)
 {
     constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q, NA = D == 3 ? 6 : 3;
     constexpr int CA[6] = {0, 1, D == 3 ? 2 : 0, 0, 0, 1};
     constexpr int CB[6] = {0, 1, D == 3 ? 2 : 1, 1, 2, 2};
     long long q[Q];
     int e2;
-    if (fixed_pops<LAT>(g, f, n, x, y, z, q, e2)) {
+    if (fixed_pops<LAT>(g, f, n, x, y, z, q, e2, skip)) {
+        if (skip) return;
         long long r = 0, jj[3] = {0, 0, 0}, ss[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
         for (int i = 0; i < Q; ++i) {

@@ -21,6 +21,7 @@
 #pragma once
 
 #include "lbm_fused_f32.cuh"
+#include "lbm_pdl.cuh"
 
 namespace lbmf2 {
 
@@ -182,6 +183,8 @@ k_step2d(GeoF g, PhysF p, const uint8_t *__restrict__ mask, const ST *__restrict
          const float *__restrict__ rho_src, float *__restrict__ rho_dst, int *__restrict__ status)
 {
     __shared__ Shared2 sm;
+    lbmpdl::step_trigger();
+    lbmpdl::step_wait();
     tile2d<MASK, ST, E64>(g, p, mask, f, fout, status, blockIdx.x, blockIdx.y, sm, rho_src, rho_dst);
 }
 
@@ -193,6 +196,8 @@ k_step2d_batch(const MemberF *__restrict__ members, const WorkItem *__restrict__
     __shared__ Shared2 sm;
     const WorkItem w = items[blockIdx.x];
     const MemberF &m = members[w.member];
+    lbmpdl::step_trigger();
+    lbmpdl::step_wait();
     const ST *src = static_cast<const ST *>(m.src);
     ST *dst = static_cast<ST *>(m.dst);
     if (m.mask)

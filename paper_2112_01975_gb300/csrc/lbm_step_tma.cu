@@ -25,8 +25,7 @@ void launch_b(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_item
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     const int bytes = (int)sizeof(lbmf::SharedWT<1>);
     opt_in(lbmf::k_step_f32_wstma_batch<MASK, EOSK>, bytes, done);
-    lbmf::k_step_f32_wstma_batch<MASK, EOSK>
-        <<<n_items, 2 * lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(batch, items);
+    lbmpdl::launch_step(true, lbmf::k_step_f32_wstma_batch<MASK, EOSK>, n_items, 2 * lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s, batch, items);
 }
 
 template <typename ST, bool MASK>
@@ -35,8 +34,7 @@ void launch_bs(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_ite
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
     opt_in(lbmf::k_step_shifted_tmtma_batch<ST, MASK>, bytes, done);
-    lbmf::k_step_shifted_tmtma_batch<ST, MASK>
-        <<<n_items, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(batch, items);
+    lbmpdl::launch_step(false, lbmf::k_step_shifted_tmtma_batch<ST, MASK>, n_items, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s, batch, items);
 }
 
 template <bool MASK, int EOSK>
@@ -48,8 +46,7 @@ void launch_k(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     const int bytes = (int)sizeof(lbmf::SharedWT<1>);
     opt_in(lbmf::k_step_f32_wstma<1, MASK, EOSK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
-    lbmf::k_step_f32_wstma<1, MASK, EOSK><<<grid, 2 * L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
-                                                                                 status);
+    lbmpdl::launch_step(true, lbmf::k_step_f32_wstma<1, MASK, EOSK>, grid, 2 * L::TX * L::TY, bytes, s, g, p, mask, maps, src, dst, status);
 }
 
 template <bool MASK>
@@ -75,8 +72,7 @@ void launch_s(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     const int bytes = (int)sizeof(lbmf::SharedSWT<1, ST>);
     opt_in(lbmf::k_step_shifted_wstma<1, ST, MASK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
-    lbmf::k_step_shifted_wstma<1, ST, MASK><<<grid, 2 * L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
-                                                                                   rho_src, rho_dst, status);
+    lbmpdl::launch_step(false, lbmf::k_step_shifted_wstma<1, ST, MASK>, grid, 2 * L::TX * L::TY, bytes, s, g, p, mask, maps, src, dst, rho_src, rho_dst, status);
 }
 
 template <typename ST, bool MASK>
@@ -88,8 +84,7 @@ void launch_t(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
     opt_in(lbmf::k_step_shifted_tmtma<1, ST, MASK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
-    lbmf::k_step_shifted_tmtma<1, ST, MASK><<<grid, L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst,
-                                                                              rho_src, rho_dst, status);
+    lbmpdl::launch_step(false, lbmf::k_step_shifted_tmtma<1, ST, MASK>, grid, L::TX * L::TY, bytes, s, g, p, mask, maps, src, dst, rho_src, rho_dst, status);
 }
 
 }  // namespace
