@@ -602,17 +602,24 @@ void launch_fused_e64(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 
 // The D2Q9 step of a reduced storage from population buffer k: one kernel,
 // whatever form, chunk or tile the handle names (lbm_step2d.cuh).
-template <typename ST, bool MASK, bool E64>
-void launch_2d_m(lbm_ctx *h, cudaStream_t s, int k)
+template <typename ST, bool MASK, bool E64, bool REST>
+void launch_2d_r(lbm_ctx *h, cudaStream_t s, int k)
 {
     const GeoF &g = h->geof;
     const dim3 grid((g.nx + lbmf2::TX - 1) / lbmf2::TX, (g.nz + lbmf2::TY - 1) / lbmf2::TY);
     // (five blocks per SM are resident: more of them leave a successor no room)
     const long long blocks = (long long)grid.x * grid.y;
     const bool overlap = lbmpdl::side_by_side(blocks, h->sms) || blocks > 5 * h->sms;
-    lbmpdl::launch_step(overlap, lbmf2::k_step2d<MASK, ST, E64>, grid, lbmf2::NT, 0, s, g, h->physf, h->mask,
+    lbmpdl::launch_step(overlap, lbmf2::k_step2d<MASK, ST, E64, REST>, grid, lbmf2::NT, 0, s, g, h->physf, h->mask,
                         static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]), h->rs[k], h->rs[k ^ 1],
                         h->status);
+}
+
+template <typename ST, bool MASK, bool E64>
+void launch_2d_m(lbm_ctx *h, cudaStream_t s, int k)
+{
+    if (lbmf::at_rest(h->physf)) launch_2d_r<ST, MASK, E64, true>(h, s, k);
+    else                         launch_2d_r<ST, MASK, E64, false>(h, s, k);
 }
 
 template <typename ST>
@@ -625,6 +632,17 @@ void launch_2d(lbm_ctx *h, cudaStream_t s, int k)
         if (h->e64) launch_2d_m<ST, false, true>(h, s, k);
         else        launch_2d_m<ST, false, false>(h, s, k);
     }
+}
+
+template <int LAT, bool MASK>
+void launch_fused_rest(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
+{
+    static std::atomic<unsigned long long> done{0};   // devices already opted in
+    using L = lbmf::LatF<LAT>;
+    const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
+    smem_opt_in(lbmf::k_step_f32<LAT, MASK, false, true>, bytes, done);
+    lbmf::k_step_f32<LAT, MASK, false, true><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+        h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
 template <int LAT>
@@ -643,6 +661,12 @@ void launch_fused(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
     if (h->variant == LBM_FUSED_WARP_SPECIALISED) {
         if (has_solid(h)) launch_fused_ws<LAT, true>(h, s, src, dst);
         else              launch_fused_ws<LAT, false>(h, s, src, dst);
+        return;
+    }
+    if (lbmf::at_rest(h->physf) && (h->variant == LBM_FUSED_TMEM || h->variant == LBM_FUSED_PLAIN)) {
+        // nothing to keep between the phases: the two forms are one
+        if (has_solid(h)) launch_fused_rest<LAT, true>(h, s, src, dst);
+        else              launch_fused_rest<LAT, false>(h, s, src, dst);
         return;
     }
     if (h->variant == LBM_FUSED_TMEM) {
@@ -682,14 +706,14 @@ void launch_f32(lbm_ctx *h, cudaStream_t s, int k)
     else                        launch_fused<1>(h, s, f32(h, k), f32(h, k ^ 1));
 }
 
-template <int LAT, typename ST, bool E64, bool MASK>
+template <int LAT, typename ST, bool E64, bool MASK, bool REST = false>
 void launch_shifted_e(lbm_ctx *h, cudaStream_t s, int k)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
     const int bytes = (int)sizeof(lbmf::SharedS<LAT>);
-    smem_opt_in(lbmf::k_step_shifted<LAT, ST, E64, MASK>, bytes, done);
+    smem_opt_in(lbmf::k_step_shifted<LAT, ST, E64, MASK, REST>, bytes, done);
     using L = lbmf::LatF<LAT>;
-    lbmf::k_step_shifted<LAT, ST, E64, MASK><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    lbmf::k_step_shifted<LAT, ST, E64, MASK, REST><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]),
         h->rs[k], h->rs[k ^ 1], h->status);
 }
@@ -733,6 +757,8 @@ void launch_shifted_m(lbm_ctx *h, cudaStream_t s, int k)
         return;
     }
     if (h->e64) launch_shifted_e<LAT, ST, true, MASK>(h, s, k);
+    else if (lbmf::at_rest(h->physf) && (h->variant == LBM_FUSED_TMEM || h->variant == LBM_FUSED_PLAIN))
+        launch_shifted_e<LAT, ST, false, MASK, true>(h, s, k);   // nothing to keep between the phases
     else if (h->variant == LBM_FUSED_TMEM) launch_shifted_tm<LAT, ST, MASK>(h, s, k);
     else if (LAT == 1 && h->variant == LBM_FUSED_WS_TMEM) launch_shifted_wstm<ST, MASK>(h, s, k);
     else launch_shifted_e<LAT, ST, false, MASK>(h, s, k);
@@ -1629,7 +1655,7 @@ struct lbm_batch_ctx {
     // a step: launches of up to kBatchMembers TMA-staged D3Q27 members, and
     // one of all members that have no such form (or of all D2Q9 members)
     struct Launch {
-        bool tma, solid;
+        bool tma, solid, rest;   // rest: every member relaxes with time 1
         int first, n_items, eos;
         lbmf::BatchT args[2];   // TMA-staged: by step parity
     };
@@ -1666,9 +1692,11 @@ void launch_batch_plain(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, in
 }
 
 template <typename ST>
-void launch_batch_2d(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
+void launch_batch_2d(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, bool rest, int parity, cudaStream_t s)
 {
-    lbmpdl::launch_step(n > 5 * b->members[0]->sms, lbmf2::k_step2d_batch<ST>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
+    const bool overlap = n > 5 * b->members[0]->sms;
+    if (rest) lbmpdl::launch_step(overlap, lbmf2::k_step2d_batch<ST, true>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
+    else lbmpdl::launch_step(overlap, lbmf2::k_step2d_batch<ST, false>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
 }
 
 // One step of every member.
@@ -1677,15 +1705,15 @@ void batch_launch(lbm_batch_ctx *b, int parity, cudaStream_t s)
     for (const lbm_batch_ctx::Launch &l : b->steps) {
         const lbmf::WorkItem *items = b->d_items + l.first;
         if (l.tma) {
-            if (b->storage == LBM_F32) lbmtma::launch_batch(l.args[parity], items, l.n_items, l.eos, l.solid, s);
+            if (b->storage == LBM_F32) lbmtma::launch_batch(l.args[parity], items, l.n_items, l.eos, l.solid, l.rest, s);
             else if (b->storage == LBM_F16S)
-                lbmtma::launch_batch_shifted<__half>(l.args[parity], items, l.n_items, l.solid, s);
+                lbmtma::launch_batch_shifted<__half>(l.args[parity], items, l.n_items, l.solid, l.rest, s);
             else
-                lbmtma::launch_batch_shifted<__nv_bfloat16>(l.args[parity], items, l.n_items, l.solid, s);
+                lbmtma::launch_batch_shifted<__nv_bfloat16>(l.args[parity], items, l.n_items, l.solid, l.rest, s);
         } else if (b->lattice != LBM_D2Q9) launch_batch_plain(b, items, l.n_items, parity, s);
-        else if (b->storage == LBM_F32) launch_batch_2d<float>(b, items, l.n_items, parity, s);
-        else if (b->storage == LBM_F16S) launch_batch_2d<__half>(b, items, l.n_items, parity, s);
-        else launch_batch_2d<__nv_bfloat16>(b, items, l.n_items, parity, s);
+        else if (b->storage == LBM_F32) launch_batch_2d<float>(b, items, l.n_items, l.rest, parity, s);
+        else if (b->storage == LBM_F16S) launch_batch_2d<__half>(b, items, l.n_items, l.rest, parity, s);
+        else launch_batch_2d<__nv_bfloat16>(b, items, l.n_items, l.rest, parity, s);
     }
 }
 
@@ -1846,9 +1874,11 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
         l.first = (int)items.size();
         l.n_items = (int)part.size();
         l.eos = b->members[which[0]]->physf.eos;
+        l.rest = true;
         for (size_t k = 0; k < which.size(); ++k) {
             const lbm_ctx *h = b->members[which[k]];
             l.solid = l.solid || h->any_solid;
+            l.rest = l.rest && lbmf::at_rest(h->physf);
             if (h->physf.eos != l.eos) l.eos = -1;
             for (int par = 0; par < 2; ++par) {
                 lbmf::MemberT &m = l.args[par].m[k];
@@ -1871,6 +1901,8 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
         lbm_batch_ctx::Launch l = {};
         l.first = (int)items.size();
         l.n_items = (int)plain.size();
+        l.rest = true;
+        for (const lbm_ctx *h : b->members) l.rest = l.rest && lbmf::at_rest(h->physf);
         b->grid = std::min(l.n_items, 2 * sms);
         items.insert(items.end(), plain.begin(), plain.end());
         b->steps.push_back(l);

@@ -72,7 +72,7 @@ __device__ __forceinline__ void halo2(int k, int &r, int &c)
     c = e < 2 ? e : AX - 4 + e;
 }
 
-template <bool MASK, typename ST, bool E64>
+template <bool MASK, typename ST, bool E64, bool REST>
 __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint8_t *__restrict__ mask,
                                        const ST *__restrict__ f, ST *__restrict__ fout,
                                        int *__restrict__ status, int bx, int by, Shared2 &sm,
@@ -131,7 +131,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
         } else {
             m = node_moments<0, E64>(p, fi[u], ring1);
         }
-        const float psi = E64 && !solid[u] ? m.psi64 : sqrtf(fabsf(m.d));
+        const float psi = E64 && !solid[u] ? m.psi64 : root_f(fabsf(m.d));
         sm.rp[r][c] = f2(m.rho, psi);
         if (ring1) {
             sm.g[0][r - 1][c - 1] = m.gx;
@@ -161,23 +161,19 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
                           pref * 0.5f * (sm.g[1][ty + 2][tx + 1] - sm.g[1][ty][tx + 1])};
     const float inv = own.uv.w;
     const float un[3] = {own.uv.x, own.uv.y, own.uv.z};
-    float2 ES[3][3], A[3][3];
-    factors_f<0>(rho, inv, un, F, Phi, ES, A);
-    // post = f* + (1 - omega)(f - feq), pushed to r + c_i (halfway bounce-back at solids)
+    const PostF<0, REST, SHIFT> post(rho, inv, un, F, Phi, omw);
+    // pushed to r + c_i (halfway bounce-back at solids)
     const int X[3] = {wrapf(x - 1, nx), x, wrapf(x + 1, nx)};
     const int Y[3] = {wrapf(y - 1, ny), y, wrapf(y + 1, ny)};
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const float2 es = __fmul2_rn(A[L::cx(i) + 1][1], ES[2][L::cz(i) + 1]);   // (feq, f*)
-        const float post = SHIFT ? fmaf(fmaf(omw, fi[0][i] - es.x, es.y), inv, -weight_f<0>(i))
-                                 : fmaf(omw, fi[0][i] - es.x, es.y);
         const unsigned dst = (unsigned)X[L::cx(i) + 1] + (unsigned)g.px * (unsigned)Y[L::cz(i) + 1];
-        if (MASK && mask[dst]) fout[(Q - 1 - i) * N + n] = from_f<ST>(post);
-        else                   fout[i * N + dst] = from_f<ST>(post);
+        if (MASK && mask[dst]) fout[(Q - 1 - i) * N + n] = from_f<ST>(post(i, fi[0]));
+        else                   fout[i * N + dst] = from_f<ST>(post(i, fi[0]));
     }
 }
 
-template <bool MASK, typename ST, bool E64>
+template <bool MASK, typename ST, bool E64, bool REST>
 __global__ void __launch_bounds__(NT)
 k_step2d(GeoF g, PhysF p, const uint8_t *__restrict__ mask, const ST *__restrict__ f, ST *__restrict__ fout,
          const float *__restrict__ rho_src, float *__restrict__ rho_dst, int *__restrict__ status)
@@ -185,11 +181,11 @@ k_step2d(GeoF g, PhysF p, const uint8_t *__restrict__ mask, const ST *__restrict
     __shared__ Shared2 sm;
     lbmpdl::step_trigger();
     lbmpdl::step_wait();
-    tile2d<MASK, ST, E64>(g, p, mask, f, fout, status, blockIdx.x, blockIdx.y, sm, rho_src, rho_dst);
+    tile2d<MASK, ST, E64, REST>(g, p, mask, f, fout, status, blockIdx.x, blockIdx.y, sm, rho_src, rho_dst);
 }
 
 // The same over the tiles of many lattices: block b takes item b.
-template <typename ST>
+template <typename ST, bool REST>
 __global__ void __launch_bounds__(NT)
 k_step2d_batch(const MemberF *__restrict__ members, const WorkItem *__restrict__ items)
 {
@@ -201,9 +197,9 @@ k_step2d_batch(const MemberF *__restrict__ members, const WorkItem *__restrict__
     const ST *src = static_cast<const ST *>(m.src);
     ST *dst = static_cast<ST *>(m.dst);
     if (m.mask)
-        tile2d<true, ST, false>(m.g, m.p, m.mask, src, dst, m.status, w.bx, w.by, sm, m.rho_src, m.rho_dst);
+        tile2d<true, ST, false, REST>(m.g, m.p, m.mask, src, dst, m.status, w.bx, w.by, sm, m.rho_src, m.rho_dst);
     else
-        tile2d<false, ST, false>(m.g, m.p, m.mask, src, dst, m.status, w.bx, w.by, sm, m.rho_src, m.rho_dst);
+        tile2d<false, ST, false, REST>(m.g, m.p, m.mask, src, dst, m.status, w.bx, w.by, sm, m.rho_src, m.rho_dst);
 }
 
 }  // namespace lbmf2

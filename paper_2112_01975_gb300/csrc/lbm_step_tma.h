@@ -1,6 +1,6 @@
 // Launcher of the TMA-staged fused FP32 step (k_step_f32_wstma), compiled in
 // its own translation unit (lbm_step_tma.cu): one kernel per equation of
-// state and solid-node mode, 2 x 6 instantiations, built in parallel with
+// state, solid-node mode and relaxation (time 1 or another), built in parallel with
 // the rest of the library. Internal to the library (not part of the C ABI).
 #pragma once
 
@@ -35,11 +35,12 @@ void launch_shifted_tm(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t 
                        cudaStream_t s);
 
 // One step of the n_items items over the members of a batch (`solid`: one of
-// them has solid nodes; eos: that of all of them, or -1).
+// them has solid nodes; eos: that of all of them, or -1; rest: all of them
+// relax with time 1, at_rest).
 void launch_batch(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, int eos, bool solid,
-                  cudaStream_t s);
+                  bool rest, cudaStream_t s);
 template <typename ST>
 void launch_batch_shifted(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_items, bool solid,
-                          cudaStream_t s);
+                          bool rest, cudaStream_t s);
 
 }  // namespace lbmtma
