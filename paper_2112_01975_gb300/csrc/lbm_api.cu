@@ -42,6 +42,7 @@ struct lbm_ctx {
     double t_over_tc, tau;
     std::vector<uint8_t> mask_host, zsolid_host;
     bool any_solid = false;
+    int *walls = nullptr;   // D3Q27 reduced storage with solids: GeoF::wplane and GeoF::walls
     int sms = 148;         // SMs of the device
     int sweep_chunk = 16;  // planes per block of the D3Q27 force sweep (FP64 kernels); 0: direct sums
     int device;
@@ -240,20 +241,6 @@ double excess_pressure_host(int eos, double a, double b, double RT, double aalph
     return P - r / 3.0;
 }
 
-dim3 node_block(const Geo &g)
-{
-    int bx = g.nx >= 128 ? 128 : ((g.nx + 31) / 32) * 32;
-    return dim3(bx, 1, 1);
-}
-
-dim3 node_grid(const Geo &g)
-{
-    dim3 b = node_block(g);
-    return dim3((g.nx + b.x - 1) / b.x, g.ny, g.nz);
-}
-
-void make_tensor_maps(lbm_ctx *h);
-
 // Makespan of n_full blocks of cost cf, then n_tail of cost ct <= cf, each
 // taken by the first of `slots` that is free.
 double makespan(long long n_full, double cf, long long n_tail, double ct, long long slots)
@@ -270,6 +257,20 @@ double makespan(long long n_full, double cf, long long n_tail, double ct, long l
     }
     return b;
 }
+
+dim3 node_block(const Geo &g)
+{
+    int bx = g.nx >= 128 ? 128 : ((g.nx + 31) / 32) * 32;
+    return dim3(bx, 1, 1);
+}
+
+dim3 node_grid(const Geo &g)
+{
+    dim3 b = node_block(g);
+    return dim3((g.nx + b.x - 1) / b.x, g.ny, g.nz);
+}
+
+void make_tensor_maps(lbm_ctx *h);
 
 // The chunk of planes per block that ends the step first: a block of c planes
 // marches through c + 4. `resident` blocks share an SM; two together take
@@ -336,6 +337,43 @@ void leave_auto_form(lbm_ctx *h)
     drop_graphs(h);  // the captured graph holds the chosen form
 }
 
+// The wall bits of the planes within one of a solid node, in an allocation of
+// the handle's own (4 bytes per node of those planes and 8 per plane).
+int make_wall_bits(lbm_ctx *h)
+{
+    if (h->lattice != LBM_D3Q27 || h->storage == LBM_F64 || !h->any_solid) return LBM_OK;
+    const Geo &g = h->geo;
+    std::vector<int> table, planes;   // number of each z's plane; z of each plane
+    try {
+        table.assign(g.nz, -1);
+        for (int z = 0; z < g.nz; ++z)
+            if (h->zsolid_host[(z + g.nz - 1) % g.nz] || h->zsolid_host[z] || h->zsolid_host[(z + 1) % g.nz]) {
+                table[z] = (int)planes.size();
+                planes.push_back(z);
+            }
+    } catch (const std::bad_alloc &) {
+        return fail(h, LBM_ENOMEM, "no host memory for the wall planes");
+    }
+    const size_t head = align_up(sizeof(int) * 2 * g.nz), bits = sizeof(unsigned) * planes.size() * g.px * g.ny;
+    if (!h->walls && cudaMalloc(&h->walls, head + bits) != cudaSuccess) {
+        cudaGetLastError();
+        h->walls = nullptr;
+        return fail(h, LBM_ENOMEM, "cudaMalloc(%zu) for the wall bits failed", head + bits);
+    }
+    unsigned *const w = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(h->walls) + head);
+    CU(h, cudaMemcpyAsync(h->walls, table.data(), sizeof(int) * g.nz, cudaMemcpyHostToDevice, h->stream));
+    CU(h, cudaMemcpyAsync(h->walls + g.nz, planes.data(), sizeof(int) * planes.size(), cudaMemcpyHostToDevice,
+                          h->stream));
+    dim3 gr = node_grid(g);
+    gr.z = (unsigned)planes.size();
+    lbmk::k_wall_bits<<<gr, node_block(g), 0, h->stream>>>(g, h->mask, h->walls + g.nz, w);
+    CU(h, cudaGetLastError());
+    CU(h, cudaStreamSynchronize(h->stream));   // before the host vectors go
+    h->geof.wplane = h->walls;
+    h->geof.walls = w;
+    return LBM_OK;
+}
+
 int ensure_memory(lbm_ctx *h)
 {
     if (h->fv[0]) return LBM_OK;
@@ -388,6 +426,11 @@ int ensure_memory(lbm_ctx *h)
                               cudaMemcpyHostToDevice, h->stream));
     }
     CU(h, cudaMemsetAsync(h->status, 0, sizeof(int) * 4, h->stream));
+    const int rc = make_wall_bits(h);
+    if (rc != LBM_OK) {
+        h->fv[0] = nullptr;   // not laid out: the next call starts over
+        return rc;
+    }
     CU(h, cudaStreamSynchronize(h->stream));
     make_tensor_maps(h);
     if (h->variant == LBM_FUSED_WS_TMA && !h->tmap_ready) h->variant = LBM_FUSED_WS_TMEM;
@@ -490,11 +533,15 @@ int sweep_chunk(const Geo &g, int sms)
 {
     const long long tiles = (long long)((g.nx + lbmk::SWX - 1) / lbmk::SWX) *
                             ((g.ny + lbmk::SWY - 1) / lbmk::SWY);
+    // c planes cost 200 c + 256; two blocks share an SM at half speed each. The
+    // last, shorter chunk of each column fills in (128^3: chunk 29 667 us, 18
+    // 690, 14 684, 32 731).
     int best = 1;
     double cost = 1e300;
     for (int c = 1; c <= g.nz; ++c) {
-        const long long blocks = tiles * ((g.nz + c - 1) / c);
-        const double t = (double)((blocks + sms - 1) / sms) * (c * 200.0 + 4 * 64.0);
+        const long long full = tiles * (g.nz / c), tail = g.nz % c ? tiles : 0;
+        const double cf = c * 200.0 + 256.0, ct = g.nz % c * 200.0 + 256.0;
+        const double t = full + tail <= sms ? cf : 2.0 * makespan(full, cf, tail, ct, 2ll * sms);
         if (t < cost) {
             cost = t;
             best = c;
@@ -2213,6 +2260,7 @@ void lbm_destroy(lbm_handle h)
     drop_graphs(h);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->owns_base && h->base) cudaFree(h->base);
+    if (h->walls) cudaFree(h->walls);
     if (h->bn) cudaFree(h->bn);
     if (h->bmask) cudaFree(h->bmask);
     if (h->bq) cudaFree(h->bq);

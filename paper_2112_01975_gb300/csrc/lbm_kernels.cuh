@@ -784,6 +784,24 @@ __global__ void k_fill_solid(Geo g, Phys p, const uint8_t *__restrict__ mask,
     for (int a = 0; a < D; ++a) { u[a * g.N + n] = 0.0; gflux[a * g.N + n] = 0.0; }
 }
 
+// Wall bits of the planes near solids (GeoF::walls): bit i of node (x, y, z): its
+// neighbour along c_i is solid. planes: the z of each plane.
+__global__ void k_wall_bits(Geo g, const uint8_t *__restrict__ mask, const int *__restrict__ planes,
+                            unsigned *__restrict__ walls)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= g.nx) return;
+    const int y = blockIdx.y, z = planes[blockIdx.z];
+    const int X[3] = {wrapm(x - 1, g.nx), x, wrapp(x + 1, g.nx)};
+    const int Y[3] = {wrapm(y - 1, g.ny), y, wrapp(y + 1, g.ny)};
+    const int Z[3] = {wrapm(z - 1, g.nz), z, wrapp(z + 1, g.nz)};
+    unsigned w = 0;
+#pragma unroll
+    for (int i = 0; i < 27; ++i)
+        w |= (unsigned)mask[entry(g, X[cxi(i) + 1], Y[cyi(i) + 1], Z[czi(i) + 1])] << i;
+    walls[(size_t)g.px * g.ny * blockIdx.z + (unsigned)x + (unsigned)g.px * (unsigned)y] = w;
+}
+
 // Mass and momentum: fixed grid, fixed per-thread stride order and a fixed
 // shuffle tree, so the sums are bitwise reproducible run to run.
 constexpr int RED_THREADS = 256;
