@@ -908,11 +908,11 @@ int decode_to(lbm_ctx *h, int k, double *out)
     return LBM_OK;
 }
 
-template <int LAT>
+template <int LAT, bool INIT = false>
 int encode_from(lbm_ctx *h, const Geo &gf, const double *f)   // gf: the layout of f
 {
     const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    lbmk::k_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, gf, h->mask, f, h->rs[0], h->rs[1]);
+    lbmk::k_density<LAT, INIT><<<gr, bl, 0, h->stream>>>(h->geo, gf, h->mask, f, h->rs[0], h->rs[1]);
     if (h->storage == LBM_F16S)
         lbmk::k_encode_shifted<LAT, __half><<<gr, bl, 0, h->stream>>>(
             h->geo, gf, f, h->rs[0], static_cast<__half *>(h->fv[0]));
@@ -1058,17 +1058,17 @@ int launch_init(lbm_ctx *h, const double *rho0, const double *u0)
         TempF64 t;
         int rc = temp_alloc(h, t);
         if (rc) return rc;
-        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT>{h->mask, h->rp, u0, t.p});
-        rc = encode_from<LAT>(h, h->geo, t.p);
+        lbmk::k_init<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0, t.p);
+        rc = encode_from<LAT, true>(h, h->geo, t.p);
         if (rc) return rc;
         CU(h, cudaGetLastError());
         CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
         return LBM_OK;
     }
     if (h->storage == LBM_F32)
-        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT, float>{h->mask, h->rp, u0, f32(h, h->cur)});
+        lbmk::k_init<LAT, float><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0, f32(h, h->cur));
     else
-        launch_sweep<LAT>(h, h->stream, lbmk::InitBody<LAT>{h->mask, h->rp, u0, f64(h, h->cur)});
+        lbmk::k_init<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, u0, f64(h, h->cur));
     CU(h, cudaGetLastError());
     return LBM_OK;
 }

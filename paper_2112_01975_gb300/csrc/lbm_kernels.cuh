@@ -146,10 +146,41 @@ __device__ __forceinline__ double signed_psi_of(double d)
     return positive(d) ? r : -r;
 }
 
+// The same equations of state as pressures, for the initial state and the
+// walls' virtual density (see korteweg_force).
+__device__ __forceinline__ double eos_pressure(const Phys &p, double rho)
+{
+    switch (p.eos) {
+    case 0:  // van der Waals
+        return rho * p.RT / (1.0 - p.b * rho) - p.a * rho * rho;
+    case 1: {  // Peng-Robinson, one division
+        const double d1 = 1.0 - p.b * rho, d2 = 1.0 + 2.0 * p.b * rho - p.b * p.b * rho * rho;
+        return (rho * p.RT * d2 - p.a * p.alpha * rho * rho * d1) / (d1 * d2);
+    }
+    case 2: {  // Redlich-Kwong-Soave, one division
+        const double d1 = 1.0 - p.b * rho, d2 = 1.0 + p.b * rho;
+        return (rho * p.RT * d2 - p.a * p.alpha * rho * rho * d1) / (d1 * d2);
+    }
+    case 3: {  // Carnahan-Starling
+        const double e = 0.25 * p.b * rho;
+        const double om = 1.0 - e;
+        return rho * p.RT * (1.0 + e + e * e - e * e * e) / (om * om * om) - p.a * rho * rho;
+    }
+    case 4: {  // Shan-Chen, psi_SC = 1 - exp(-rho); RT holds the coupling G
+        const double q = 1.0 - exp(-rho);
+        return rho * (1.0 / 3.0) + p.RT * (1.0 / 6.0) * q * q;
+    }
+    default: {  // Shan-Chen, psi_SC = exp(-1/rho)
+        const double q = exp(-1.0 / rho);
+        return rho * (1.0 / 3.0) + p.RT * (1.0 / 6.0) * q * q;
+    }
+    }
+}
+
 __device__ __forceinline__ double signed_psi(const Phys &p, double rho)
 {
-    double inv;
-    return signed_psi_of(excess_pressure(p, rho, inv));
+    const double d = eos_pressure(p, rho) - rho * (1.0 / 3.0);
+    return d > 0.0 ? sqrt(d) : -sqrt(-d);
 }
 
 __device__ __forceinline__ int wrapm(int v, int n) { return v < 0 ? v + n : v; }
@@ -724,49 +755,112 @@ __global__ void k_init_density(Geo g, Phys p, const uint8_t *__restrict__ mask,
     rp[n] = make_double2(rho, signed_psi(p, rho));
 }
 
+// Korteweg force at one node, summed by itself: for the initial state, which is
+// formed once and stays the same to the bit whatever the step's sums do (the
+// last bit of an FP64 sum decides, once in a while, how a population rounds to
+// 16 or 32 bits, and a density ratio of 1e4 carries that far).
+//   F = -2 (s psi)_c S_psi - kappa rho_c S_rho + rho_c g,
+//   S_psi = sum_i (w_i/cs2) c_i [4/3 psi(r+c_i) - 1/6 psi(r+2c_i)],
+//   S_rho = sum_i (w_i/cs2) c_i [2 rho(r+c_i) - rho(r+2c_i)]   (Eq. Kforce_final).
+// w_i/cs2 c_ia = 1/2 W(c_ib) W(c_ic) c_ia with the 1D weights W(0) = 2/3,
+// W(+-1) = 1/6 of Eq. wi, so each ring sums neighbours by their number of
+// nonzero transverse components (centre, edge, corner) before weighting.
+template <int LAT>
+__device__ __forceinline__ void korteweg_force(const Geo &g, const Phys &p,
+                                               const double2 *__restrict__ rp, int x, int y,
+                                               int z, double rho_c, double spsi_c, double *F)
+{
+    constexpr int D = Lattice<LAT>::D;
+    double Spsi[3] = {0.0, 0.0, 0.0}, Srho[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int s = 1; s <= 2; ++s) {
+        const int xm = wrapm(x - s, g.nx), xp = wrapp(x + s, g.nx);
+        const int ym = wrapm(y - s, g.ny), yp = wrapp(y + s, g.ny);
+        int zm = 0, zp = 0;
+        if (D == 3) { zm = wrapm(z - s, g.nz); zp = wrapp(z + s, g.nz); }
+        const int X[3] = {xm, x, xp}, Y[3] = {ym, y, yp}, Z[3] = {zm, z, zp};
+        double ap[3][3], ar[3][3];  // [component][0 centre, 1 edge, 2 corner]
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { ap[a][k] = 0.0; ar[a][k] = 0.0; }
+        // each pair (c_i, -c_i) once: differences of the two neighbours, added
+        // with the sign of c_ia to every component where c_ia != 0
+#pragma unroll
+        for (int i = Lattice<LAT>::Q / 2 + 1; i < Lattice<LAT>::Q; ++i) {
+            const int c[3] = {cxi(i), cyi(i), D == 3 ? czi(i) : 0};
+            const unsigned np_ = entry(g, X[c[0] + 1], Y[c[1] + 1], Z[c[2] + 1]);
+            const unsigned nm_ = entry(g, X[1 - c[0]], Y[1 - c[1]], Z[1 - c[2]]);
+            const double2 vp = rp[np_], vm = rp[nm_];
+            const double dps = fabs(vp.y) - fabs(vm.y);
+            const double drh = vp.x - vm.x;
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                if (c[a] == 0) continue;
+                const int k = (a != 0 && c[0] != 0) + (a != 1 && c[1] != 0) + (a != 2 && c[2] != 0);
+                if (c[a] > 0) { ap[a][k] += dps; ar[a][k] += drh; }
+                else          { ap[a][k] -= dps; ar[a][k] -= drh; }
+            }
+        }
+        const double gp = s == 1 ? 4.0 / 3.0 : -1.0 / 6.0;
+        const double gr = s == 1 ? 2.0 : -1.0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            double dp, dr;
+            if (D == 3) {
+                dp = (2.0 / 9.0) * ap[a][0] + (1.0 / 18.0) * ap[a][1] + (1.0 / 72.0) * ap[a][2];
+                dr = (2.0 / 9.0) * ar[a][0] + (1.0 / 18.0) * ar[a][1] + (1.0 / 72.0) * ar[a][2];
+            } else {
+                dp = (1.0 / 3.0) * ap[a][0] + (1.0 / 12.0) * ap[a][1];
+                dr = (1.0 / 3.0) * ar[a][0] + (1.0 / 12.0) * ar[a][1];
+            }
+            Spsi[a] += gp * dp;
+            Srho[a] += gr * dr;
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < D; ++a) F[a] = -2.0 * spsi_c * Spsi[a] - p.kappa * rho_c * Srho[a] + rho_c * p.g[a];
+}
+
 // Initial populations at rest in the physical velocity: the equilibrium at
 // the bare velocity u = U0 - F/(2 rho0), F the Korteweg force of the initial
 // density (rp, filled by k_init_density and k_fill_solid), so that
 // U = u + F/(2 rho) of Sec. 2.3.5 equals U0 at t = 0. Zero at solid nodes.
-// The body of the force sweep.
 template <int LAT, typename T = double>
-struct InitBody {
-    const uint8_t *mask;
-    const double2 *rp;
-    const double *u0;
-    T *f;
-
-    __device__ __forceinline__ void operator()(const Geo &g, const Phys &p, unsigned n, int x, int y, int z,
-                                               const double *sp, const double *sr) const
-    {
-        constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
-        if (mask[n]) {
+__global__ void k_init(Geo g, Phys p, const uint8_t *__restrict__ mask,
+                       const double2 *__restrict__ rp, const double *__restrict__ u0,
+                       T *__restrict__ f)
+{
+    constexpr int D = Lattice<LAT>::D, Q = Lattice<LAT>::Q;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= g.nx) return;
+    const int y = blockIdx.y, z = blockIdx.z;
+    const unsigned n = entry(g, x, y, z), m = entry(flat(g), x, y, z);
+    if (mask[n]) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + n] = (T)0;
-            return;
-        }
-        const unsigned m = entry(flat(g), x, y, z);
-        const double2 c = rp[n];
-        const double rho = c.x, half = 0.5 / rho;
-        double F[3];
-        force_of_sums<LAT>(p, rho, c.y, sp, sr, F);
-        double E[3][3];
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const double ua = fma(-F[a], half, u0 ? u0[a * (size_t)g.M + m] : 0.0);
-            const double t = 0.5 * ua, h = fma(t, ua, 1.0 / 6.0);
-            E[a][0] = h - t;
-            E[a][1] = fma(-2.0, h, 1.0);
-            E[a][2] = h + t;
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            double eq = rho * E[0][cxi(i) + 1] * E[1][cyi(i) + 1];
-            if (D == 3) eq *= E[2][czi(i) + 1];
-            f[(size_t)i * g.N + n] = (T)eq;
-        }
+        for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + n] = (T)0;
+        return;
     }
-};
+    const double2 c = rp[n];
+    const double rho = c.x;
+    double F[3] = {0.0, 0.0, 0.0};
+    korteweg_force<LAT>(g, p, rp, x, y, z, rho, c.y, F);
+    double E[3][3];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const double ua = (u0 ? u0[a * (size_t)g.M + m] : 0.0) - F[a] / (2.0 * rho);
+        const double ze = 1.0 / 3.0 + ua * ua;
+        E[a][0] = 0.5 * (ze - ua);
+        E[a][1] = 1.0 - ze;
+        E[a][2] = 0.5 * (ze + ua);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        double eq = rho * E[0][cxi(i) + 1] * E[1][cyi(i) + 1];
+        if (D == 3) eq *= E[2][czi(i) + 1];
+        f[(size_t)i * g.N + n] = (T)eq;
+    }
+}
 
 template <int LAT>
 __global__ void k_fill_solid(Geo g, Phys p, const uint8_t *__restrict__ mask,
@@ -893,8 +987,9 @@ __global__ void k_decode_shifted(Geo g, const ST *__restrict__ h, const float *_
 // solid nodes stays for good): each fluid node's density, -1 at solid nodes
 // (their populations' sources are the fluid nodes that bounced them; see the
 // decoders).
-// gf: the layout of f (the caller's or the library's).
-template <int LAT>
+// gf: the layout of f (the caller's or the library's). INIT: the initial state,
+// summed in FP64 one after the other.
+template <int LAT, bool INIT>
 __global__ void k_density(Geo g, Geo gf, const uint8_t *__restrict__ mask, const double *__restrict__ f,
                           float *__restrict__ rho0, float *__restrict__ rho1)
 {
@@ -904,20 +999,46 @@ __global__ void k_density(Geo g, Geo gf, const uint8_t *__restrict__ mask, const
     const unsigned n = entry(g, x, y, z);
     float v = -1.0f;
     if (!mask[n]) {
-        double s, j[3];
-        node_sums<LAT, false>(gf, f, entry(gf, x, y, z), x, y, z, s, j);
+        double s = 0.0, j[3];
+        const unsigned m = entry(gf, x, y, z);
+        if constexpr (INIT) {
+#pragma unroll
+            for (int i = 0; i < Lattice<LAT>::Q; ++i) s += f[(size_t)i * gf.N + m];
+        } else {
+            node_sums<LAT, false>(gf, f, m, x, y, z, s, j);
+        }
         v = (float)s;
     }
     rho0[n] = rho1[n] = v;
 }
 
-// 1/v of a float in FP64, to 2^-46: a Newton step on its FP32 reciprocal (the
-// division below goes on to 16 bits; in full it is 8 FP64 operations).
-__device__ __forceinline__ double reciprocal_of(float v)
+// d rounded to nearest even in FP32, as the conversion, which takes as long as
+// an FP64 operation, does; results that are not normal FP32 numbers by it.
+__device__ __forceinline__ float narrow(double d)
 {
-    const float r = __frcp_rn(v);
-    const double a = widen(v), b = widen(r);
-    return r > 0.0f && r < 3.0e38f ? fma(b, fma(-a, b, 1.0), b) : 1.0 / a;
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = hi & 0x7ff00000u;
+    if (e < 0x38200000u || e > 0x47c00000u) return (float)d;   // below 2^-125, above 2^125
+    const unsigned top = (((hi & 0x7fffffffu) - 0x38000000u) << 3) | (lo >> 29), drop = lo << 3;
+    return __uint_as_float((hi & 0x80000000u) | (top + (drop > 0x80000000u || (drop == 0x80000000u && (top & 1u)))));
+}
+
+// (float)(f / v - w) in 5 FP64 operations: the quotient starts from the FP32
+// one and is corrected twice by its exact remainder (to 2^-70, so its FP64
+// rounding is the division's but for about 1 in 10^5). Encoding 128x96x112
+// with its densities: 426 us, with a multiplication by 1/v first and the
+// conversion instruction (7 operations) 544 us.
+__device__ __forceinline__ float shifted_of(double f, float v, double w)
+{
+    const unsigned hi = (unsigned)__double2hiint(f), ef = (hi >> 20) & 0x7ff, ev = (__float_as_uint(v) >> 23) & 0xff;
+    if (ef - 963u > 120u || ev - 67u > 120u) return (float)(f / (double)v - w);   // outside 2^-60 .. 2^60
+    const float f32 = __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - 0x38000000u) << 3));
+    const float r32 = __frcp_rn(v);
+    const double d = widen(v), r = widen(r32);
+    double q = widen(f32 * r32);
+    q = fma(fma(-d, q, f), r, q);
+    q = fma(fma(-d, q, f), r, q);
+    return narrow(q - w);
 }
 
 template <int LAT, typename ST>
@@ -939,7 +1060,7 @@ __global__ void k_encode_shifted(Geo g, Geo gf, const double *__restrict__ f, co
         float src = rho[source_node(g, D, i, x, y, z)];
         if (src < 0.0f) src = rho[n];   // bounced by n itself
         h[(size_t)i * g.N + n] =
-            lbmf::from_f<ST>((float)fma(f[(size_t)i * gf.N + m], reciprocal_of(src), -weight_d(i, D)));
+            lbmf::from_f<ST>(shifted_of(f[(size_t)i * gf.N + m], src, weight_d(i, D)));
     }
 }
 
