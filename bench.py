@@ -46,11 +46,16 @@ ALG_BYTES_PER_LU = {  # populations read once and written once per lattice updat
     (1, "bf16s"): 2 * 27 * 2 + 8,
     (0, "bf16s"): 2 * 9 * 2 + 8,
 }
-# FP64 flops per node executed by the collide kernel (D3Q27), counted from
-# the source: two stencil rings 244 (13 neighbour-pair differences of two
-# fields, 54 signed adds, 42 for the weights, per ring), force 15, Phi 9,
-# 1/rho 1, product-form factors 54, partial products 78, collision 81.
-COLLIDE_FP64_FLOPS_PER_NODE = 482
+# FP64 flops per node executed by the D3Q27 collision kernel (k_force_sweep3
+# with its collision), counted from the source: force sums of two fields 98
+# (per field: x sums 12 with the tile's halo rows, y sums 14, z sums 23), force
+# 11, Phi 3, 1/rho and its factor 3, product-form factors 54, partial products
+# 26, collision 135; at relaxation time 1, where the equilibrium and the
+# populations drop out, the last three are 33, 12 and 27.
+def collide_fp64_flops(tau: float) -> int:
+    return 187 if tau == 1.0 else 330
+
+
 FP64_PEAK_TFLOPS = 1.25   # GB300 nominal FP64 rate (context; the roofline uses the live probe)
 
 
@@ -70,18 +75,18 @@ def fp64_peak():
 # tile rows, fused-step form); each entry records the SHA-256 prefix of the fused kernel's
 # source it was taken on, and is not used once that source has changed.
 MEASURED_TRAFFIC = {
-    # k_step_f32_wstma, 32 x 8 tiles, chunk 208 (one 208-plane and one
-    # 48-plane chunk per column, as at full size), on the impact scaled to
-    # 192x192x256: 1113.8 + 968.3 MB for 9,437,184 nodes
+    # k_step_f32_wstma, 32 x 8 tiles, chunk 247 (one 247-plane and one
+    # 9-plane chunk per column, as at full size), on the impact scaled to
+    # 192x192x256: 1118.3 + 965.5 MB for 9,437,184 nodes
     # (profiles/k_step_f32_wstma_d3q27_impact_192x192x256.md)
     ("d3q27_impact_384x384x256_pr_tr0.5", "f32", 8, 4): {
-        "bytes_per_node": 220.62, "src_sha": "7afd52481196669b"},
+        "bytes_per_node": 220.81, "src_sha": "f6d58c9291f8e24e"},
     # k_step_shifted_tmtma (FP16-shifted, Tensor Memory with TMA-staged
-    # planes), 32 x 8 tiles, chunk 224, on the same scaled impact: 585.6 +
-    # 502.3 MB for 9,437,184 nodes
+    # planes), 32 x 8 tiles, chunk 208, on the same scaled impact: 586.6 +
+    # 500.7 MB for 9,437,184 nodes
     # (profiles/k_step_shifted_tmtma_d3q27_impact_192x192x256.md)
     ("d3q27_impact_384x384x256_pr_tr0.5", "f16s", 8, 5): {
-        "bytes_per_node": 115.28, "src_sha": "7afd52481196669b"},
+        "bytes_per_node": 115.22, "src_sha": "f6d58c9291f8e24e"},
 }
 FUSED_SRC = os.path.join(ROOT, "paper_2112_01975_gb300", "csrc", "lbm_fused_f32_body.cuh")
 
@@ -622,14 +627,14 @@ def main():
                     "chunk": chunk, "tile": f"{tile[0]}x{tile[1]}"}
     else:
         achieved = alg / (ms_collide * 1e-3) / 1e9
-        tflops = COLLIDE_FP64_FLOPS_PER_NODE * nodes / (ms_collide * 1e-3) / 1e12
+        tflops = collide_fp64_flops(w.tau) * nodes / (ms_collide * 1e-3) / 1e12
         p64, p64_src = fp64_peak()
         roofline = {"bound": "alu", "achieved": tflops, "peak": p64,
                     "unit": "TFLOP/s", "frac": tflops / p64,
                     "traffic": None,
-                    "kernel": "k_collide (FP64)",
+                    "kernel": "k_force_sweep3 (FP64 force sweep and collision)",
                     "peak_source": p64_src, "nominal_peak": FP64_PEAK_TFLOPS,
-                    "flops_per_node": COLLIDE_FP64_FLOPS_PER_NODE,
+                    "flops_per_node": collide_fp64_flops(w.tau),
                     "ms_per_launch": ms_collide, "ms_moments_kernel": ms_macro,
                     "hbm_achieved_gbs": achieved, "hbm_frac": achieved / peak}
 
@@ -663,10 +668,10 @@ def main():
         ms64, _ = timed_steps(h, stream, k64, dist, local)
         m64, c64 = h.time_kernels(10)
         p64, p64_src = fp64_peak()
-        t64 = COLLIDE_FP64_FLOPS_PER_NODE * nodes / (c64 * 1e-3) / 1e12
+        t64 = collide_fp64_flops(w.tau) * nodes / (c64 * 1e-3) / 1e12
         f64 = {"value": nodes * k64 * world / (ms64 * 1e-3) / 1e6, "unit": "MLUPS",
                "steps": k64, "ms_per_step": ms64 / k64,
-               "roofline": {"bound": "alu", "kernel": "k_collide (FP64)",
+               "roofline": {"bound": "alu", "kernel": "k_force_sweep3 (FP64 force sweep and collision)",
                             "achieved": t64, "peak": p64, "unit": "TFLOP/s", "frac": t64 / p64,
                             "peak_source": p64_src, "nominal_peak": FP64_PEAK_TFLOPS,
                             "ms_per_launch": c64, "ms_moments_kernel": m64}}

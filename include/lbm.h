@@ -273,8 +273,8 @@ int lbm_time_kernels(lbm_handle h, int64_t n, double *ms);
  * fused FP32 step, >= 1. A tuning knob: results do not depend on it. Until
  * the form, tile or chunk is set or tuned, a D3Q27 handle takes the form and
  * the chunk that suit its lattice; once one of them is set, the others are
- * the plain form's (LBM_FUSED_PLAIN, 8 rows, chunk 16). D2Q9 steps, which march along nothing, take
- * it and run the same. */
+ * the plain form's (LBM_FUSED_PLAIN, 8 rows, chunk 16). D2Q9 steps, which
+ * march along nothing, take it and run the same. */
 int lbm_set_chunk(lbm_handle h, int chunk);
 
 /* Pick the chunk of the fused FP32 step by timing candidates (4 to 128
@@ -287,8 +287,8 @@ int lbm_set_chunk(lbm_handle h, int chunk);
  * LBM_F32 storage it also picks the form of the step
  * (lbm_set_fused_variant), and for D3Q27 the tile height, 8 or 7
  * rows of 32 nodes (7 rows fill every SM with two CTAs in one wave where 8
- * rows leave some SMs with one, e.g. at 128^3); the shifted storages and
- * batches keep the plain form with 8 rows. Forms, tiles and chunks
+ * rows leave some SMs with one, e.g. at 128^3); the shifted storages keep
+ * 8 rows. Forms, tiles and chunks
  * change the work split only: results are bitwise the same. Synchronising;
  * allocates and frees one state-sized buffer; on failure the handle keeps
  * the form, tile and chunk it had. */

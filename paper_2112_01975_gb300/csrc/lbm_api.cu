@@ -42,7 +42,6 @@ struct lbm_ctx {
     double t_over_tc, tau;
     std::vector<uint8_t> mask_host, zsolid_host;
     bool any_solid = false;
-    int *walls = nullptr;   // D3Q27 reduced storage with solids: GeoF::wplane and GeoF::walls
     int sms = 148;         // SMs of the device
     int sweep_chunk = 16;  // planes per block of the D3Q27 force sweep (FP64 kernels); 0: direct sums
     int device;
@@ -54,7 +53,7 @@ struct lbm_ctx {
     void *fv[2] = {nullptr, nullptr};   // population buffers (double, float or 16-bit)
     float *rs[2] = {nullptr, nullptr};  // shifted storage: source densities of buffer k
     double2 *rp = nullptr;
-    double *u = nullptr, *gflux = nullptr, *partial = nullptr, *sums = nullptr;
+    double *u = nullptr, *gflux = nullptr /* D3Q27 reduced storage: the wall bits */, *partial = nullptr, *sums = nullptr;
     uint8_t *mask = nullptr;
     int *status = nullptr;
     int cur = 0;
@@ -337,8 +336,9 @@ void leave_auto_form(lbm_ctx *h)
     drop_graphs(h);  // the captured graph holds the chosen form
 }
 
-// The wall bits of the planes within one of a solid node, in an allocation of
-// the handle's own (4 bytes per node of those planes and 8 per plane).
+// The wall bits of the planes within one of a solid node (4 bytes per node of
+// those planes and 8 per plane of the lattice), in the region of rho u_a^3 (24
+// bytes per node), which reduced storage does not use.
 int make_wall_bits(lbm_ctx *h)
 {
     if (h->lattice != LBM_D3Q27 || h->storage == LBM_F64 || !h->any_solid) return LBM_OK;
@@ -354,22 +354,20 @@ int make_wall_bits(lbm_ctx *h)
     } catch (const std::bad_alloc &) {
         return fail(h, LBM_ENOMEM, "no host memory for the wall planes");
     }
-    const size_t head = align_up(sizeof(int) * 2 * g.nz), bits = sizeof(unsigned) * planes.size() * g.px * g.ny;
-    if (!h->walls && cudaMalloc(&h->walls, head + bits) != cudaSuccess) {
-        cudaGetLastError();
-        h->walls = nullptr;
-        return fail(h, LBM_ENOMEM, "cudaMalloc(%zu) for the wall bits failed", head + bits);
-    }
-    unsigned *const w = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(h->walls) + head);
-    CU(h, cudaMemcpyAsync(h->walls, table.data(), sizeof(int) * g.nz, cudaMemcpyHostToDevice, h->stream));
-    CU(h, cudaMemcpyAsync(h->walls + g.nz, planes.data(), sizeof(int) * planes.size(), cudaMemcpyHostToDevice,
+    const size_t head = align_up(sizeof(int) * 2 * g.nz);
+    if (head + sizeof(unsigned) * planes.size() * g.px * g.ny > sizeof(double) * 3 * g.N)
+        return fail(h, LBM_EINVAL, "no room for the wall bits");   // not for any lattice of 5 or more nodes a side
+    int *const walls = reinterpret_cast<int *>(h->gflux);
+    unsigned *const w = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(walls) + head);
+    CU(h, cudaMemcpyAsync(walls, table.data(), sizeof(int) * g.nz, cudaMemcpyHostToDevice, h->stream));
+    CU(h, cudaMemcpyAsync(walls + g.nz, planes.data(), sizeof(int) * planes.size(), cudaMemcpyHostToDevice,
                           h->stream));
     dim3 gr = node_grid(g);
     gr.z = (unsigned)planes.size();
-    lbmk::k_wall_bits<<<gr, node_block(g), 0, h->stream>>>(g, h->mask, h->walls + g.nz, w);
+    lbmk::k_wall_bits<<<gr, node_block(g), 0, h->stream>>>(g, h->mask, walls + g.nz, w);
     CU(h, cudaGetLastError());
     CU(h, cudaStreamSynchronize(h->stream));   // before the host vectors go
-    h->geof.wplane = h->walls;
+    h->geof.wplane = walls;
     h->geof.walls = w;
     return LBM_OK;
 }
@@ -856,7 +854,7 @@ int launch_step(lbm_ctx *h, cudaStream_t s, int *nk)
         const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
         const double *src = f64(h, h->cur);
         double *dst = f64(h, h->cur ^ 1);
-        lbmpdl::launch_step(overlap64(h), lbmk::k_macro<LAT, const double *>, gr, bl, 0, s, h->geo, h->phys, h->mask, src, h->rp,
+        lbmpdl::launch_step(overlap64(h), lbmk::k_macro<LAT, true, const double *>, gr, bl, 0, s, h->geo, h->phys, h->mask, src, h->rp,
                             h->u, h->gflux, h->status);
         launch_collide64<LAT>(h, s, src, dst);
         *nk = 2;
@@ -1008,13 +1006,13 @@ void with_pops(const lbm_ctx *h, int k, const Fn &fn)
     }
 }
 
-// Side fields (rho, s psi), u and rho u_a^3 of the current state.
+// Side fields (rho, s psi) and u of the current state.
 template <int LAT>
 void launch_macro(lbm_ctx *h)
 {
     with_pops(h, h->cur, [&](auto f) {
-        lbmk::k_macro<LAT><<<node_grid(h->geo), node_block(h->geo), 0, h->stream>>>(
-            h->geo, h->phys, h->mask, f, h->rp, h->u, h->gflux, h->status);
+        lbmk::k_macro<LAT, false><<<node_grid(h->geo), node_block(h->geo), 0, h->stream>>>(
+            h->geo, h->phys, h->mask, f, h->rp, h->u, nullptr, h->status);
     });
 }
 
@@ -1051,7 +1049,7 @@ int launch_init(lbm_ctx *h, const double *rho0, const double *u0)
     const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
     // side fields first: the initial force needs rho and s psi of every node
     lbmk::k_fill_solid<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, h->u,
-                                                      h->gflux);
+                                                      h->storage == LBM_F64 ? h->gflux : nullptr);
     lbmk::k_init_density<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, rho0, h->rp);
     h->launches += 3;
     if (shifted(h->storage)) {
@@ -1078,7 +1076,7 @@ int launch_fill_solid(lbm_ctx *h)
 {
     const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
     lbmk::k_fill_solid<LAT><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, h->rp, h->u,
-                                                      h->gflux);
+                                                      h->storage == LBM_F64 ? h->gflux : nullptr);
     CU(h, cudaGetLastError());
     h->launches += 1;
     return LBM_OK;
@@ -2063,10 +2061,10 @@ int lbm_time_kernels(lbm_handle h, int64_t n, double *ms)
             const double *src = f64(h, h->cur);
             double *dst = f64(h, h->cur ^ 1);
             if (h->lattice == LBM_D2Q9)
-                lbmk::k_macro<0><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, h->rp,
+                lbmk::k_macro<0, true><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, h->rp,
                                                            h->u, h->gflux, h->status);
             else
-                lbmk::k_macro<1><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, h->rp,
+                lbmk::k_macro<1, true><<<gr, bl, 0, h->stream>>>(h->geo, h->phys, h->mask, src, h->rp,
                                                            h->u, h->gflux, h->status);
             CU(h, cudaEventRecord(ev[3 * k + 1], h->stream));
             if (h->lattice == LBM_D2Q9) launch_collide64<0>(h, h->stream, src, dst);
@@ -2260,7 +2258,6 @@ void lbm_destroy(lbm_handle h)
     drop_graphs(h);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->owns_base && h->base) cudaFree(h->base);
-    if (h->walls) cudaFree(h->walls);
     if (h->bn) cudaFree(h->bn);
     if (h->bmask) cudaFree(h->bmask);
     if (h->bq) cudaFree(h->bq);

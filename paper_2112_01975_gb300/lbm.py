@@ -314,10 +314,9 @@ class LBM:
         self._check(_lib.lbm_set_chunk(self._h, int(chunk)))
 
     def autotune(self) -> int:
-        """Time the fused step's chunk candidates (and, for FP32, its three
-        forms and, for D3Q27, the 8- and 7-row tiles) on the current state
-        (which is restored) and keep the fastest; returns the chunk (0 for
-        FP64)."""
+        """Time the D3Q27 fused step's forms, tile heights and chunks on the
+        current state (which is restored) and keep the fastest; returns the
+        chunk (0 for FP64; D2Q9 has one form and times nothing)."""
         c = C.c_int()
         self._check(_lib.lbm_autotune(self._h, C.byref(c)))
         return c.value
@@ -354,7 +353,8 @@ class LBM:
 
 
 class Batch:
-    """Several FP32 lattices of one type advanced together (lbm_batch_*)."""
+    """Several lattices of one type and reduced storage advanced together
+    (lbm_batch_*)."""
 
     def __init__(self, members):
         self.members = list(members)
