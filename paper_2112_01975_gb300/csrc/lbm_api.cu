@@ -418,8 +418,11 @@ int ensure_memory(lbm_ctx *h)
     {   // planes of the fused step's march axis (z; the 2D y axis for D2Q9) that hold a solid
         const size_t plane = (size_t)h->geof.nx * h->geof.ny;
         h->zsolid_host.assign(h->geof.nz, 0);
-        for (size_t n = 0; n < h->geo.M; ++n)
-            if (h->mask_host[n]) h->zsolid_host[n / plane] = 1;
+        for (int z = 0; z < h->geof.nz; ++z) {
+            uint8_t any = 0;
+            for (size_t n = 0; n < plane; ++n) any |= h->mask_host[z * plane + n];
+            h->zsolid_host[z] = any != 0;
+        }
         CU(h, cudaMemcpyAsync(const_cast<uint8_t *>(h->geof.zsolid), h->zsolid_host.data(), h->geof.nz,
                               cudaMemcpyHostToDevice, h->stream));
     }
