@@ -276,9 +276,10 @@ void make_tensor_maps(lbm_ctx *h);
 // 1.31 times as long per plane as one alone (measured: 5.4 against 4.1 us,
 // shifted storage at 128^3). The last, shorter chunk of each column fills the
 // SMs that the whole ones leave. Measured, TMA-staged forms, the choice here
-// against the best chunk of a scan: FP32 64^3 24.8 us (chunk 7; 8: 26.6),
-// 128^3 110.8 (56; 64: 122.7, 16: 145), 160^3 200 (108; 54: 205), 256^3 786
-// (223; 64: 828); FP16-shifted 128^3 177 (29; 32: 192), 256^3 1161 (223).
+// against others: FP32 64^3 22.9 us (chunk 7; 8: 24.2), 128^3 96.6 (56; 64:
+// 102.9, 16: 125), 160^3 171 (108; 54: 176), 256^3 683 (223; 64: 702);
+// FP16-shifted 128^3 161 (29; 32: 173), 256^3 1059 (223; 64: 1139). Furthest
+// from the best of a scan: 97x61x75 FP32 51.1 (47.5).
 int best_chunk(const GeoF &g, int rows, int sms, int resident)
 {
     const long long tiles = (long long)((g.nx + 31) / 32) * ((g.ny + rows - 1) / rows);
@@ -302,14 +303,16 @@ constexpr int kDefaultChunk3 = 16;
 // Form and chunk of a D3Q27 handle of reduced storage that the caller has
 // left open: with tensor maps the TMA-staged form of the storage, the
 // fastest of the forms at every size measured, each at its best chunk (FP32
-// 64^3 25 us against 29 for the next, 128^3 111 against 160, 256^3 786
-// against 1177; FP16-shifted 128^3 177 against 203, 256^3 1161 against
-// 1404). The Tensor Memory form without tensor maps, where a column of the
-// halo lies in no box (box_pos; 153 x 145 x 131 FP32: 215 us against 290) and,
+// 64^3 22.9 us against 32.7 for the Tensor Memory form, 128^3 97 against 149,
+// 256^3 683 against 1085; FP16-shifted 128^3 161 against 184, 256^3 1059
+// against 1321). The Tensor Memory form without tensor maps, where a column of the
+// halo lies in no box (box_pos; 153 x 145 x 131 FP32: 205 us, before faster
+// reciprocals 215 against 290) and,
 // in shifted storage, where the tiles hang over the lattice by more than a
 // tenth: there it reads less, while the TMA-staged form's nine copies cost the
-// same (98 x 61 x 75: 71 against 80 us, 45 x 37 x 60: 36 against 41, 150^3: 309
-// against 300; FP32 98 x 61 x 75: 53 against 47). With the FP64 EOS the plain
+// same (98 x 61 x 75: 66 us, 45 x 37 x 60: 33; before faster reciprocals 71
+// against 80 and 36 against 41; 150^3: 319 against 275; FP32 98 x 61 x 75 then
+// 53 against 47). With the FP64 EOS the plain
 // one. The fixed default before, plain at chunk 16: FP32 64^3 62, 128^3 184,
 // 256^3 1208; FP16-shifted 258, 1649.
 void choose_form(lbm_ctx *h)
@@ -1099,8 +1102,8 @@ int launch_reduce(lbm_ctx *h)
 }
 
 // Between two graph replays the GPU idles for 1 to 3 us, as long as a step of a
-// small lattice (64^2 FP32: 4.3 us a step with graphs of two steps, 2.9 with
-// 16, 2.8 with 32). Sequences of at least twice that on lattices whose step is
+// small lattice (64^2 FP32: 4.3 us a step with graphs of two steps, 2.6 with
+// 16, and 32 gain 3 % on that). Sequences of at least twice that on lattices whose step is
 // short (under about 50 us) replay graphs of kLongSteps steps.
 constexpr int kLongSteps = 16;
 constexpr unsigned kLongNodes = 1u << 20;
