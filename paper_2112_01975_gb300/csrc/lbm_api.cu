@@ -511,13 +511,11 @@ void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
     if constexpr (LAT == 1) {
         const int chunk = h->sweep_chunk;
         if (chunk == 0) {
-            lbmpdl::launch_step(false, lbmk::k_force_direct3<Body>, node_grid(g), node_block(g), 0, s, g, h->phys,
-                                h->rp, body);
+            lbmk::k_force_direct3<Body><<<node_grid(g), node_block(g), 0, s>>>(g, h->phys, h->rp, body);
             return;
         }
         const dim3 grid(tx, (g.ny + lbmk::SWY - 1) / lbmk::SWY, (g.nz + chunk - 1) / chunk);
-        lbmpdl::launch_step(false, lbmk::k_force_sweep3<Body>, grid, lbmk::SWX * lbmk::SWY, 0, s, g, h->phys, h->rp, chunk,
-                            body);
+        lbmk::k_force_sweep3<Body><<<grid, lbmk::SWX * lbmk::SWY, 0, s>>>(g, h->phys, h->rp, chunk, body);
     } else if (tx * ((g.ny + 7) / 8) < h->sms) {
         lbmpdl::launch_step(overlap64(h), lbmk::k_force_sweep2<2, 4, Body>, dim3(tx, (g.ny + 1) / 2), 128, 0, s, g, h->phys, h->rp,
                             body);

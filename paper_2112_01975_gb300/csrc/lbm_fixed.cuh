@@ -61,7 +61,7 @@ __device__ __forceinline__ long long shift_down(unsigned long long v, int k)
 // Node n = (x, y, z): q[i] 2^e2 = population i. skip: nothing is formed (the
 // populations have been requested by then, beside what `skip` waits for).
 template <int LAT>
-__device__ __forceinline__ bool fixed_pops(const Geo &g, const double *__restrict__ f, unsigned n, int, int, int,
+__device__ __forceinline__ bool fixed_pops(const Geo &g, const double *f, unsigned n, int, int, int,
                                            long long *q, int &e2, bool skip)
 {
     constexpr int Q = Lattice<LAT>::Q;
@@ -86,7 +86,7 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const double *__restric
 }
 
 template <int LAT>
-__device__ __forceinline__ bool fixed_pops(const Geo &g, const float *__restrict__ f, unsigned n, int, int, int,
+__device__ __forceinline__ bool fixed_pops(const Geo &g, const float *f, unsigned n, int, int, int,
                                            long long *q, int &e2, bool skip)
 {
     constexpr int Q = Lattice<LAT>::Q;

@@ -293,8 +293,6 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
         off[k] = (unsigned)wrap_any((int)blockIdx.x * SWX - 2 + hc[k], g.nx) +
                  (unsigned)g.px * (unsigned)wrap_any((int)blockIdx.y * SWY - 2 + hr[k], g.ny);
     }
-    lbmpdl::step_trigger();
-    lbmpdl::step_wait();
     int zq = z0 - 2 < 0 ? z0 - 2 + g.nz : z0 - 2;
     double2 v0 = rp[off[0] + plane * (unsigned)zq], v1 = two ? rp[off[1] + plane * (unsigned)zq] : v0;
     // sums under way, per field (|psi|, rho) and component, after plane q:
@@ -361,8 +359,6 @@ template <typename Body>
 __global__ void __launch_bounds__(128)
 k_force_direct3(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
 {
-    lbmpdl::step_trigger();
-    lbmpdl::step_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -409,7 +405,7 @@ k_force_direct3(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
 // instructions, so the tile with fewer of them per warp on more SMs wins.
 template <int ROWS, int NW, typename Body>
 __global__ void __launch_bounds__(32 * NW)
-k_force_sweep2(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
+k_force_sweep2(Geo g, Phys p, const double2 *rp, Body body)
 {
     __shared__ SweepSmem sm;
     static_assert(ROWS <= SWY && ROWS <= NW, "a warp per row of the tile");

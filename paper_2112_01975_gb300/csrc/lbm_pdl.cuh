@@ -9,6 +9,13 @@
 // successor start as soon as all its own blocks have (step_trigger()).
 // Launched any other way, or with `overlap` false, step_wait() does not wait.
 //
+// So the kernel is resident while what it will read is still written: that
+// data is not read-only for the kernel's lifetime, and its loads are plain
+// ones, through pointers that are neither __ldg's nor const __restrict__ (the
+// compiler may take those through the non-coherent path, or above the
+// wait). Masks, wall bits, tensor maps and work items, which no step writes,
+// may be read either way and before the wait.
+//
 // Blocks that wait also take up room: a successor that fits beside its
 // predecessor is handed out while SMs are unevenly busy and stays that way.
 // Measured (us a step, with and without): D2Q9 FP32 64^2 2.82 / 2.92, 128^2

@@ -74,9 +74,8 @@ __device__ __forceinline__ void halo2(int k, int &r, int &c)
 
 template <bool MASK, typename ST, bool E64, bool REST>
 __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint8_t *__restrict__ mask,
-                                       const ST *__restrict__ f, ST *__restrict__ fout,
-                                       int *__restrict__ status, int bx, int by, Shared2 &sm,
-                                       const float *__restrict__ rho_src, float *__restrict__ rho_dst)
+                                       const ST *f, ST *__restrict__ fout, int *__restrict__ status, int bx,
+                                       int by, Shared2 &sm, const float *rho_src, float *__restrict__ rho_dst)
 {
     constexpr bool SHIFT = IsShifted<ST>::value;
     using L = LatF<0>;
@@ -105,15 +104,15 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
             float src[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                src[i] = __ldg(rho_src + ((unsigned)X[L::cx(i) + 1] + (unsigned)g.px * (unsigned)Y[L::cz(i) + 1]));
+                src[i] = rho_src[(unsigned)X[L::cx(i) + 1] + (unsigned)g.px * (unsigned)Y[L::cz(i) + 1]];
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const float own = MASK && src[i] < 0.0f ? src[Q / 2] : src[i];
-                fi[u][i] = (weight_f<0>(i) + to_f(__ldg(f + (i * N + n)))) * own;
+                fi[u][i] = (weight_f<0>(i) + to_f(f[i * N + n])) * own;
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) fi[u][i] = to_f(__ldg(f + (i * N + n)));
+            for (int i = 0; i < Q; ++i) fi[u][i] = to_f(f[i * N + n]);
         }
     }
     NodeM own = {};
@@ -175,8 +174,8 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
 
 template <bool MASK, typename ST, bool E64, bool REST>
 __global__ void __launch_bounds__(NT)
-k_step2d(GeoF g, PhysF p, const uint8_t *__restrict__ mask, const ST *__restrict__ f, ST *__restrict__ fout,
-         const float *__restrict__ rho_src, float *__restrict__ rho_dst, int *__restrict__ status)
+k_step2d(GeoF g, PhysF p, const uint8_t *__restrict__ mask, const ST *f, ST *__restrict__ fout,
+         const float *rho_src, float *__restrict__ rho_dst, int *__restrict__ status)
 {
     __shared__ Shared2 sm;
     lbmpdl::step_trigger();

@@ -34,7 +34,8 @@ void launch_bs(const lbmf::BatchT &batch, const lbmf::WorkItem *items, int n_ite
     static std::atomic<unsigned long long> done{0};   // devices whose kernel is opted in
     const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
     opt_in(lbmf::k_step_shifted_tmtma_batch<ST, MASK, REST>, bytes, done);
-    lbmpdl::launch_step(false, lbmf::k_step_shifted_tmtma_batch<ST, MASK, REST>, n_items, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s, batch, items);
+    lbmf::k_step_shifted_tmtma_batch<ST, MASK, REST>
+        <<<n_items, lbmf::LatF<1>::TX * lbmf::LatF<1>::TY, bytes, s>>>(batch, items);
 }
 
 template <bool MASK, int EOSK, bool REST>
@@ -80,7 +81,8 @@ void launch_s(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     const int bytes = (int)sizeof(lbmf::SharedSWT<1, ST>);
     opt_in(lbmf::k_step_shifted_wstma<1, ST, MASK>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
-    lbmpdl::launch_step(false, lbmf::k_step_shifted_wstma<1, ST, MASK>, grid, 2 * L::TX * L::TY, bytes, s, g, p, mask, maps, src, dst, rho_src, rho_dst, status);
+    lbmf::k_step_shifted_wstma<1, ST, MASK>
+        <<<grid, 2 * L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst, rho_src, rho_dst, status);
 }
 
 template <typename ST, bool MASK, bool REST>
@@ -92,7 +94,8 @@ void launch_t(const lbmf::GeoF &g, const lbmf::PhysF &p, const uint8_t *mask, co
     const int bytes = (int)sizeof(lbmf::SharedSB<1, ST>);
     opt_in(lbmf::k_step_shifted_tmtma<1, ST, MASK, REST>, bytes, done);
     const dim3 grid((g.nx + L::TX - 1) / L::TX, (g.ny + L::TY - 1) / L::TY, (g.nz + g.chunk - 1) / g.chunk);
-    lbmpdl::launch_step(false, lbmf::k_step_shifted_tmtma<1, ST, MASK, REST>, grid, L::TX * L::TY, bytes, s, g, p, mask, maps, src, dst, rho_src, rho_dst, status);
+    lbmf::k_step_shifted_tmtma<1, ST, MASK, REST>
+        <<<grid, L::TX * L::TY, bytes, s>>>(g, p, mask, maps, src, dst, rho_src, rho_dst, status);
 }
 
 }  // namespace
