@@ -130,7 +130,7 @@ __device__ __forceinline__ void tile2d(const GeoF &g, const PhysF &p, const uint
         } else {
             m = node_moments<0, E64>(p, fi[u], ring1);
         }
-        const float psi = E64 && !solid[u] ? m.psi64 : root_f(fabsf(m.d));
+        const float psi = E64 && !solid[u] ? m.psi64 : sqrtf(fabsf(m.d));
         sm.rp[r][c] = f2(m.rho, psi);
         if (ring1) {
             sm.g[0][r - 1][c - 1] = m.gx;
