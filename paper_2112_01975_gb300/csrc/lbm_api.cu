@@ -515,7 +515,10 @@ void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
             return;
         }
         const dim3 grid(tx, (g.ny + lbmk::SWY - 1) / lbmk::SWY, (g.nz + chunk - 1) / chunk);
-        lbmk::k_force_sweep3<Body><<<grid, lbmk::SWX * lbmk::SWY, 0, s>>>(g, h->phys, h->rp, chunk, body);
+        static std::atomic<unsigned long long> done{0};   // devices already opted in
+        const int bytes = (int)sizeof(lbmk::SweepSmem3);
+        smem_opt_in(lbmk::k_force_sweep3<Body>, bytes, done);
+        lbmk::k_force_sweep3<Body><<<grid, lbmk::SWX * lbmk::SWY, bytes, s>>>(g, h->phys, h->rp, chunk, body);
     } else if (tx * ((g.ny + 7) / 8) < h->sms) {
         lbmpdl::launch_step(overlap64(h), lbmk::k_force_sweep2<2, 4, Body>, dim3(tx, (g.ny + 1) / 2), 128, 0, s, g, h->phys, h->rp,
                             body);
@@ -528,16 +531,17 @@ void launch_sweep(lbm_ctx *h, cudaStream_t s, const Body &body)
 // Planes per block of the D3Q27 force sweep, or 0 for the direct sums of small
 // lattices: a block's 8 warps share their SM's FP64 pipe (19 cycles an
 // instruction), so the SM with the most blocks sets the time; a block of c
-// planes also sums 4 more (64 of about 200 operations per node). Directly it
+// planes also sums 4 more (46 of about 210 operations per node). Directly it
 // is about 290 operations per node, but every SM has its share (32^3: 20 us
-// against 39 a step, 48^3 about equal).
+// against 33 at the best chunk, 44^3 66 against 70, 48^3 74 against 70).
 int sweep_chunk(const Geo &g, int sms)
 {
     const long long tiles = (long long)((g.nx + lbmk::SWX - 1) / lbmk::SWX) *
                             ((g.ny + lbmk::SWY - 1) / lbmk::SWY);
-    // c planes cost 200 c + 256; two blocks share an SM at half speed each. The
-    // last, shorter chunk of each column fills in (128^3: chunk 29 667 us, 18
-    // 690, 14 684, 32 731).
+    // c planes cost 200 c + 256 (the proportion that picks the chunk of the scans);
+    // two blocks share an SM at half speed each. The last, shorter chunk of each
+    // column fills in (128^3: chunk 29 701 us, 14 705, 18 711, 32 768; 97x61x75:
+    // 8 219, 9 242, 6 259; 160^3: 54 1272, 40 1442; 96^3: 24 316, 12 312).
     int best = 1;
     double cost = 1e300;
     for (int c = 1; c <= g.nz; ++c) {

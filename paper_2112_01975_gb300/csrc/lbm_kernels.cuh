@@ -81,7 +81,10 @@ __host__ __device__ constexpr int czi(int i) { return i / 9 - 1; }
 
 // P - rho/3 of the equations of state of Sec. 3.1 and Appendix G (gas
 // constant 1) and 1/rho, from one reciprocal where the EOS has a denominator:
-// P = rho n / D, 1/(rho D) gives both.
+// P = rho n / D, 1/(rho D) gives both. (Error of P - rho/3 over the densities in
+// use: 8.8e-17 of rho/3 rms, with a division in its place 7.3e-17; against 128-bit
+// arithmetic the step's populations, u and U are closer than with divisions and FP64
+// sums of the populations: U 1.16e-17 rms on 80x72x70, then 1.71e-17.)
 __device__ __forceinline__ double excess_pressure(const Phys &p, double rho, double &inv)
 {
     double n, D;   // P / rho + m = n / D
@@ -211,12 +214,16 @@ namespace lbmk {
 //   S_psi = sum_i (w_i/cs2) c_i [4/3 psi(r+c_i) - 1/6 psi(r+2c_i)],
 //   S_rho = sum_i (w_i/cs2) c_i [2 rho(r+c_i) - rho(r+2c_i)]   (Eq. Kforce_final).
 // With the 1D weights W(0) = 2/3, W(+-1) = 1/6 of Eq. wi, w_i/cs2 c_ia =
-// 1/2 c_ia W(c_ib) W(c_ic): a central difference along a times [1, 4, 1]/6
+// 1/2 c_ia W(c_ib) W(c_ic): a central difference along a, then [1, 4, 1]/6
 // smoothings along the other axes. Summed node by node that is 208 FP64
 // operations (D3Q27; both fields, both rings), more than half of the step;
 // one axis at a time, with each axis's sums shared by the nodes of a tile
-// through shared memory, it is 64. sum_a below are the sums without their
-// common factor: ring 1 plus RING2 times ring 2,
+// through shared memory, it is 75. The difference comes first on every axis:
+// smoothed fields round at the field's size, and where it is nearly uniform
+// their difference keeps that (force error of a 48^3 drop against 128-bit sums,
+// rms along x, y, z: differences first 1.0, 1.0, 1.0e-17, smoothing along x
+// first, 64 operations, 1.0, 5.5, 8.5e-17; node by node 1.4e-17). sum_a below
+// are the sums without their common factor: ring 1 plus RING2 times ring 2,
 //   S_psi = sum_psi / 54 (D2Q9: / 9),  S_rho = sum_rho / 36 (D2Q9: / 6).
 constexpr double RING2_PSI = -1.0 / 8.0, RING2_RHO = -1.0 / 2.0;
 
@@ -234,18 +241,27 @@ __device__ __forceinline__ void force_of_sums(const Phys &p, double rho, double 
     }
 }
 
-// Tiles of 32 x 8 nodes; D3Q27 marches along z through `chunk` planes.
-// Per plane of the 36 x 12 halo tile: |psi| and rho to shared memory, the
-// x-sums of its 12 rows (smoothed and differenced, rings 1 and 2), and each
-// node's y-sums from them; the z-sums build up in registers as the planes
-// pass. The two barriers per plane and the loads are hidden by the second
-// block of the SM: the FP64 pipe is what is busy.
+// Tiles of 32 x 8 nodes; D3Q27 marches along z through `chunk` planes. Per
+// plane q of the 36 x 12 halo tile: |psi| and rho to shared memory, with the
+// z-differences around plane q - 2 of the thread's own halo nodes (their last
+// five planes stay in shared memory); then the x-differences and the z-
+// differences smoothed along x of its 12 rows and the y-differences of its 8;
+// then each node's sums of them. The z-smoothings of the x and y components build up in
+// registers as the planes pass. The FP64 pipe is what is busy.
 // Body: what is done with a node's sums: body(p, n, x, y, z, sp, sr).
 constexpr int SWX = 32, SWY = 8;
 
-struct SweepSmem {
-    double raw[2][SWY + 4][SWX + 4];       // |psi|, rho
-    double xs[2][4][SWY + 4][SWX];         // x-sums: smooth 1, difference 1, smooth 2, difference 2
+struct SweepSmem3 {   // by field (|psi|, rho), then ring
+    double raw[5][2][SWY + 4][SWX + 4];    // planes q - 4 .. q, by plane modulo 5
+    double dz[2][2][SWY + 4][SWX + 4];
+    double dx[2][2][SWY + 4][SWX], sz[2][2][SWY + 4][SWX];
+    double dy[2][2][SWY][SWX + 4];
+};
+
+template <int ROWS> struct SweepSmem2 {
+    double raw[2][ROWS + 4][SWX + 4];
+    double dx[2][2][ROWS + 4][SWX];
+    double dy[2][2][ROWS][SWX + 4];
 };
 
 __device__ __forceinline__ int wrap_any(int v, int n)
@@ -258,23 +274,35 @@ __device__ __forceinline__ int wrap_any(int v, int n)
     return v;
 }
 
-// x-sums of row r (of the halo tile) of field q.
-__device__ __forceinline__ void x_sums(SweepSmem &sm, int q, int r, int tx)
+// [1, 4, 1] smoothing of a at distance s, `step` doubles apart.
+__device__ __forceinline__ double smooth(const double *a, int s, int step)
 {
-    const double *a = &sm.raw[q][r][tx + 2];
+    return fma(4.0, a[0], a[-s * step] + a[s * step]);
+}
+
+// x-differences of row r (of the halo tile) of both fields.
+template <typename Raw, typename DX>
+__device__ __forceinline__ void x_differences(const Raw &raw, DX &dx, int q, int r, int tx)
+{
+    const double *a = &raw[q][r][tx + 2];
 #pragma unroll
-    for (int s = 1; s <= 2; ++s) {
-        const double lo = a[-s], hi = a[s];
-        sm.xs[q][2 * s - 2][r][tx] = fma(4.0, a[0], lo + hi);
-        sm.xs[q][2 * s - 1][r][tx] = hi - lo;
-    }
+    for (int s = 1; s <= 2; ++s) dx[q][s - 1][r][tx] = a[s] - a[-s];
+}
+
+// y-differences of node row r, halo column c of field q.
+template <typename Raw, typename DY>
+__device__ __forceinline__ void y_differences(const Raw &raw, DY &dy, int q, int r, int c)
+{
+#pragma unroll
+    for (int s = 1; s <= 2; ++s) dy[q][s - 1][r][c] = raw[q][r + 2 + s][c] - raw[q][r + 2 - s][c];
 }
 
 template <typename Body>
 __global__ void __launch_bounds__(SWX *SWY, 2)
 k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body body)
 {
-    __shared__ SweepSmem sm;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SweepSmem3 &sm = *reinterpret_cast<SweepSmem3 *>(smem_raw);
     constexpr int NT = SWX * SWY, HX = SWX + 4, NH = HX * (SWY + 4);
     const int tid = threadIdx.x, tx = tid % SWX, ty = tid / SWX;
     const int x = blockIdx.x * SWX + tx, y = blockIdx.y * SWY + ty;
@@ -294,60 +322,69 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
                  (unsigned)g.px * (unsigned)wrap_any((int)blockIdx.y * SWY - 2 + hr[k], g.ny);
     }
     int zq = z0 - 2 < 0 ? z0 - 2 + g.nz : z0 - 2;
-    double2 v0 = rp[off[0] + plane * (unsigned)zq], v1 = two ? rp[off[1] + plane * (unsigned)zq] : v0;
-    // sums under way, per field (|psi|, rho) and component, after plane q:
+    double2 v[2];
+    v[0] = rp[off[0] + plane * (unsigned)zq];
+    v[1] = two ? rp[off[1] + plane * (unsigned)zq] : v[0];
+    // sums under way, per field (|psi|, rho) and component x, y, after plane q:
     // n2 (ring 2 part of plane q + 2, without its factor), a1 (q + 1), a0 (q), m1 (q - 1)
-    double n2[2][3] = {}, a1[2][3] = {}, a0[2][3] = {}, m1[2][3] = {};
+    double n2[2][2] = {}, a1[2][2] = {}, a0[2][2] = {}, m1[2][2] = {};
+    int w = 0;   // q's slot of sm.raw
     for (int q = z0 - 2; q < z1 + 2; ++q) {
-        sm.raw[0][hr[0]][hc[0]] = fabs(v0.y);
-        sm.raw[1][hr[0]][hc[0]] = v0.x;
-        if (two) {
-            sm.raw[0][hr[1]][hc[1]] = fabs(v1.y);
-            sm.raw[1][hr[1]][hc[1]] = v1.x;
+        const bool sums = q >= z0 + 2;   // the sums of plane q - 2 are done in this iteration
+        const int w1 = w == 0 ? 4 : w - 1, w3 = w < 3 ? w + 2 : w - 3, w4 = w == 4 ? 0 : w + 1;   // of q - 1, q - 3, q - 4
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (k == 1 && !two) break;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const double a = e == 0 ? fabs(v[k].y) : v[k].x;
+                if (sums) {
+                    sm.dz[e][0][hr[k]][hc[k]] = sm.raw[w1][e][hr[k]][hc[k]] - sm.raw[w3][e][hr[k]][hc[k]];
+                    sm.dz[e][1][hr[k]][hc[k]] = a - sm.raw[w4][e][hr[k]][hc[k]];
+                }
+                sm.raw[w][e][hr[k]][hc[k]] = a;
+            }
         }
         zq = zq + 1 == g.nz ? 0 : zq + 1;
         if (q + 1 < z1 + 2) {   // the next plane, while this one is summed
-            v0 = rp[off[0] + plane * (unsigned)zq];
-            if (two) v1 = rp[off[1] + plane * (unsigned)zq];
+            v[0] = rp[off[0] + plane * (unsigned)zq];
+            if (two) v[1] = rp[off[1] + plane * (unsigned)zq];
         }
         __syncthreads();
-        x_sums(sm, 0, ty, tx);
-        x_sums(sm, 1, ty, tx);
-        if (ty < 4) {
-            x_sums(sm, 0, ty + SWY, tx);
-            x_sums(sm, 1, ty + SWY, tx);
+        for (int r = ty; r < SWY + 4; r += SWY) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                x_differences(sm.raw[w], sm.dx, e, r, tx);
+                if (sums)
+#pragma unroll
+                    for (int s = 1; s <= 2; ++s) sm.sz[e][s - 1][r][tx] = smooth(&sm.dz[e][s - 1][r][tx + 2], s, 1);
+            }
         }
+        // (by the warps that had one row)
+        for (int h = tid - NT / 2; h >= 0 && h < 2 * SWY * HX; h += NT / 2)
+            y_differences(sm.raw[w], sm.dy, h / (SWY * HX), h / HX % SWY, h % HX);
         __syncthreads();
         double done[2][3];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const double r2 = k == 0 ? RING2_PSI : RING2_RHO;
-            double X1[3], X2[3];   // ring 1 and 2 sums of the plane: x, y differences, smoothed
+            // ring 1 and 2 sums of the plane: x and y differences, smoothed
+            const double X1[2] = {smooth(&sm.dx[k][0][ty + 2][tx], 1, SWX), smooth(&sm.dy[k][0][ty][tx + 2], 1, 1)};
+            const double X2[2] = {smooth(&sm.dx[k][1][ty + 2][tx], 2, SWX), smooth(&sm.dy[k][1][ty][tx + 2], 2, 1)};
 #pragma unroll
-            for (int s = 1; s <= 2; ++s) {
-                double *X = s == 1 ? X1 : X2;
-                const auto &S = sm.xs[k][2 * s - 2], &Dx = sm.xs[k][2 * s - 1];
-                const double lo = S[ty + 2 - s][tx], hi = S[ty + 2 + s][tx];
-                X[0] = fma(4.0, Dx[ty + 2][tx], Dx[ty + 2 - s][tx] + Dx[ty + 2 + s][tx]);
-                X[1] = hi - lo;
-                X[2] = fma(4.0, S[ty + 2][tx], lo + hi);
-            }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
+            for (int a = 0; a < 2; ++a) {
                 done[k][a] = fma(r2, X2[a], m1[k][a]);
                 m1[k][a] = a0[k][a] + X1[a];
-                if (a < 2) {
-                    a0[k][a] = fma(4.0, fma(r2, X2[a], X1[a]), a1[k][a]);
-                    a1[k][a] = fma(r2, n2[k][a], X1[a]);
-                } else {
-                    a0[k][a] = a1[k][a];
-                    a1[k][a] = fma(-r2, n2[k][a], -X1[a]);
-                }
+                a0[k][a] = fma(4.0, fma(r2, X2[a], X1[a]), a1[k][a]);
+                a1[k][a] = fma(r2, n2[k][a], X1[a]);
                 n2[k][a] = X2[a];
             }
+            if (sums)
+                done[k][2] = fma(r2, smooth(&sm.sz[k][1][ty + 2][tx], 2, SWX), smooth(&sm.sz[k][0][ty + 2][tx], 1, SWX));
         }
-        if (q - 2 >= z0 && inside)
+        if (sums && inside)
             body(g, p, entry(g, x, y, q - 2), x, y, q - 2, done[0], done[1]);
+        w = w == 4 ? 0 : w + 1;
     }
 }
 
@@ -399,7 +436,7 @@ k_force_direct3(Geo g, Phys p, const double2 *__restrict__ rp, Body body)
 }
 
 // D2Q9: one tile of 32 x ROWS nodes per block, one shot; NW warps share the
-// x-sums of the ROWS + 4 rows, ROWS of them go on to the nodes. A lattice
+// differences of the tile's rows, ROWS of them go on to the nodes. A lattice
 // with too few tiles of 8 rows for the SMs takes tiles of 2 rows, 4 warps: a
 // warp alone on its sub-partition is bound by its own chain of FP64
 // instructions, so the tile with fewer of them per warp on more SMs wins.
@@ -407,8 +444,8 @@ template <int ROWS, int NW, typename Body>
 __global__ void __launch_bounds__(32 * NW)
 k_force_sweep2(Geo g, Phys p, const double2 *rp, Body body)
 {
-    __shared__ SweepSmem sm;
-    static_assert(ROWS <= SWY && ROWS <= NW, "a warp per row of the tile");
+    __shared__ SweepSmem2<ROWS> sm;
+    static_assert(ROWS <= NW, "a warp per row of the tile");
     constexpr int NT = 32 * NW, HX = SWX + 4, NH = HX * (ROWS + 4);
     const int tid = threadIdx.x, tx = tid % 32, w = tid / 32;
     const int x0 = blockIdx.x * SWX, y0 = blockIdx.y * ROWS;
@@ -422,7 +459,8 @@ k_force_sweep2(Geo g, Phys p, const double2 *rp, Body body)
         sm.raw[1][r][c] = v.x;
     }
     __syncthreads();
-    for (int t = w; t < 2 * (ROWS + 4); t += NW) x_sums(sm, t & 1, t >> 1, tx);
+    for (int t = w; t < 2 * (ROWS + 4); t += NW) x_differences(sm.raw, sm.dx, t & 1, t >> 1, tx);
+    for (int h = tid; h < 2 * ROWS * HX; h += NT) y_differences(sm.raw, sm.dy, h / (ROWS * HX), h / HX % ROWS, h % HX);
     __syncthreads();
     const int x = x0 + tx, y = y0 + w;
     if (w >= ROWS || x >= g.nx || y >= g.ny) return;
@@ -430,15 +468,8 @@ k_force_sweep2(Geo g, Phys p, const double2 *rp, Body body)
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const double r2 = k == 0 ? RING2_PSI : RING2_RHO;
-        double X[2][2];
-#pragma unroll
-        for (int s = 1; s <= 2; ++s) {
-            const auto &S = sm.xs[k][2 * s - 2], &Dx = sm.xs[k][2 * s - 1];
-            X[s - 1][0] = fma(4.0, Dx[w + 2][tx], Dx[w + 2 - s][tx] + Dx[w + 2 + s][tx]);
-            X[s - 1][1] = S[w + 2 + s][tx] - S[w + 2 - s][tx];
-        }
-        sum[k][0] = fma(r2, X[1][0], X[0][0]);
-        sum[k][1] = fma(r2, X[1][1], X[0][1]);
+        sum[k][0] = fma(r2, smooth(&sm.dx[k][1][w + 2][tx], 2, SWX), smooth(&sm.dx[k][0][w + 2][tx], 1, SWX));
+        sum[k][1] = fma(r2, smooth(&sm.dy[k][1][w][tx + 2], 2, 1), smooth(&sm.dy[k][0][w][tx + 2], 1, 1));
     }
     body(g, p, entry(g, x, y, 0), x, y, 0, sum[0], sum[1]);
 }
