@@ -54,8 +54,7 @@ __device__ __forceinline__ double fixed_to_double(long long s, int e2)
 // way in every step).
 __device__ __forceinline__ long long shift_down(unsigned long long v, int k)
 {
-    k = min(k, 63);
-    return (long long)((v + (1ull << (k - 1))) >> k);
+    return k > 63 ? 0 : (long long)((v + (1ull << (k - 1))) >> k);
 }
 
 // Node n = (x, y, z): q[i] 2^e2 = population i. skip: nothing is formed (the
