@@ -4,23 +4,31 @@
 // populations: 53 FP64 additions on D3Q27 for density and momentum alone,
 // each as long as 76 integer issue slots, plus a conversion of the same
 // length per population in 32- and 16-bit storage. Here the populations
-// become 64-bit integers in units of 2^(E - 57), E the exponent of the
-// largest (shifted storage: 2^(E - 56) with E that of the largest source
-// density), so that their sums are exact; one integer-to-double conversion
-// per moment rounds to 53 bits. What a population loses is below 2^-57 of
-// the largest, less than the roundings of a sum in FP64 (2^-53 of the
-// partial sum each): against 80-bit arithmetic, density, u and U of FP64
-// D3Q27 and D2Q9 drops are 1.1 (1 step) to 3 times (200 steps) closer than
-// with FP64 sums.
+// become 64-bit integers, so that their sums are exact; one integer-to-double
+// conversion per moment rounds to 53 bits. With E the exponent of the node's
+// largest population, unit and most that one population loses:
+//   FP64     2^(E - 57)   half a unit (rounded to nearest)
+//   FP32     2^(E - 57)   nothing down to 2^-34 of the largest, below that less
+//                         than a unit (truncated)
+//   shifted  2^(E - 56)   half a unit, and the 2^-60 or less of its source density's
+//                         power of two that the product drops: 1.5 units in all
+// which is less than the roundings of a sum in FP64 (2^-53 of the partial sum
+// each). Against 80-bit arithmetic, density, u and U of FP64 D3Q27 and D2Q9
+// drops are 1.1 (1 step) to 3 times (200 steps) closer than with FP64 sums;
+// against exact sums of FP16 and BF16 D3Q27 populations the density is 2 and
+// the momentum 1.5 to 2 times closer.
 //
 // Populations that are not positive normal numbers of a moderate range
-// (negative ones, infinities and NaN among them) return false: the caller
-// sums those nodes in FP64.
+// (negative ones, infinities and NaN among them), and in shifted storage those
+// of which the largest is below 1/16 or so of a source's density, return
+// false: the caller sums those nodes in FP64.
 #pragma once
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 namespace lbmk {
 
@@ -106,8 +114,11 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const float *f, unsigne
 }
 
 // Shifted storage: (w_i + h_i) rho(r - c_i), the node's own density where the
-// source is solid (density -1). w_i + h_i in units of 2^-57 (h_i split into a
-// multiple of 2^-25 and the rest), times the 31-bit mantissa of the density.
+// source is solid (density -1). w_i + h_i in units of 2^-62 (exact in FP16,
+// whose values are multiples of 2^-24, and down to 2^-54 in BF16), times the
+// 31-bit mantissa of the density. (Units of 2^-55 of the largest source density
+// are as fast, but the density is off by 2.7e-16 rms, in FP64 sums 1.1e-16 and
+// here 0.5e-16, and by up to 2e-13 beside a density 6.6e4 times as large.)
 template <int LAT, typename ST>
 __device__ __forceinline__ bool fixed_pops(const Geo &g, const Shifted<ST> &f, unsigned n, int x, int y, int z,
                                            long long *q, int &e2, bool skip)
@@ -128,24 +139,34 @@ __device__ __forceinline__ bool fixed_pops(const Geo &g, const Shifted<ST> &f, u
     }
     if (skip) return true;
     const unsigned own = s[Q / 2];
+    float largest = 0.0f;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
+        const float w = (float)(W1[cxi(i) + 1] * W1[cyi(i) + 1] * (D == 3 ? W1[czi(i) + 1] : 1.0));
         if (s[i] >> 31) s[i] = own;
         top = max(top, s[i]);
         htop = max(htop, __float_as_uint(h[i]) & 0x7fffffffu);
+        largest = fmaxf(largest, fabsf((w + h[i]) * __uint_as_float(s[i])));
     }
-    const int E = (int)(top >> 23);
-    if (E < 72 || E >= 0xff || htop >= 0x40000000u) return false;   // |h| < 2
-    e2 = E - 127 - 55;
+    const int E = (int)(__float_as_uint(largest) >> 23), Es = (int)(top >> 23);
+    // |h| < 1 keeps w + h and the product within 63 bits; Es >= 255: infinities,
+    // NaN and negative densities
+    if (E < 72 || Es >= 0xff || Es > E + 4 || htop >= 0x3f800000u) return false;
+    e2 = E - 127 - 56;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        constexpr double unit = 144115188075855872.0;   // 2^57
-        const long long w = (long long)(W1[cxi(i) + 1] * W1[cyi(i) + 1] * (D == 3 ? W1[czi(i) + 1] : 1.0) * unit);
-        const float a = h[i] * 33554432.0f, ai = rintf(a);   // 2^25
-        const long long X57 = w + ((long long)(int)ai << 32) + (int)((a - ai) * 4294967296.0f);
+        constexpr double unit = 4611686018427387904.0;   // 2^62
+        long long wh = (long long)(W1[cxi(i) + 1] * W1[cyi(i) + 1] * (D == 3 ? W1[czi(i) + 1] : 1.0) * unit);
+        const float a = h[i] * 1073741824.0f;   // 2^30
+        if constexpr (std::is_same<ST, __half>::value) {
+            wh += (long long)(int)a << 32;
+        } else {
+            const float ai = floorf(a);
+            wh += ((long long)(int)ai << 32) + (unsigned)((a - ai) * 4294967296.0f);
+        }
         const int m = (int)(((s[i] & 0x7fffffu) | 0x800000u) << 7);   // 2^30 <= m < 2^31
-        const long long P = (long long)(int)(X57 >> 32) * m + (long long)__umulhi((unsigned)X57, (unsigned)m);
-        const int k = min(E - (int)(s[i] >> 23), 62);
+        const long long P = (long long)(int)(wh >> 32) * m + (long long)__umulhi((unsigned)wh, (unsigned)m);
+        const int k = min(E + 4 - (int)(s[i] >> 23), 62);
         q[i] = (P + ((1ll << k) >> 1)) >> k;
     }
     return true;
