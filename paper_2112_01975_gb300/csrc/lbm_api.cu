@@ -653,6 +653,28 @@ void launch_fused_e64(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
+// Whether `blocks` blocks of `threads` threads of a kernel leave its successor
+// room for less than a block per SM, going by the blocks of it that an SM holds
+// at once (its registers decide: 4 to 6 of the D2Q9 kernels' instantiations;
+// asked once, the library is built for one architecture). D2Q9 with and without
+// overlap, us a step: FP32, time 1 (6 an SM), 960x200 (4.9 blocks an SM) 5.14 /
+// 5.00, 928x224 (5.3) 5.26 / 5.66; other times (5 an SM), 768x200 (3.9) 4.73 /
+// 4.62, 704x240 (4.3) 4.76 / 5.14; FP16 960x200 6.67 / 6.04, 928x224 6.70 / 7.19
+// and 768x200 5.65 / 5.27, 704x240 5.68 / 6.18.
+template <typename Kern>
+bool leaves_no_room(Kern kernel, long long blocks, int threads, int sms, std::atomic<int> &known)
+{
+    int n = known.load();
+    if (n == 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, 0) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            return false;
+        }
+        known.store(n);
+    }
+    return blocks > (n - 1ll) * sms;
+}
+
 // The D2Q9 step of a reduced storage from population buffer k: one kernel,
 // whatever form, chunk or tile the handle names (lbm_step2d.cuh).
 template <typename ST, bool MASK, bool E64, bool REST>
@@ -660,9 +682,10 @@ void launch_2d_r(lbm_ctx *h, cudaStream_t s, int k)
 {
     const GeoF &g = h->geof;
     const dim3 grid((g.nx + lbmf2::TX - 1) / lbmf2::TX, (g.nz + lbmf2::TY - 1) / lbmf2::TY);
-    // (five blocks per SM are resident: more of them leave a successor no room)
+    static std::atomic<int> known{0};
     const long long blocks = (long long)grid.x * grid.y;
-    const bool overlap = lbmpdl::side_by_side(blocks, h->sms) || blocks > 5 * h->sms;
+    const bool overlap = lbmpdl::side_by_side(blocks, h->sms) ||
+                         leaves_no_room(lbmf2::k_step2d<MASK, ST, E64, REST>, blocks, lbmf2::NT, h->sms, known);
     lbmpdl::launch_step(overlap, lbmf2::k_step2d<MASK, ST, E64, REST>, grid, lbmf2::NT, 0, s, g, h->physf, h->mask,
                         static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]), h->rs[k], h->rs[k ^ 1],
                         h->status);
@@ -1744,12 +1767,19 @@ void launch_batch_plain(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, in
     }
 }
 
+template <typename ST, bool REST>
+void launch_batch_2d_r(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
+{
+    static std::atomic<int> known{0};
+    const bool overlap = leaves_no_room(lbmf2::k_step2d_batch<ST, REST>, n, lbmf2::NT, b->members[0]->sms, known);
+    lbmpdl::launch_step(overlap, lbmf2::k_step2d_batch<ST, REST>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
+}
+
 template <typename ST>
 void launch_batch_2d(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, bool rest, int parity, cudaStream_t s)
 {
-    const bool overlap = n > 5 * b->members[0]->sms;
-    if (rest) lbmpdl::launch_step(overlap, lbmf2::k_step2d_batch<ST, true>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
-    else lbmpdl::launch_step(overlap, lbmf2::k_step2d_batch<ST, false>, n, lbmf2::NT, 0, s, b->d_members[parity], items);
+    if (rest) launch_batch_2d_r<ST, true>(b, items, n, parity, s);
+    else      launch_batch_2d_r<ST, false>(b, items, n, parity, s);
 }
 
 // One step of every member.

@@ -23,7 +23,7 @@
 // 7.9 / 8.3, 96^2 14.9 / 8.5; D3Q27 FP32 TMA-staged (one block per SM) 32^3 9.6 /
 // 10.1, 64^3 19.7 / 20.4, 128^3 105.1 / 105.2; FP16-shifted 32^3 23.3 / 21.3. So
 // it is used where two steps' blocks have an SM each or nearly (side_by_side), where
-// a step's blocks leave no room for the next ones', and not in between.
+// a step's blocks leave no room for the next ones' (leaves_no_room), and not in between.
 #pragma once
 
 #include <cuda_runtime.h>

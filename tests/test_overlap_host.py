@@ -87,3 +87,13 @@ def test_only_waiting_kernels_are_launched_overlapped():
             continue
         for m in re.finditer(r"lbmpdl::launch_step\(([^,]+),\s*(?:\w+::)*(\w+)", t):
             assert m.group(2) in waits, (name, m.group(2))
+
+
+def test_room_is_asked_of_the_kernel():
+    """Whether a D2Q9 step leaves its successor room follows from the blocks that
+    an SM holds of that kernel, not from a number in the source."""
+    api = sources()["lbm_api.cu"]
+    assert "cudaOccupancyMaxActiveBlocksPerMultiprocessor" in api
+    for fn in ("launch_2d_r", "launch_batch_2d_r"):
+        body = block(api, api.index("void %s(" % fn))
+        assert "leaves_no_room(lbmf2::k_step2d" in body and not re.search(r"\d\s*\*\s*[\w>\[\].-]*sms", body), body
