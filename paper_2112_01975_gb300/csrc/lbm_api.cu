@@ -2136,11 +2136,12 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
         if (chunk_out) *chunk_out = 0;
         return LBM_OK;   // the FP64 step has no tile parameters
     }
+    if (h->bad) return fail(h, LBM_ESTATE, "state holds a non-finite density; re-initialise");
     if (h->lattice == LBM_D2Q9) {   // nor has the D2Q9 step: its chunk changes nothing
+        if ((rc = read_status(h))) return rc;
         if (chunk_out) *chunk_out = h->geof.chunk;
         return LBM_OK;
     }
-    if (h->bad) return fail(h, LBM_ESTATE, "state holds a non-finite density; re-initialise");
     const size_t bytes = pop_bytes(h->storage) * (size_t)h->Q * h->geo.N;
     const size_t rbytes = shifted(h->storage) ? sizeof(float) * h->geo.N : 0;
     void *save = nullptr;
