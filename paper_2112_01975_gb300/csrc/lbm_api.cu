@@ -346,17 +346,12 @@ int make_wall_bits(lbm_ctx *h)
 {
     if (h->lattice != LBM_D3Q27 || h->storage == LBM_F64 || !h->any_solid) return LBM_OK;
     const Geo &g = h->geo;
-    std::vector<int> table, planes;   // number of each z's plane; z of each plane
-    try {
-        table.assign(g.nz, -1);
-        for (int z = 0; z < g.nz; ++z)
-            if (h->zsolid_host[(z + g.nz - 1) % g.nz] || h->zsolid_host[z] || h->zsolid_host[(z + 1) % g.nz]) {
-                table[z] = (int)planes.size();
-                planes.push_back(z);
-            }
-    } catch (const std::bad_alloc &) {
-        return fail(h, LBM_ENOMEM, "no host memory for the wall planes");
-    }
+    std::vector<int> table(g.nz, -1), planes;   // number of each z's plane; z of each plane
+    for (int z = 0; z < g.nz; ++z)
+        if (h->zsolid_host[(z + g.nz - 1) % g.nz] || h->zsolid_host[z] || h->zsolid_host[(z + 1) % g.nz]) {
+            table[z] = (int)planes.size();
+            planes.push_back(z);
+        }
     const size_t head = align_up(sizeof(int) * 2 * g.nz);
     if (head + sizeof(unsigned) * planes.size() * g.px * g.ny > sizeof(double) * 3 * g.N)
         return fail(h, LBM_EINVAL, "no room for the wall bits");   // not for any lattice of 5 or more nodes a side
@@ -375,9 +370,10 @@ int make_wall_bits(lbm_ctx *h)
     return LBM_OK;
 }
 
-int ensure_memory(lbm_ctx *h)
+// Lay out the device memory (allocated here unless bound) and fill what stays
+// as it is: masks, wall bits, tensor maps.
+int lay_out(lbm_ctx *h)
 {
-    if (h->fv[0]) return LBM_OK;
     Layout L = layout_for(h->D, h->Q, h->geo.N, h->storage, h->geof.nz);
     if (!h->base) {
         void *p = nullptr;
@@ -408,11 +404,7 @@ int ensure_memory(lbm_ctx *h)
     // the mask with the rows' padding, if any, marked solid
     std::vector<uint8_t> padded;
     if (h->geo.px != h->geo.nx) {
-        try {
-            padded.assign(h->geo.N, 1);
-        } catch (const std::bad_alloc &) {
-            return fail(h, LBM_ENOMEM, "no host memory for the padded mask");
-        }
+        padded.assign(h->geo.N, 1);
         for (size_t r = 0; r < (size_t)h->geo.ny * h->geo.nz; ++r)
             memcpy(&padded[r * h->geo.px], &h->mask_host[r * h->geo.nx], h->geo.nx);
     }
@@ -431,16 +423,39 @@ int ensure_memory(lbm_ctx *h)
     }
     CU(h, cudaMemsetAsync(h->status, 0, sizeof(int) * 4, h->stream));
     const int rc = make_wall_bits(h);
-    if (rc != LBM_OK) {
-        h->fv[0] = nullptr;   // not laid out: the next call starts over
-        return rc;
-    }
+    if (rc != LBM_OK) return rc;
     CU(h, cudaStreamSynchronize(h->stream));
     make_tensor_maps(h);
     if (h->variant == LBM_FUSED_WS_TMA && !h->tmap_ready) h->variant = LBM_FUSED_WS_TMEM;
     if (h->variant == LBM_FUSED_TM_TMA && !h->tmap_ready) h->variant = LBM_FUSED_TMEM;
     choose_form(h);
     return LBM_OK;
+}
+
+// The device memory laid out, on the handle's first use of it. After a failure
+// nothing is (fv[0] null): the next call starts over.
+int ensure_memory(lbm_ctx *h)
+{
+    if (h->fv[0]) return LBM_OK;
+    int rc;
+    try {
+        rc = lay_out(h);
+    } catch (const std::bad_alloc &) {
+        rc = fail(h, LBM_ENOMEM, "no host memory to lay out the lattice");
+    }
+    if (rc == LBM_OK) return rc;
+    cudaStreamSynchronize(h->stream);   // copies from host memory that is about to go
+    cudaGetLastError();
+    h->fv[0] = nullptr;
+    h->geof.wplane = nullptr;
+    h->geof.walls = nullptr;
+    if (h->owns_base) {
+        cudaFree(h->base);
+        h->base = nullptr;
+        h->owns_base = false;
+        h->bytes = 0;
+    }
+    return rc;
 }
 
 bool has_solid(const lbm_ctx *h) { return h->any_solid; }
