@@ -315,8 +315,7 @@ int lbm_set_tile(lbm_handle h, int tile_y);
  * storage from its first use of device memory on (LBM_FUSED_TMEM where there
  * is none, where nx leaves remainder 1 by 4 (FP32) or 8 (shifted), or where
  * the tiles of shifted storage hang far over the lattice; LBM_FUSED_PLAIN
- * with LBM_FLAG_EOS_F64). For other nx that are not a multiple of 4 or 8 the
- * TMA-staged forms run only by that choice or lbm_autotune's.
+ * with LBM_FLAG_EOS_F64).
  *   LBM_FUSED_PLAIN: one thread group per tile; each entering
  *     plane's densities, pseudo-potentials and velocities are formed, the
  *     block synchronises, and the plane two behind collides and streams,
@@ -347,17 +346,16 @@ enum {
  *     warp-specialised form with the Tensor Memory staging, the producer that
  *     loads a node leaving its populations in the lane of the consumer that
  *     collides it.
- *   LBM_FUSED_WS_TMA (D3Q27, 32 x 8 tiles; FP32 with nx a multiple of 4, or
- *     shifted storage with nx a multiple of 8): the LBM_FUSED_WS_TMEM form
- *     with each entering plane's populations on the tile's halo copied into
+ *   LBM_FUSED_WS_TMA (D3Q27, 32 x 8 tiles; FP32 or shifted storage): the
+ *     LBM_FUSED_WS_TMEM form with each entering plane's populations on the tile's halo copied into
  *     shared memory by the tensor-memory-access unit (nine bulk tensor
  *     copies per plane, requested two planes ahead) instead of loaded by the
  *     producers; 215 KB (FP32) or 175 KB of shared memory per block. The
  *     tensor maps are made when the handle's device memory is laid out; if
  *     the CUDA driver offers no tensor-map encoder, a handle set to this
  *     form runs LBM_FUSED_WS_TMEM (lbm_get_fused_variant says which).
- *   LBM_FUSED_TM_TMA (shifted storage only; D3Q27, 32 x 8 tiles, nx a
- *     multiple of 8): the LBM_FUSED_TMEM form (one thread group, two blocks
+ *   LBM_FUSED_TM_TMA (shifted storage only; D3Q27, 32 x 8 tiles):
+ *     the LBM_FUSED_TMEM form (one thread group, two blocks
  *     per SM) with each entering plane copied into shared memory by the
  *     tensor-memory-access unit in one stage, requested a phase ahead (one
  *     copy per plane where the tile's halo stays inside the lattice, nine
@@ -367,9 +365,9 @@ enum {
  * LBM_FUSED_PLAIN with LBM_F64 storage or LBM_FLAG_EOS_F64, or
  * LBM_FUSED_WARP_SPECIALISED with shifted storage, LBM_FUSED_TM_TMA with
  * LBM_F32, or LBM_FUSED_WS_TMEM, LBM_FUSED_WS_TMA or LBM_FUSED_TM_TMA with
- * D2Q9 or 7-row tiles, or the TMA-staged forms with nx not a multiple of 4
- * (FP32) or 8 (shifted) or, after the memory is laid out, without tensor
- * maps. */
+ * D2Q9 or 7-row tiles, or the TMA-staged forms without tensor maps or, before
+ * the memory is laid out, with nx not a multiple of 4 (FP32) or 8 (shifted);
+ * afterwards any nx takes them, as rows are padded. */
 int lbm_set_fused_variant(lbm_handle h, int variant);
 
 /* *variant = the form of the fused step in use (LBM_FUSED_PLAIN before the

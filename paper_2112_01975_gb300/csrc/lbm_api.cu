@@ -2269,11 +2269,13 @@ int lbm_set_fused_variant(lbm_handle h, int variant)
         return fail(h, LBM_EINVAL, "the one-group TMA-staged form is a form of shifted storage");
     if (variant >= LBM_FUSED_WS_TMEM && (h->lattice != LBM_D3Q27 || h->tile_rows != 8))
         return fail(h, LBM_EINVAL, "the warp-specialised Tensor Memory forms run D3Q27 32 x 8 tiles");
+    // with the memory laid out the tensor maps decide (rows are padded for them,
+    // so that what lbm_autotune or the handle chose can be set); before that, the width
+    const int mult = tma_nx_multiple(h->storage);
     if ((variant == LBM_FUSED_WS_TMA || variant == LBM_FUSED_TM_TMA) &&
-        (!tma_nx_multiple(h->storage) || h->geo.nx % tma_nx_multiple(h->storage) ||
-         (h->fv[0] && !h->tmap_ready)))
-        return fail(h, LBM_EINVAL, "the TMA-staged form needs FP32 storage with nx a multiple of 4 or shifted "
-                                   "storage with nx a multiple of 8, and the CUDA driver's tensor-map encoder");
+        (!mult || (h->fv[0] ? !h->tmap_ready : h->geo.nx % mult != 0)))
+        return fail(h, LBM_EINVAL, "the TMA-staged forms need FP32 or shifted storage and the CUDA driver's tensor-map "
+                                   "encoder and, before the memory is laid out, nx a multiple of 4 (FP32) or 8 (shifted)");
     if (h->storage == LBM_F64 && variant != LBM_FUSED_PLAIN)
         return fail(h, LBM_EINVAL, "the FP64 step has one form");
     if (h->e64 && variant != LBM_FUSED_PLAIN)

@@ -1,5 +1,6 @@
 """lbm_autotune of D2Q9 lattices, whose step has nothing to tune: a state that
-is not finite is still reported."""
+is not finite is still reported. And the form that a lattice of any width
+reports, by its own choice or tuned, can be set on it and on another."""
 import numpy as np
 import pytest
 
@@ -44,3 +45,36 @@ def test_autotune_reports_a_diverged_state(lbm, lattice, storage, seen):
     assert e.value.code == (ESTATE if seen else ENONFINITE)
     g.init(rho)
     assert g.autotune() >= 1
+
+
+@pytest.mark.parametrize("storage", [1, 2, 3])
+@pytest.mark.parametrize("nx", [38, 41, 64, 97])
+def test_a_reported_form_can_be_set(lbm, storage, nx):
+    w = inputs.DROP_D3Q27_128
+    n = (nx, 24, 16)
+    rho = inputs.add_noise(inputs.drop(*n, 5.0, w.rho_v, w.rho_l), 1e-3, 5)
+
+    def make():
+        g = lbm.LBM(1, *n, w.eos, w.t_over_tc, w.kappa, 0.8, a=w.a, b=w.b, storage=storage)
+        g.init(rho)
+        return g
+
+    ref = make()
+    ref.set_fused_variant(lbm.FUSED_PLAIN)
+    ref.step(5)
+    want = ref.get_populations()
+    tuned = make()
+    own = tuned.fused_variant
+    chunk = tuned.autotune()
+    # the TMA-staged forms of the storage run at any width
+    staged = lbm.FUSED_WS_TMA if storage == lbm.F32 else lbm.FUSED_TM_TMA
+    for v in {own, tuned.fused_variant, staged, lbm.FUSED_WS_TMA}:
+        g = make()
+        g.set_fused_variant(v)
+        g.set_chunk(chunk)
+        assert g.fused_variant == v
+        g.step(5)
+        assert np.array_equal(g.get_populations(), want)
+    tuned.set_fused_variant(tuned.fused_variant)
+    tuned.step(5)
+    assert np.array_equal(tuned.get_populations(), want)
