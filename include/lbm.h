@@ -374,13 +374,14 @@ int lbm_set_fused_variant(lbm_handle h, int variant);
  * device memory is laid out, if none was set). */
 int lbm_get_fused_variant(lbm_handle h, int *variant);
 
-/* ---- Batches: many lattices advanced by one persistent launch ----------
+/* ---- Batches: many lattices advanced together --------------------------
  * A batch holds count >= 1 distinct, initialised handles with the same
  * storage (LBM_F32, LBM_F16S or LBM_BF16S, not LBM_F64) and the same lattice
- * type, of any sizes and parameters; otherwise LBM_EINVAL. Each
- * lbm_batch_step launch gives every member one time step (the fused step of
- * that storage over all members' tiles, in the TMA-staged form for D3Q27;
- * a step of more than 32 D3Q27 members takes a launch for each 32); steps after the first replay a CUDA graph of two launches. Each
+ * type, of any sizes and parameters; otherwise LBM_EINVAL. Each step gives
+ * every member one time step in one launch (the fused step of that storage
+ * over all members' tiles, in the TMA-staged form for D3Q27; more than 32
+ * D3Q27 members take a launch for each 32); steps after the first replay a
+ * CUDA graph of two steps, long calls on small members one of 16. Each
  * member's result is bitwise the same as stepping it alone. While the batch
  * exists the members' work is ordered on the batch's stream (members must
  * not be stepped, initialised or written individually); lbm_batch_destroy

@@ -576,12 +576,10 @@ int sweep_chunk(const Geo &g, int sms)
 double *f64(lbm_ctx *h, int k) { return static_cast<double *>(h->fv[k]); }
 float *f32(lbm_ctx *h, int k) { return static_cast<float *>(h->fv[k]); }
 
-template <int LAT>
-dim3 fused_grid(const GeoF &g, int rows = lbmf::LatF<LAT>::TY)
+dim3 fused_grid(const GeoF &g, int rows = lbmf::LatF<1>::TY)
 {
-    using L = lbmf::LatF<LAT>;
-    const int ty = LAT == 1 ? rows : L::TY;
-    return dim3((g.nx + L::TX - 1) / L::TX, (g.ny + ty - 1) / ty, (g.nz + g.chunk - 1) / g.chunk);
+    using L = lbmf::LatF<1>;
+    return dim3((g.nx + L::TX - 1) / L::TX, (g.ny + rows - 1) / rows, (g.nz + g.chunk - 1) / g.chunk);
 }
 
 // The same parameters as the 7-row build's types (one source, one layout).
@@ -602,7 +600,7 @@ void launch_fused_r7(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
         static std::atomic<unsigned long long> done{0};   // devices already opted in
         const int bytes = (int)sizeof(lbmf7::SharedF<1>);
         smem_opt_in(lbmf7::k_step_f32_tm<1, MASK>, bytes, done);
-        lbmf7::k_step_f32_tm<1, MASK><<<fused_grid<1>(h->geof, L::TY), L::TX * L::TY, bytes, s>>>(
+        lbmf7::k_step_f32_tm<1, MASK><<<fused_grid(h->geof, L::TY), L::TX * L::TY, bytes, s>>>(
             as_layout<lbmf7::GeoF>(h->geof), as_layout<lbmf7::PhysF>(h->physf), h->mask, src, dst,
             h->status);
         return;
@@ -611,7 +609,7 @@ void launch_fused_r7(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
         static std::atomic<unsigned long long> done{0};   // devices already opted in
         const int bytes = (int)sizeof(lbmf7::SharedWS<1>);
         smem_opt_in(lbmf7::k_step_f32_ws<1, MASK>, bytes, done);
-        lbmf7::k_step_f32_ws<1, MASK><<<fused_grid<1>(h->geof, L::TY), 2 * L::TX * L::TY, bytes, s>>>(
+        lbmf7::k_step_f32_ws<1, MASK><<<fused_grid(h->geof, L::TY), 2 * L::TX * L::TY, bytes, s>>>(
             as_layout<lbmf7::GeoF>(h->geof), as_layout<lbmf7::PhysF>(h->physf), h->mask, src, dst,
             h->status);
         return;
@@ -619,19 +617,19 @@ void launch_fused_r7(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
     static std::atomic<unsigned long long> done{0};   // devices already opted in
     const int bytes = (int)sizeof(lbmf7::SharedF<1>);
     smem_opt_in(lbmf7::k_step_f32<1, MASK>, bytes, done);
-    lbmf7::k_step_f32<1, MASK><<<fused_grid<1>(h->geof, L::TY), L::TX * L::TY, bytes, s>>>(
+    lbmf7::k_step_f32<1, MASK><<<fused_grid(h->geof, L::TY), L::TX * L::TY, bytes, s>>>(
         as_layout<lbmf7::GeoF>(h->geof), as_layout<lbmf7::PhysF>(h->physf), h->mask, src, dst,
         h->status);
 }
 
-template <int LAT, bool MASK>
+template <bool MASK>
 void launch_fused_tm(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    using L = lbmf::LatF<LAT>;
-    const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
-    smem_opt_in(lbmf::k_step_f32_tm<LAT, MASK>, bytes, done);
-    lbmf::k_step_f32_tm<LAT, MASK><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    using L = lbmf::LatF<1>;
+    const int bytes = (int)sizeof(lbmf::SharedF<1>);
+    smem_opt_in(lbmf::k_step_f32_tm<1, MASK>, bytes, done);
+    lbmf::k_step_f32_tm<1, MASK><<<fused_grid(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
@@ -642,29 +640,29 @@ void launch_fused_wstm(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
     using L = lbmf::LatF<1>;
     const int bytes = (int)sizeof(lbmf::SharedWS<1>);
     smem_opt_in(lbmf::k_step_f32_wstm<1, MASK>, bytes, done);
-    lbmf::k_step_f32_wstm<1, MASK><<<fused_grid<1>(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
+    lbmf::k_step_f32_wstm<1, MASK><<<fused_grid(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
-template <int LAT, bool MASK>
+template <bool MASK>
 void launch_fused_ws(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    using L = lbmf::LatF<LAT>;
-    const int bytes = (int)sizeof(lbmf::SharedWS<LAT>);
-    smem_opt_in(lbmf::k_step_f32_ws<LAT, MASK>, bytes, done);
-    lbmf::k_step_f32_ws<LAT, MASK><<<fused_grid<LAT>(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
+    using L = lbmf::LatF<1>;
+    const int bytes = (int)sizeof(lbmf::SharedWS<1>);
+    smem_opt_in(lbmf::k_step_f32_ws<1, MASK>, bytes, done);
+    lbmf::k_step_f32_ws<1, MASK><<<fused_grid(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
-template <int LAT, bool MASK>
+template <bool MASK>
 void launch_fused_e64(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    using L = lbmf::LatF<LAT>;
-    const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
-    smem_opt_in(lbmf::k_step_f32<LAT, MASK, true>, bytes, done);
-    lbmf::k_step_f32<LAT, MASK, true><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    using L = lbmf::LatF<1>;
+    const int bytes = (int)sizeof(lbmf::SharedF<1>);
+    smem_opt_in(lbmf::k_step_f32<1, MASK, true>, bytes, done);
+    lbmf::k_step_f32<1, MASK, true><<<fused_grid(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
@@ -725,67 +723,67 @@ void launch_2d(lbm_ctx *h, cudaStream_t s, int k)
     }
 }
 
-template <int LAT, bool MASK>
+template <bool MASK>
 void launch_fused_rest(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    using L = lbmf::LatF<LAT>;
-    const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
-    smem_opt_in(lbmf::k_step_f32<LAT, MASK, false, true>, bytes, done);
-    lbmf::k_step_f32<LAT, MASK, false, true><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    using L = lbmf::LatF<1>;
+    const int bytes = (int)sizeof(lbmf::SharedF<1>);
+    smem_opt_in(lbmf::k_step_f32<1, MASK, false, true>, bytes, done);
+    lbmf::k_step_f32<1, MASK, false, true><<<fused_grid(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, src, dst, h->status);
 }
 
-template <int LAT>
+// One D3Q27 step of FP32 storage.
 void launch_fused(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 {
     if (h->e64) {   // the plain 32 x 8 form only
-        if (has_solid(h)) launch_fused_e64<LAT, true>(h, s, src, dst);
-        else              launch_fused_e64<LAT, false>(h, s, src, dst);
+        if (has_solid(h)) launch_fused_e64<true>(h, s, src, dst);
+        else              launch_fused_e64<false>(h, s, src, dst);
         return;
     }
-    if (LAT == 1 && h->tile_rows == 7) {
+    if (h->tile_rows == 7) {
         if (has_solid(h)) launch_fused_r7<true>(h, s, src, dst);
         else              launch_fused_r7<false>(h, s, src, dst);
         return;
     }
     if (h->variant == LBM_FUSED_WARP_SPECIALISED) {
-        if (has_solid(h)) launch_fused_ws<LAT, true>(h, s, src, dst);
-        else              launch_fused_ws<LAT, false>(h, s, src, dst);
+        if (has_solid(h)) launch_fused_ws<true>(h, s, src, dst);
+        else              launch_fused_ws<false>(h, s, src, dst);
         return;
     }
     if (lbmf::at_rest(h->physf) && (h->variant == LBM_FUSED_TMEM || h->variant == LBM_FUSED_PLAIN)) {
         // nothing to keep between the phases: the two forms are one
-        if (has_solid(h)) launch_fused_rest<LAT, true>(h, s, src, dst);
-        else              launch_fused_rest<LAT, false>(h, s, src, dst);
+        if (has_solid(h)) launch_fused_rest<true>(h, s, src, dst);
+        else              launch_fused_rest<false>(h, s, src, dst);
         return;
     }
     if (h->variant == LBM_FUSED_TMEM) {
-        if (has_solid(h)) launch_fused_tm<LAT, true>(h, s, src, dst);
-        else              launch_fused_tm<LAT, false>(h, s, src, dst);
+        if (has_solid(h)) launch_fused_tm<true>(h, s, src, dst);
+        else              launch_fused_tm<false>(h, s, src, dst);
         return;
     }
-    if (LAT == 1 && h->variant == LBM_FUSED_WS_TMA) {   // D3Q27, 32 x 8 tiles, tensor maps made
+    if (h->variant == LBM_FUSED_WS_TMA) {   // D3Q27, 32 x 8 tiles, tensor maps made
         lbmtma::launch(h->geof, h->physf, h->mask, h->tmaps[src == h->fv[0] ? 0 : 1], src, dst, h->status,
                        has_solid(h), s);
         return;
     }
-    if (LAT == 1 && h->variant == LBM_FUSED_WS_TMEM) {   // D3Q27, 32 x 8 tiles
+    if (h->variant == LBM_FUSED_WS_TMEM) {   // D3Q27, 32 x 8 tiles
         if (has_solid(h)) launch_fused_wstm<true>(h, s, src, dst);
         else              launch_fused_wstm<false>(h, s, src, dst);
         return;
     }
     static std::atomic<unsigned long long> done_m{0}, done_f{0};   // devices already opted in
-    using L = lbmf::LatF<LAT>;
-    const int bytes = (int)sizeof(lbmf::SharedF<LAT>);
-    const dim3 gr = fused_grid<LAT>(h->geof);
+    using L = lbmf::LatF<1>;
+    const int bytes = (int)sizeof(lbmf::SharedF<1>);
+    const dim3 gr = fused_grid(h->geof);
     if (has_solid(h)) {
-        smem_opt_in(lbmf::k_step_f32<LAT, true>, bytes, done_m);
-        lbmf::k_step_f32<LAT, true><<<gr, L::TX * L::TY, bytes, s>>>(h->geof, h->physf, h->mask, src,
+        smem_opt_in(lbmf::k_step_f32<1, true>, bytes, done_m);
+        lbmf::k_step_f32<1, true><<<gr, L::TX * L::TY, bytes, s>>>(h->geof, h->physf, h->mask, src,
                                                                     dst, h->status);
     } else {
-        smem_opt_in(lbmf::k_step_f32<LAT, false>, bytes, done_f);
-        lbmf::k_step_f32<LAT, false><<<gr, L::TX * L::TY, bytes, s>>>(h->geof, h->physf, h->mask, src,
+        smem_opt_in(lbmf::k_step_f32<1, false>, bytes, done_f);
+        lbmf::k_step_f32<1, false><<<gr, L::TX * L::TY, bytes, s>>>(h->geof, h->physf, h->mask, src,
                                                                      dst, h->status);
     }
 }
@@ -794,29 +792,29 @@ void launch_fused(lbm_ctx *h, cudaStream_t s, const float *src, float *dst)
 void launch_f32(lbm_ctx *h, cudaStream_t s, int k)
 {
     if (h->lattice == LBM_D2Q9) launch_2d<float>(h, s, k);
-    else                        launch_fused<1>(h, s, f32(h, k), f32(h, k ^ 1));
+    else                        launch_fused(h, s, f32(h, k), f32(h, k ^ 1));
 }
 
-template <int LAT, typename ST, bool E64, bool MASK, bool REST = false>
+template <typename ST, bool E64, bool MASK, bool REST = false>
 void launch_shifted_e(lbm_ctx *h, cudaStream_t s, int k)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    const int bytes = (int)sizeof(lbmf::SharedS<LAT>);
-    smem_opt_in(lbmf::k_step_shifted<LAT, ST, E64, MASK, REST>, bytes, done);
-    using L = lbmf::LatF<LAT>;
-    lbmf::k_step_shifted<LAT, ST, E64, MASK, REST><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    const int bytes = (int)sizeof(lbmf::SharedS<1>);
+    smem_opt_in(lbmf::k_step_shifted<1, ST, E64, MASK, REST>, bytes, done);
+    using L = lbmf::LatF<1>;
+    lbmf::k_step_shifted<1, ST, E64, MASK, REST><<<fused_grid(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]),
         h->rs[k], h->rs[k ^ 1], h->status);
 }
 
-template <int LAT, typename ST, bool MASK>
+template <typename ST, bool MASK>
 void launch_shifted_tm(lbm_ctx *h, cudaStream_t s, int k)
 {
     static std::atomic<unsigned long long> done{0};   // devices already opted in
-    const int bytes = (int)sizeof(lbmf::SharedS<LAT>);
-    smem_opt_in(lbmf::k_step_shifted_tm<LAT, ST, MASK>, bytes, done);
-    using L = lbmf::LatF<LAT>;
-    lbmf::k_step_shifted_tm<LAT, ST, MASK><<<fused_grid<LAT>(h->geof), L::TX * L::TY, bytes, s>>>(
+    const int bytes = (int)sizeof(lbmf::SharedS<1>);
+    smem_opt_in(lbmf::k_step_shifted_tm<1, ST, MASK>, bytes, done);
+    using L = lbmf::LatF<1>;
+    lbmf::k_step_shifted_tm<1, ST, MASK><<<fused_grid(h->geof), L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]),
         h->rs[k], h->rs[k ^ 1], h->status);
 }
@@ -828,38 +826,38 @@ void launch_shifted_wstm(lbm_ctx *h, cudaStream_t s, int k)
     const int bytes = (int)sizeof(lbmf::SharedSWS<1>);
     smem_opt_in(lbmf::k_step_shifted_wstm<1, ST, MASK>, bytes, done);
     using L = lbmf::LatF<1>;
-    lbmf::k_step_shifted_wstm<1, ST, MASK><<<fused_grid<1>(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
+    lbmf::k_step_shifted_wstm<1, ST, MASK><<<fused_grid(h->geof), 2 * L::TX * L::TY, bytes, s>>>(
         h->geof, h->physf, h->mask, static_cast<const ST *>(h->fv[k]), static_cast<ST *>(h->fv[k ^ 1]),
         h->rs[k], h->rs[k ^ 1], h->status);
 }
 
-template <int LAT, typename ST, bool MASK>
+template <typename ST, bool MASK>
 void launch_shifted_m(lbm_ctx *h, cudaStream_t s, int k)
 {
-    if (LAT == 1 && !h->e64 && h->variant == LBM_FUSED_WS_TMA) {   // tensor maps made
+    if (!h->e64 && h->variant == LBM_FUSED_WS_TMA) {   // tensor maps made
         lbmtma::launch_shifted(h->geof, h->physf, h->mask, h->tmaps[k], static_cast<const ST *>(h->fv[k]),
                                static_cast<ST *>(h->fv[k ^ 1]), h->rs[k], h->rs[k ^ 1], h->status, MASK, s);
         return;
     }
-    if (LAT == 1 && !h->e64 && h->variant == LBM_FUSED_TM_TMA) {   // tensor maps made
+    if (!h->e64 && h->variant == LBM_FUSED_TM_TMA) {   // tensor maps made
         lbmtma::launch_shifted_tm(h->geof, h->physf, h->mask, h->tmaps[k], static_cast<const ST *>(h->fv[k]),
                                   static_cast<ST *>(h->fv[k ^ 1]), h->rs[k], h->rs[k ^ 1], h->status, MASK,
                                   s);
         return;
     }
-    if (h->e64) launch_shifted_e<LAT, ST, true, MASK>(h, s, k);
+    if (h->e64) launch_shifted_e<ST, true, MASK>(h, s, k);
     else if (lbmf::at_rest(h->physf) && (h->variant == LBM_FUSED_TMEM || h->variant == LBM_FUSED_PLAIN))
-        launch_shifted_e<LAT, ST, false, MASK, true>(h, s, k);   // nothing to keep between the phases
-    else if (h->variant == LBM_FUSED_TMEM) launch_shifted_tm<LAT, ST, MASK>(h, s, k);
-    else if (LAT == 1 && h->variant == LBM_FUSED_WS_TMEM) launch_shifted_wstm<ST, MASK>(h, s, k);
-    else launch_shifted_e<LAT, ST, false, MASK>(h, s, k);
+        launch_shifted_e<ST, false, MASK, true>(h, s, k);   // nothing to keep between the phases
+    else if (h->variant == LBM_FUSED_TMEM) launch_shifted_tm<ST, MASK>(h, s, k);
+    else if (h->variant == LBM_FUSED_WS_TMEM) launch_shifted_wstm<ST, MASK>(h, s, k);
+    else launch_shifted_e<ST, false, MASK>(h, s, k);
 }
 
-template <int LAT, typename ST>
+template <typename ST>
 void launch_shifted_t(lbm_ctx *h, cudaStream_t s, int k)
 {
-    if (has_solid(h)) launch_shifted_m<LAT, ST, true>(h, s, k);
-    else              launch_shifted_m<LAT, ST, false>(h, s, k);
+    if (has_solid(h)) launch_shifted_m<ST, true>(h, s, k);
+    else              launch_shifted_m<ST, false>(h, s, k);
 }
 
 // One step of shifted storage from population buffer k.
@@ -870,8 +868,8 @@ void launch_shifted(lbm_ctx *h, cudaStream_t s, int k)
         if (half) launch_2d<__half>(h, s, k);
         else      launch_2d<__nv_bfloat16>(h, s, k);
     } else {
-        if (half) launch_shifted_t<1, __half>(h, s, k);
-        else      launch_shifted_t<1, __nv_bfloat16>(h, s, k);
+        if (half) launch_shifted_t<__half>(h, s, k);
+        else      launch_shifted_t<__nv_bfloat16>(h, s, k);
     }
 }
 
@@ -1769,6 +1767,8 @@ void launch_batch_plain_shifted(lbm_batch_ctx *b, const lbmf::WorkItem *items, i
         b->d_members[parity], items, n);
 }
 
+// D3Q27 members without tensor maps: no encoder in the CUDA driver, or rows that
+// could not be padded (row_pitch).
 void launch_batch_plain(lbm_batch_ctx *b, const lbmf::WorkItem *items, int n, int parity, cudaStream_t s)
 {
     if (b->storage == LBM_F16S) launch_batch_plain_shifted<__half>(b, items, n, parity, s);
@@ -2180,23 +2180,20 @@ int lbm_autotune(lbm_handle h, int *chunk_out)
     const int chunk0 = h->geof.chunk, rows0 = h->tile_rows;   // restored on failure
     const bool auto0 = h->auto_form;
     h->auto_form = false;
-    // FP32: the plain, warp-specialised and Tensor Memory kernels; D3Q27 FP32
-    // also 32 x 8 and 32 x 7 tiles (the shifted and batched steps use plain
-    // 32 x 8)
+    // every form of the storage; FP32 also 32 x 8 and 32 x 7 tiles (the forms up
+    // to LBM_FUSED_TMEM)
     const bool fp32 = h->storage == LBM_F32 && !h->e64;   // the FP64-EOS form is plain 32 x 8
-    const bool two_heights = h->lattice == LBM_D3Q27 && fp32;
     const int variant0 = h->variant;
     int best = h->geof.chunk, best_rows = h->tile_rows, best_variant = h->variant;
     double best_ms = 1e30;
     for (int var = 0; var <= LBM_FUSED_TM_TMA && rc == LBM_OK; ++var) {
-        // shifted storage: plain, Tensor Memory and (D3Q27) the two warp-specialised Tensor Memory forms
+        // shifted storage: no warp-specialised form without Tensor Memory
         if (var > 0 && (h->e64 || (!fp32 && var == LBM_FUSED_WARP_SPECIALISED))) continue;
-        if (var >= LBM_FUSED_WS_TMEM && h->lattice != LBM_D3Q27) continue;
         if ((var == LBM_FUSED_WS_TMA || var == LBM_FUSED_TM_TMA) && !h->tmap_ready) continue;
         if (var == LBM_FUSED_TM_TMA && !shifted(h->storage)) continue;   // a form of shifted storage
         h->variant = var;
         for (int rows : {8, 7}) {
-            if (rows == 7 && (!two_heights || var >= LBM_FUSED_WS_TMEM)) continue;
+            if (rows == 7 && (!fp32 || var >= LBM_FUSED_WS_TMEM)) continue;
             h->tile_rows = rows;
             for (size_t j = 0; j < cands.size(); ++j) {
                 const int c = cands[j];
