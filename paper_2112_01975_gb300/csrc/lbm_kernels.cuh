@@ -1055,7 +1055,8 @@ __device__ __forceinline__ float narrow(double d)
 }
 
 // (float)(f / v - w) in 5 FP64 operations: the quotient starts from the FP32
-// one and is corrected twice by its exact remainder (to 2^-70, so its FP64
+// one and is corrected twice by its exact remainder, a fused multiply-add's
+// (P. W. Markstein, IBM J. Res. Dev. 34, 1990, 111; to 2^-70, so its FP64
 // rounding is the division's but for about 1 in 10^5). Encoding 128x96x112
 // with its densities: 426 us, with a multiplication by 1/v first and the
 // conversion instruction (7 operations) 544 us.
