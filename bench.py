@@ -47,13 +47,14 @@ ALG_BYTES_PER_LU = {  # populations read once and written once per lattice updat
     (0, "bf16s"): 2 * 9 * 2 + 8,
 }
 # FP64 flops per node executed by the D3Q27 collision kernel (k_force_sweep3
-# with its collision), counted from the source: force sums of two fields 98
-# (per field: x sums 12 with the tile's halo rows, y sums 14, z sums 23), force
+# with its collision), counted from the source: force sums of two fields 111
+# (per field and with the tile's halo: differences 9, x smoothing of the z
+# differences 9, each node's smoothings 18, z sums and rings 20), force
 # 11, Phi 3, 1/rho and its factor 3, product-form factors 54, partial products
 # 26, collision 135; at relaxation time 1, where the equilibrium and the
 # populations drop out, the last three are 33, 12 and 27.
 def collide_fp64_flops(tau: float) -> int:
-    return 187 if tau == 1.0 else 330
+    return 200 if tau == 1.0 else 343
 
 
 FP64_PEAK_TFLOPS = 1.25   # GB300 nominal FP64 rate (context; the roofline uses the live probe)
@@ -77,16 +78,16 @@ def fp64_peak():
 MEASURED_TRAFFIC = {
     # k_step_f32_wstma, 32 x 8 tiles, chunk 247 (one 247-plane and one
     # 9-plane chunk per column, as at full size), on the impact scaled to
-    # 192x192x256: 1118.3 + 965.5 MB for 9,437,184 nodes
+    # 192x192x256: 1116.2 + 964.1 MB for 9,437,184 nodes
     # (profiles/k_step_f32_wstma_d3q27_impact_192x192x256.md)
     ("d3q27_impact_384x384x256_pr_tr0.5", "f32", 8, 4): {
-        "bytes_per_node": 220.81, "src_sha": "f6d58c9291f8e24e"},
+        "bytes_per_node": 220.43, "src_sha": "76cdd479947f5188"},
     # k_step_shifted_tmtma (FP16-shifted, Tensor Memory with TMA-staged
-    # planes), 32 x 8 tiles, chunk 208, on the same scaled impact: 586.6 +
-    # 500.7 MB for 9,437,184 nodes
+    # planes), 32 x 8 tiles, chunk 240, on the same scaled impact: 583.4 +
+    # 504.3 MB for 9,437,184 nodes
     # (profiles/k_step_shifted_tmtma_d3q27_impact_192x192x256.md)
     ("d3q27_impact_384x384x256_pr_tr0.5", "f16s", 8, 5): {
-        "bytes_per_node": 115.22, "src_sha": "f6d58c9291f8e24e"},
+        "bytes_per_node": 115.26, "src_sha": "76cdd479947f5188"},
 }
 FUSED_SRC = os.path.join(ROOT, "paper_2112_01975_gb300", "csrc", "lbm_fused_f32_body.cuh")
 

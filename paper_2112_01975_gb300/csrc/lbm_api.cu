@@ -276,10 +276,10 @@ void make_tensor_maps(lbm_ctx *h);
 // 1.31 times as long per plane as one alone (measured: 5.4 against 4.1 us,
 // shifted storage at 128^3). The last, shorter chunk of each column fills the
 // SMs that the whole ones leave. Measured, TMA-staged forms, the choice here
-// against others: FP32 64^3 22.9 us (chunk 7; 8: 24.2), 128^3 96.6 (56; 64:
-// 102.9, 16: 125), 160^3 171 (108; 54: 176), 256^3 683 (223; 64: 702);
-// FP16-shifted 128^3 161 (29; 32: 173), 256^3 1059 (223; 64: 1139). Furthest
-// from the best of a scan: 97x61x75 FP32 51.1 (47.5).
+// against others: FP32 64^3 24.1 us (chunk 7; 8: 25.1), 128^3 104 (56; 64:
+// 114, 16: 135), 160^3 187 (108; 54: 191), 256^3 723 (223; 64: 762);
+// FP16-shifted 128^3 166 (29; 32: 179), 256^3 1093 (223; 64: 1174). Furthest
+// from the best of a scan: 97x61x75 FP32 53.3 (50.5).
 int best_chunk(const GeoF &g, int rows, int sms, int resident)
 {
     const long long tiles = (long long)((g.nx + 31) / 32) * ((g.ny + rows - 1) / rows);
@@ -303,17 +303,14 @@ constexpr int kDefaultChunk3 = 16;
 // Form and chunk of a D3Q27 handle of reduced storage that the caller has
 // left open: with tensor maps the TMA-staged form of the storage, the
 // fastest of the forms at every size measured, each at its best chunk (FP32
-// 64^3 22.9 us against 32.7 for the Tensor Memory form, 128^3 97 against 149,
-// 256^3 683 against 1085; FP16-shifted 128^3 161 against 184, 256^3 1059
-// against 1321). The Tensor Memory form without tensor maps, where a column of the
-// halo lies in no box (box_pos; 153 x 145 x 131 FP32: 205 us, before faster
-// reciprocals 215 against 290) and,
+// 64^3 24.1 us against 34.8 for the Tensor Memory form, 128^3 104 against 154,
+// 256^3 723 against 1127; FP16-shifted 128^3 166 against 190, 256^3 1093
+// against 1363). The Tensor Memory form without tensor maps, where a column of the
+// halo lies in no box (box_pos; 153 x 145 x 131 FP32: 206 us against 222) and,
 // in shifted storage, where the tiles hang over the lattice by more than a
 // tenth: there it reads less, while the TMA-staged form's nine copies cost the
-// same (98 x 61 x 75: 66 us, 45 x 37 x 60: 33; before faster reciprocals 71
-// against 80 and 36 against 41; 150^3: 319 against 275; FP32 98 x 61 x 75 then
-// 53 against 47). With the FP64 EOS the plain
-// one. The fixed default before, plain at chunk 16: FP32 64^3 62, 128^3 184,
+// same (98 x 61 x 75: 66 us against 75, 45 x 37 x 60: 31 against 38; 150^3, which
+// fills its tiles: 329 against 285). With the FP64 EOS the plain one. The fixed default before, plain at chunk 16: FP32 64^3 62, 128^3 184,
 // 256^3 1208; FP16-shifted 258, 1649.
 void choose_form(lbm_ctx *h)
 {
@@ -1141,7 +1138,7 @@ int launch_reduce(lbm_ctx *h)
 
 // Between two graph replays the GPU idles for 1 to 3 us, as long as a step of a
 // small lattice (64^2 FP32: 4.3 us a step with graphs of two steps, 2.6 with
-// 16, and 32 gain 3 % on that). Sequences of at least twice that on lattices whose step is
+// 16, and 32 gained 3 % on that). Sequences of at least twice that on lattices whose step is
 // short (under about 50 us) replay graphs of kLongSteps steps.
 constexpr int kLongSteps = 16;
 constexpr unsigned kLongNodes = 1u << 20;

@@ -391,7 +391,7 @@ k_force_sweep3(Geo g, Phys p, const double2 *__restrict__ rp, int chunk, Body bo
 // D3Q27 without sharing, one node per thread: each pair of opposite neighbours
 // once, by weight class (208 operations). For lattices so small that the
 // tiles above would be few, each summing five planes for one of its own
-// (24^3: 15 us a step, with tiles 38).
+// (32^3: 20 us, with tiles 33; sweep_chunk has the rule).
 template <typename Body>
 __global__ void __launch_bounds__(128)
 k_force_direct3(Geo g, Phys p, const double2 *__restrict__ rp, Body body)

@@ -18,10 +18,11 @@
 //
 // Blocks that wait also take up room: a successor that fits beside its
 // predecessor is handed out while SMs are unevenly busy and stays that way.
-// Measured (us a step, with and without): D2Q9 FP32 64^2 2.82 / 2.92, 128^2
-// 2.84 / 3.26, 256^2 3.82 / 3.60, 384^2 4.85 / 4.63, 512^2 6.76 / 7.09; FP64 64^2
-// 7.9 / 8.3, 96^2 14.9 / 8.5; D3Q27 FP32 TMA-staged (one block per SM) 32^3 9.6 /
-// 10.1, 64^3 19.7 / 20.4, 128^3 105.1 / 105.2; FP16-shifted 32^3 23.3 / 21.3. So
+// Measured (us a step, with and without): D2Q9 FP32 64^2 2.60 / 2.82, 128^2
+// 2.70 / 2.84, 256^2 3.79 / 3.34, 384^2 5.13 / 4.13, 512^2 6.16 / 6.44; FP64 64^2
+// 7.4 / 8.2, 96^2 11.7 / 8.1, 301x202 38.5 / 20.0; D3Q27 FP32 TMA-staged (one
+// block per SM) 32^3 9.0 / 9.5, 64^3 18.9 / 19.5, 128^3 101.2 / 101.6; the shifted
+// D3Q27 kernels, which lost by it (32^3 23.3 / 21.3), do not overlap. So
 // it is used where two steps' blocks have an SM each or nearly (side_by_side), where
 // a step's blocks leave no room for the next ones' (leaves_no_room), and not in between.
 #pragma once

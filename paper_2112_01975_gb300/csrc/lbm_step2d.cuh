@@ -9,10 +9,10 @@
 // and collides its own node, whose populations and moments stayed in
 // registers. Forming the halo's moments again in each tile costs 36 x 12 /
 // (32 x 8) = 1.7 times the moments; they are a small part of the step.
-// Measured (us per step, graph replays, FP32 / FP16-shifted) against the
+// Measured (us per step, graph replays, FP32 / FP16-shifted, time 1) against the
 // tile of 128 x 1 nodes marching along y that ran before, at its default
-// chunk of 64 rows: 512^2 8.4 / 9.4 against 90 / 140 (17 / 25 at its best
-// chunk, 4), 64^2 4.3 / 5.2 against 72. 32 x 4 tiles: the same up to 256^2,
+// chunk of 64 rows: 512^2 6.2 / 7.7 against 90 / 140 (17 / 25 at its best
+// chunk, 4), 64^2 2.6 / 3.1 against 72. 32 x 4 tiles: the same up to 256^2,
 // 10-20 % slower above.
 // The arithmetic is that of the D3Q27 tile (node_moments, force_f,
 // factors_f). In the frame of LatF<0> the 2D y axis is z.
