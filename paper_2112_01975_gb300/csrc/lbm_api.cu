@@ -964,13 +964,13 @@ int encode_from(lbm_ctx *h, const Geo &gf, const double *f)   // gf: the layout 
     return LBM_OK;
 }
 
-// Every node's populations from layout ga and type A to gb and B.
+// Populations from rows of pa entries of type A to rows of pb of B.
 template <typename A, typename B>
-void convert_pops(lbm_ctx *h, const Geo &ga, const Geo &gb, const A *in, B *out)
+void convert_pops(lbm_ctx *h, int pa, int pb, const A *in, B *out)
 {
-    const dim3 gr = node_grid(h->geo), bl = node_block(h->geo);
-    if (h->lattice == LBM_D2Q9) lbmk::k_convert<0><<<gr, bl, 0, h->stream>>>(ga, gb, in, out);
-    else                        lbmk::k_convert<1><<<gr, bl, 0, h->stream>>>(ga, gb, in, out);
+    const Geo &g = h->geo;
+    lbmk::k_convert<<<1024, 256, 0, h->stream>>>((unsigned)(h->Q * g.ny * g.nz), (unsigned)g.nx, (unsigned)pa,
+                                                 (unsigned)pb, in, out);
 }
 
 int temp_alloc(lbm_ctx *h, TempF64 &t)
@@ -1552,17 +1552,21 @@ int lbm_get_populations(lbm_handle h, double *f, int on_device)
         }
     } else if (h->storage == LBM_F32) {
         if (on_device) {
-            convert_pops(h, h->geo, lbmk::flat(h->geo), f32(h, h->cur), f);
+            convert_pops(h, h->geo.px, h->geo.nx, f32(h, h->cur), f);
             CU(h, cudaGetLastError());
             h->launches += 1;
         } else {
-            std::vector<float> tmp((size_t)h->Q * h->geo.N);
-            CU(h, cudaMemcpyAsync(tmp.data(), f32(h, h->cur), sizeof(float) * tmp.size(),
-                                  cudaMemcpyDeviceToHost, h->stream));
+            const float *src = f32(h, h->cur);
+            if (h->geo.px != h->geo.nx) {   // without the rows' padding, through the dead buffer
+                convert_pops(h, h->geo.px, h->geo.nx, src, f32(h, h->cur ^ 1));
+                CU(h, cudaGetLastError());
+                h->launches += 1;
+                src = f32(h, h->cur ^ 1);
+            }
+            std::vector<float> tmp(QN);
+            CU(h, cudaMemcpyAsync(tmp.data(), src, sizeof(float) * QN, cudaMemcpyDeviceToHost, h->stream));
             CU(h, cudaStreamSynchronize(h->stream));
-            const size_t nx = h->geo.nx, px = h->geo.px;
-            for (size_t r = 0; r < QN / nx; ++r)   // rows, without their padding
-                for (size_t x = 0; x < nx; ++x) f[r * nx + x] = tmp[r * px + x];
+            for (size_t k = 0; k < QN; ++k) f[k] = tmp[k];
         }
     } else {
         CU(h, cudaMemcpyAsync(f, f64(h, h->cur), sizeof(double) * QN,
@@ -1599,16 +1603,19 @@ int lbm_set_populations(lbm_handle h, const double *f, int on_device)
         if (!direct) CU(h, cudaStreamSynchronize(h->stream));   // before the temporary is freed
     } else if (h->storage == LBM_F32) {
         if (on_device) {
-            convert_pops(h, lbmk::flat(h->geo), h->geo, f, f32(h, 0));
+            convert_pops(h, h->geo.nx, h->geo.px, f, f32(h, 0));
             CU(h, cudaGetLastError());
             h->launches += 1;
         } else {
-            std::vector<float> tmp((size_t)h->Q * h->geo.N);
-            const size_t nx = h->geo.nx, px = h->geo.px;
-            for (size_t r = 0; r < QN / nx; ++r)
-                for (size_t x = 0; x < nx; ++x) tmp[r * px + x] = (float)f[r * nx + x];
-            CU(h, cudaMemcpyAsync(f32(h, 0), tmp.data(), sizeof(float) * tmp.size(),
-                                  cudaMemcpyHostToDevice, h->stream));
+            std::vector<float> tmp(QN);
+            for (size_t k = 0; k < QN; ++k) tmp[k] = (float)f[k];
+            const bool pad = h->geo.px != h->geo.nx;   // the rows padded on the device, from the dead buffer
+            CU(h, cudaMemcpyAsync(f32(h, pad), tmp.data(), sizeof(float) * QN, cudaMemcpyHostToDevice, h->stream));
+            if (pad) {
+                convert_pops(h, h->geo.nx, h->geo.px, f32(h, 1), f32(h, 0));
+                CU(h, cudaGetLastError());
+                h->launches += 1;
+            }
             CU(h, cudaStreamSynchronize(h->stream));
         }
     } else {

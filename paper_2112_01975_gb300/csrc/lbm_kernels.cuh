@@ -1096,20 +1096,24 @@ __global__ void k_encode_shifted(Geo g, Geo gf, const double *__restrict__ f, co
     }
 }
 
-// Population I/O of FP32 storage: every node's populations from the layout of
-// ga and type A to that of gb and B.
-template <int LAT, typename A, typename B>
-__global__ void k_convert(Geo ga, Geo gb, const A *__restrict__ in, B *__restrict__ out)
+// Population I/O of FP32 storage: `rows` rows of nx populations (of all
+// directions, one after the other) from rows of pa entries of type A to rows of
+// pb of type B. One population a thread and turn: a node a thread, 27 populations
+// each, took 1.4 times as long on 16^3 (32 us against 22).
+template <typename A, typename B>
+__global__ void __launch_bounds__(256)
+k_convert(unsigned rows, unsigned nx, unsigned pa, unsigned pb, const A *__restrict__ in, B *__restrict__ out)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= ga.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned a = entry(ga, x, y, z), b = entry(gb, x, y, z);
-#pragma unroll
-    for (int i = 0; i < Lattice<LAT>::Q; ++i) {
-        const A v = in[(size_t)i * ga.N + a];
-        if constexpr (sizeof(A) == 4) out[(size_t)i * gb.N + b] = widen(v);
-        else                          out[(size_t)i * gb.N + b] = (B)v;
+    const size_t n = (size_t)rows * nx;
+    for (size_t k = blockIdx.x * 256u + threadIdx.x; k < n; k += (size_t)gridDim.x * 256u) {
+        size_t a = k, b = k;
+        if (pa != nx || pb != nx) {
+            const unsigned r = (unsigned)k / nx, x = (unsigned)k - r * nx;   // (at most 4e9 populations)
+            a = (size_t)r * pa + x;
+            b = (size_t)r * pb + x;
+        }
+        if constexpr (sizeof(B) == 8) out[b] = widen(in[a]);
+        else                          out[b] = (B)in[a];
     }
 }
 
