@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <new>
 #include <thread>
 #include <vector>
@@ -1742,6 +1743,7 @@ struct lbm_batch_ctx {
     std::vector<cudaStream_t> prev;   // each member's stream before the batch
     int lattice = 0, storage = LBM_F32;
     cudaStream_t stream = nullptr;
+    void *d_block = nullptr;   // the device memory of what follows
     lbmf::MemberF *d_members[2] = {nullptr, nullptr};   // step parity 0 and 1
     lbmf::WorkItem *d_items = nullptr;   // of the launches below, one after the other
     lbmf::BoxMaps *d_maps = nullptr;     // [member][buffer], TMA-staged launches
@@ -1819,47 +1821,78 @@ void batch_launch(lbm_batch_ctx *b, int parity, cudaStream_t s)
     }
 }
 
+// When the last of the items ends if each free one of `slots` takes the next:
+// runs of (planes, number of items), a block of p planes taking p + 4.5. Slots
+// that are free at the same time are kept as one entry.
+double batch_end(const std::vector<std::pair<int, long long>> &runs, int slots)
+{
+    std::map<double, long long> free{{0.0, slots}};
+    double end = 0.0;
+    for (const auto &run : runs)
+        for (long long left = run.second; left > 0;) {
+            const auto first = free.begin();
+            const double t = first->first + run.first + 4.5;
+            const long long n = std::min(left, first->second);
+            if (n == first->second) free.erase(first);
+            else                    first->second -= n;
+            free[t] += n;
+            end = std::max(end, t);
+            left -= n;
+        }
+    return end;
+}
+
 // Chunks of the members (by number) of one TMA-staged launch, and its items,
 // longest first: members' march axes in equal parts of at most `cap` planes,
-// with the cap that ends first when each free slot (SM, or half of one) takes
-// the next item.
+// with the cap that ends first when each free slot (SM, or half of one where two
+// blocks are resident and the items need them, see best_chunk) takes the next
+// item. Caps that make many times more items than there are slots balance no
+// better and are not looked at.
 std::vector<lbmf::WorkItem> batch_items(const std::vector<lbm_ctx *> &members, const std::vector<int> &which,
-                                        int slots, std::vector<int> &chunks)
+                                        int sms, int resident, std::vector<int> &chunks)
 {
-    std::vector<lbmf::WorkItem> best;
-    double best_cost = 1e300;
-    for (int cap : {1 << 30, 96, 64, 40, 24, 12}) {
-        struct Part { int k, chunk, len, bz; };
-        std::vector<Part> parts;
+    const auto tiles = [&](size_t k) {
+        const GeoF &g = members[which[k]]->geof;
+        return (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+    };
+    double best = 1e300;
+    std::vector<int> seen;
+    for (int cap : {1 << 30, 96, 64, 40, 24, 12, 8, 6, 4}) {
         std::vector<int> ch;
+        std::map<int, long long, std::greater<int>> by_length;
+        long long count = 0;
         for (size_t k = 0; k < which.size(); ++k) {
             const int nz = members[which[k]]->geof.nz, n = (nz + cap - 1) / cap, c = (nz + n - 1) / n;
             ch.push_back(c);
-            for (int bz = 0; bz * c < nz; ++bz) parts.push_back({(int)k, c, std::min(c, nz - bz * c), bz});
+            by_length[c] += tiles(k) * (nz / c);
+            if (nz % c) by_length[nz % c] += tiles(k);
+            count += tiles(k) * ((nz + c - 1) / c);
         }
-        std::stable_sort(parts.begin(), parts.end(), [](const Part &a, const Part &b) { return a.len > b.len; });
-        std::vector<lbmf::WorkItem> items;
-        std::vector<double> busy(slots, 0.0);   // a heap: the slot that is free first on top
-        double cost = 0.0;
-        for (const Part &q : parts) {
-            const GeoF &g = members[which[q.k]]->geof;
-            const int tx = (g.nx + 31) / 32, ty = (g.ny + 7) / 8;
-            for (int by = 0; by < ty; ++by)
-                for (int bx = 0; bx < tx; ++bx) {
-                    items.push_back({q.k, bx, by, q.bz});
-                    std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-                    busy.back() += q.len + 4.5;
-                    cost = std::max(cost, busy.back());
-                    std::push_heap(busy.begin(), busy.end(), std::greater<double>());
-                }
+        if (ch == seen) continue;
+        seen = ch;
+        const bool shared = resident == 2 && count > sms;
+        const int slots = shared ? 2 * sms : sms;
+        const double cost = (shared ? 1.31 : 1.0) * batch_end({by_length.begin(), by_length.end()}, slots);
+        if (cost < best) {
+            best = cost;
+            chunks = ch;
         }
-        if (cost < best_cost) {
-            best_cost = cost;
-            best.swap(items);
-            chunks.swap(ch);
-        }
+        if (count > 10ll * slots) break;
     }
-    return best;
+    struct Part { int k, len, bz; };
+    std::vector<Part> parts;
+    for (size_t k = 0; k < which.size(); ++k) {
+        const int nz = members[which[k]]->geof.nz, c = chunks[k];
+        for (int bz = 0; bz * c < nz; ++bz) parts.push_back({(int)k, std::min(c, nz - bz * c), bz});
+    }
+    std::stable_sort(parts.begin(), parts.end(), [](const Part &a, const Part &b) { return a.len > b.len; });
+    std::vector<lbmf::WorkItem> items;
+    for (const Part &q : parts) {
+        const GeoF &g = members[which[q.k]]->geof;
+        for (int by = 0; by < (g.ny + 7) / 8; ++by)
+            for (int bx = 0; bx < (g.nx + 31) / 32; ++bx) items.push_back({q.k, bx, by, q.bz});
+    }
+    return items;
 }
 
 // `steps` (even) steps from parity 0, captured once.
@@ -1888,9 +1921,7 @@ void batch_free(lbm_batch_ctx *b)
     if (!b) return;
     if (b->graph) cudaGraphExecDestroy(b->graph);
     if (b->graph_long) cudaGraphExecDestroy(b->graph_long);
-    for (auto *m : b->d_members) if (m) cudaFree(m);
-    if (b->d_items) cudaFree(b->d_items);
-    if (b->d_maps) cudaFree(b->d_maps);
+    if (b->d_block) cudaFree(b->d_block);
     for (size_t k = 0; k < b->prev.size(); ++k) b->members[k]->stream = b->prev[k];
     if (b->stream) cudaStreamDestroy(b->stream);
     cudaGetLastError();
@@ -1931,10 +1962,11 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
     std::vector<lbmf::WorkItem> items, plain;
     std::vector<lbmf::BoxMaps> maps;
     std::vector<int> staged;   // members with a TMA-staged form
+    for (int k = 0; k < count; ++k)
+        if (lattice == LBM_D3Q27 && b->members[k]->tmap_ready) staged.push_back(k);
     for (int k = 0; k < count; ++k) {
         lbm_ctx *h = b->members[k];
         const bool tma = lattice == LBM_D3Q27 && h->tmap_ready;
-        if (tma) staged.push_back(k);
         for (int par = 0; par < 2; ++par) maps.push_back(h->tmaps[par]);
         // D3Q27: 32 x 8 columns by z-chunks; D2Q9: 32 x 8 tiles of the (x, 2D y) plane
         const int tx = (h->geof.nx + 31) / 32;
@@ -1942,7 +1974,7 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
         GeoF geof = h->geof;
         if (h->auto_form && lattice == LBM_D3Q27) geof.chunk = kDefaultChunk3;   // the plain form's
         const int tz = lattice == LBM_D2Q9 ? 1 : (geof.nz + geof.chunk - 1) / geof.chunk;
-        for (int par = 0; par < 2; ++par) {
+        for (int par = 0; par < 2 && (int)staged.size() < count; ++par) {   // (staged launches carry theirs)
             lbmf::MemberF m;
             m.g = geof;
             m.p = h->physf;
@@ -1962,30 +1994,60 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
                     for (int bx = 0; bx < tx; ++bx) plain.push_back({k, bx, by, bz});
         h->stream = b->stream;   // members' later work is ordered after the batch
     }
-    const size_t db = sizeof(lbmf::MemberF) * count;
-    if (cudaMalloc(&b->d_members[0], db) != cudaSuccess || cudaMalloc(&b->d_members[1], db) != cudaSuccess ||
-        (!staged.empty() && cudaMalloc(&b->d_maps, sizeof(lbmf::BoxMaps) * maps.size()) != cudaSuccess)) return LBM_ENOMEM;
-    for (size_t first = 0; first < staged.size(); first += lbmf::kBatchMembers) {
-        const std::vector<int> which(staged.begin() + first,
-                                     staged.begin() + std::min(staged.size(), first + lbmf::kBatchMembers));
-        std::vector<int> chunks;
+    // TMA-staged launches, of as many members each as come out even (the launches
+    // of a step run one after the other), then the plain or D2Q9 one
+    const size_t n_staged = (staged.size() + lbmf::kBatchMembers - 1) / lbmf::kBatchMembers;
+    std::vector<std::vector<int>> which(n_staged), chunks(n_staged);
+    b->steps.reserve(n_staged + 1);
+    for (size_t g = 0; g < n_staged; ++g) {
+        which[g].assign(staged.begin() + staged.size() * g / n_staged, staged.begin() + staged.size() * (g + 1) / n_staged);
         const std::vector<lbmf::WorkItem> part =
-            batch_items(b->members, which, storage == LBM_F32 ? sms : 2 * sms, chunks);
-        lbm_batch_ctx::Launch l = {};
+            batch_items(b->members, which[g], sms, storage == LBM_F32 ? 1 : 2, chunks[g]);
+        b->steps.emplace_back();
+        lbm_batch_ctx::Launch &l = b->steps.back();
         l.tma = true;
         l.first = (int)items.size();
         l.n_items = (int)part.size();
-        l.eos = b->members[which[0]]->physf.eos;
+        items.insert(items.end(), part.begin(), part.end());
+    }
+    if (!plain.empty()) {
+        b->steps.emplace_back();
+        lbm_batch_ctx::Launch &l = b->steps.back();
+        l.first = (int)items.size();
+        l.n_items = (int)plain.size();
         l.rest = true;
-        for (size_t k = 0; k < which.size(); ++k) {
-            const lbm_ctx *h = b->members[which[k]];
+        for (const lbm_ctx *h : b->members) l.rest = l.rest && lbmf::at_rest(h->physf);
+        b->grid = std::min(l.n_items, 2 * sms);
+        items.insert(items.end(), plain.begin(), plain.end());
+    }
+    // one block of device memory, filled by one copy: members of both parities,
+    // tensor maps, items
+    const size_t db = sizeof(lbmf::MemberF) * desc[0].size();
+    const size_t mb = staged.empty() ? 0 : sizeof(lbmf::BoxMaps) * maps.size(), ib = sizeof(lbmf::WorkItem) * items.size();
+    const size_t o_maps = 2 * align_up(db), o_items = o_maps + align_up(mb);
+    std::vector<unsigned char> block(o_items + ib);
+    for (int par = 0; par < 2; ++par)
+        if (db) memcpy(&block[par * align_up(db)], desc[par].data(), db);
+    if (mb) memcpy(&block[o_maps], maps.data(), mb);
+    memcpy(&block[o_items], items.data(), ib);
+    if (cudaMalloc(&b->d_block, block.size()) != cudaSuccess) return LBM_ENOMEM;
+    char *const d = static_cast<char *>(b->d_block);
+    for (int par = 0; par < 2; ++par) b->d_members[par] = reinterpret_cast<lbmf::MemberF *>(d + par * align_up(db));
+    b->d_maps = reinterpret_cast<lbmf::BoxMaps *>(d + o_maps);
+    b->d_items = reinterpret_cast<lbmf::WorkItem *>(d + o_items);
+    for (size_t g = 0; g < n_staged; ++g) {
+        lbm_batch_ctx::Launch &l = b->steps[g];
+        l.eos = b->members[which[g][0]]->physf.eos;
+        l.rest = true;
+        for (size_t k = 0; k < which[g].size(); ++k) {
+            const lbm_ctx *h = b->members[which[g][k]];
             l.solid = l.solid || h->any_solid;
             l.rest = l.rest && lbmf::at_rest(h->physf);
             if (h->physf.eos != l.eos) l.eos = -1;
             for (int par = 0; par < 2; ++par) {
                 lbmf::MemberT &m = l.args[par].m[k];
                 m.g = h->geof;
-                m.g.chunk = chunks[k];
+                m.g.chunk = chunks[g][k];
                 m.p = h->physf;
                 m.mask = h->mask;
                 m.src = h->fv[h->cur ^ par];
@@ -1993,29 +2055,13 @@ int batch_build(lbm_batch_ctx *&b, const lbm_handle *members, int count)
                 m.rho_src = h->rs[h->cur ^ par];
                 m.rho_dst = h->rs[h->cur ^ par ^ 1];
                 m.status = h->status;
-                m.maps = b->d_maps + 2 * which[k] + (h->cur ^ par);
+                m.maps = b->d_maps + 2 * which[g][k] + (h->cur ^ par);
             }
         }
-        items.insert(items.end(), part.begin(), part.end());
-        b->steps.push_back(l);
     }
-    if (!plain.empty()) {
-        lbm_batch_ctx::Launch l = {};
-        l.first = (int)items.size();
-        l.n_items = (int)plain.size();
-        l.rest = true;
-        for (const lbm_ctx *h : b->members) l.rest = l.rest && lbmf::at_rest(h->physf);
-        b->grid = std::min(l.n_items, 2 * sms);
-        items.insert(items.end(), plain.begin(), plain.end());
-        b->steps.push_back(l);
-    }
-    const size_t ib = sizeof(lbmf::WorkItem) * items.size();
-    if (cudaMalloc(&b->d_items, ib) != cudaSuccess) return LBM_ENOMEM;
-    if (cudaMemcpy(b->d_members[0], desc[0].data(), db, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_members[1], desc[1].data(), db, cudaMemcpyHostToDevice) != cudaSuccess ||
-        (b->d_maps && cudaMemcpy(b->d_maps, maps.data(), sizeof(lbmf::BoxMaps) * maps.size(),
-                                 cudaMemcpyHostToDevice) != cudaSuccess) ||
-        cudaMemcpy(b->d_items, items.data(), ib, cudaMemcpyHostToDevice) != cudaSuccess) return LBM_ECUDA;
+    // on the batch's stream, which does not wait for the default one
+    if (cudaMemcpyAsync(b->d_block, block.data(), block.size(), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+        cudaStreamSynchronize(b->stream) != cudaSuccess) return LBM_ECUDA;
     return LBM_OK;
 }
 
